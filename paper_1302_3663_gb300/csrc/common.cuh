@@ -52,6 +52,36 @@ struct Ptr3d {
   double* a[3];
 };
 
+// The FP64 operator passes of the mixed-precision solves (op64.cu): the tile
+// of columns of a block, the planes of a chunk and their counts.
+constexpr int kOpThreads = 512;
+struct OpShape {
+  int TX, TY, KC;
+  int nx, ny, nc;
+};
+struct VOpArgs {
+  const float* z[3];     // flexible CG: the preconditioned residual
+  const double* u[3];    // residual: the iterate
+  const double* muc;
+  const double* mue[3];
+  const double* m[3];
+  const double* q[3];    // flexible CG: A times the last direction; residual: f
+  double* w[3];          // A z; the FP64 residual (may be null)
+  float* r32[3];
+  float* e32[3];
+  double* partial;
+  double ir;
+};
+struct POpArgs {
+  const double* p;
+  const double* f;
+  const double* beta[3];
+  float* r32;
+  float* e32;
+  double* partial;
+  double ih2;
+};
+
 // The FP32 viscous point update, Eq. (NSdis1-1) with Eq. (divergenceGrad) /
 // (divergencePartial) on the staggered grid, with every rounding written out
 // (each product, difference and fused multiply-add explicit), so that every
@@ -122,10 +152,9 @@ struct BMember {
   LevelPtrs<double> d[kMaxLevels];
   int L;                    // levels
   double inv_re;
-  double* vdiag[3];         // FP64 viscous diagonal (level 0)
-  double* cg_p[3];          // flexible-CG direction, A times it, preconditioned residual
+  OpShape op;               // the level-0 FP64 passes' blocks
+  double* cg_p[3];          // flexible-CG direction, A times it
   double* cg_q[3];
-  double* cg_z[3];
   Scalars sc;
   int* cycles;              // device-loop iterations of the last solves (viscous, pressure)
   long long* total;         // device-loop iterations so far (viscous, pressure)
@@ -244,23 +273,27 @@ void launch_p_rb_pair(const Geo& g, const LevelPtrs<float>& L, float* out, cudaS
 int pair_fill_kc(const Geo& g, int d, int TY, int waves);
 
 // Mixed precision (mixed.cu).
-int red_blocks_3d(int D, const Geo& g);
+OpShape op_shape(const Geo& g);
+int op_blocks(const OpShape& S);
+int op_blocks(int D, const Geo& g, const OpShape& S);
+void launch_v_op(bool fcg, const Geo& g, const OpShape& S, const VOpArgs& a, cudaStream_t s);
+void launch_p_op(const Geo& g, const OpShape& S, const POpArgs& a, cudaStream_t s);
 // (partial, when not null, receives the blocks' sums of r^2 and then their
-// maxima of |r|: 2 red_blocks_3d entries)
-void launch_p_residual_mixed(int D, const Geo& g, const LevelPtrs<double>& L, float* r32,
-                             float* e32, double* partial, cudaStream_t s);
-void launch_v_residual_mixed(int D, const Geo& g, const LevelPtrs<double>& L, float* const r32[3],
-                             float* const e32[3], double* const diag[3], double inv_re,
+// maxima of |r|: 2 op_blocks entries)
+void launch_p_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                             float* r32, float* e32, double* partial, cudaStream_t s);
+void launch_v_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                             float* const r32[3], float* const e32[3], double inv_re,
                              double* partial, cudaStream_t s, double* const r64[3] = nullptr);
-// Flexible CG around the FP32 V-cycle (mixed.cu): z is the V-cycle's result
-// converted to FP64; w = A z with partial z.q;
+// Flexible CG around the FP32 V-cycle: z is the V-cycle's FP32 result;
+// w = A z in FP64 with partial z.q;
 // p = z + beta p, q = w + beta q with partials p.q, p.r (2 nb entries);
 // x += alpha p, r -= alpha q, r32 = r, e32 = 0 with partial r.r. beta and
 // alpha are read from out[] slots on the device.
-void launch_fcg_apply(int D, const Geo& g, const LevelPtrs<double>& L, double* const z[3],
-                      double* const diag[3], double inv_re, double* const w[3],
-                      double* const q[3], double* partial, cudaStream_t s);
-void launch_fcg_dir(int D, const Geo& g, double* const z[3], double* const w[3], double* const p[3],
+void launch_fcg_apply(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                      float* const z[3], double inv_re, double* const w[3], double* const q[3],
+                      double* partial, cudaStream_t s);
+void launch_fcg_dir(int D, const Geo& g, float* const z[3], double* const w[3], double* const p[3],
                     double* const q[3], double* const r[3], const double* out, int sl_zq,
                     int sl_pq, double* partial, cudaStream_t s);
 // blocks of the flat direction and update passes (their partial sums)
@@ -269,14 +302,9 @@ void launch_fcg_update(int D, const Geo& g, double* const x[3], double* const p[
                        double* const q[3], double* const r[3], float* const r32[3],
                        float* const e32[3], const double* out, int sl_pq, int sl_pr,
                        double* partial, cudaStream_t s);
-// diagonal of the FP64 viscous operator on one level (formed once per step)
-void launch_v_diag(int D, const Geo& g, const LevelPtrs<double>& L, double* const diag[3],
-                   double inv_re, cudaStream_t s);
 void launch_add_correction(int D, const Geo& g, double* const x[3], float* const e[3], int ncomp,
                            cudaStream_t s);
 void launch_f32_to_f64(const float* in, double* out, long long n, cudaStream_t s);
-// three arrays of n elements each in one launch
-void launch_f32_to_f64_3(float* const in[3], double* const out[3], long long n, cudaStream_t s);
 void launch_f64_to_f32(const double* in, float* out, long long n, cudaStream_t s);
 // 1 / diagonal of the viscous operator per face component, from the FP64
 // coefficients of one level, stored in L32.idg (0 on the fixed wall faces)
@@ -353,11 +381,10 @@ void launch_b_tol_check(cudaGraphConditionalHandle h, const BMember* tab, int nm
 // counts in each member's nonconv the solves whose ||r||/||f|| exceeds slack rtol
 void launch_b_res_check(const BMember* tab, int nm, int sf, int sr, double slack,
                         cudaStream_t s);
-// mixed.cu (level 0, FP64)
+// op64.cu, mixed.cu (level 0, FP64)
 void launch_b_v_residual_mixed(const BArgs& A, bool partial, bool r64, int grid, cudaStream_t s);
 void launch_b_p_residual_mixed(const BArgs& A, bool partial, int grid, cudaStream_t s);
 void launch_b_add_correction(const BArgs& A, bool viscous, int grid, cudaStream_t s);
-void launch_b_z_to_f64(const BArgs& A, int grid, cudaStream_t s);
 void launch_b_fcg_apply(const BArgs& A, int grid, cudaStream_t s);
 void launch_b_fcg_dir(const BArgs& A, int sl_zq, int sl_pq, int grid, cudaStream_t s);
 void launch_b_fcg_update(const BArgs& A, int sl_pq, int sl_pr, int grid, cudaStream_t s);

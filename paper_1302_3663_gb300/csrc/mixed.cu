@@ -64,69 +64,57 @@ inline dim3 grd3(long long nx, long long ny, long long nz, dim3 b) {
               (unsigned)((nz + b.z - 1) / b.z));
 }
 
+// The 2D forms of the FP64 passes around the FP32 V-cycles, one thread per
+// point (a 2D grid is small: launches and latency bound it, not arithmetic).
+// The 3D forms are in op64.cu.
+//
 // FP64 pressure residual written as the FP32 right-hand side of the
 // correction equation; the FP32 correction is zeroed; per-block partial sums
 // of r^2 (for the relative-residual test) in partial[0 .. nb) and per-block
 // maxima of |r| (for the divergence the projection will leave, Eq. NSdis2 -
 // NSdis4: max |D.u| = (euler dt / sigma) max |r|) in partial[nb .. 2 nb),
 // nb the launch's blocks; a non-finite residual counts as infinity.
-template <int D>
-__device__ __forceinline__ void p_residual_mixed_body(const Blk& B, Geo g, LevelPtrs<double> L,
-                                                      float* r32, float* e32, double* partial,
-                                                      double ih2) {
+__global__ void __launch_bounds__(256) k_p_residual_mixed2(Geo g, POpArgs A) {
   __shared__ double sh[32];
+  const Blk B = own_blk();
   int i = B.x * blockDim.x + threadIdx.x;
   int j = B.y * blockDim.y + threadIdx.y;
-  int k = B.z * blockDim.z + threadIdx.z;
   double r2 = 0.0, ra = 0.0;
-  if (i < g.n[0] && j < g.n[1] && k < g.n[2]) {
-    int ci[3] = {i, j, k};
-    long long c = gidx(g, i, j, k);
-    double num = 0.0, dg = 0.0;
+  if (i < g.n[0] && j < g.n[1]) {
+    int ci[3] = {i, j, 0};
+    long long c = gidx(g, i, j, 0);
+    const double pc = A.p[c];
+    double div = 0.0;
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      const double* __restrict__ b = L.beta[a];
-      if (ci[a] > 0 || g.per[a]) {
-        double bb = b[c];
-        num += bb * L.p[c + offm(g, a, ci[a])];
-        dg += bb;
-      }
+    for (int a = 0; a < 2; ++a) {
+      const double* __restrict__ b = A.beta[a];
       if (ci[a] < g.n[a] - 1 || g.per[a]) {
         long long cp = c + offp(g, a, ci[a]);
-        double bb = b[cp];
-        num += bb * L.p[cp];
-        dg += bb;
+        div += b[cp] * (A.p[cp] - pc);
       }
+      if (ci[a] > 0 || g.per[a]) div -= b[c] * (pc - A.p[c + offm(g, a, ci[a])]);
     }
-    double r = L.pf[c] - (num - dg * L.p[c]) * ih2;   // ih2 = 1 / h^2 from the host
-    r32[c] = (float)r;
-    e32[c] = 0.0f;
+    double r = A.f[c] - div * A.ih2;
+    A.r32[c] = (float)r;
+    A.e32[c] = 0.0f;
     r2 = r * r;
     ra = fabs(r);
     if (!(ra <= CUDART_INF)) ra = CUDART_INF;
   }
-  if (partial) {
+  if (A.partial) {
     r2 = block_sum(r2, sh);
     ra = block_max(ra, sh);
     if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
       const int nb = B.gx * B.gy * B.gz;
-      partial[B.linear()] = r2;
-      partial[nb + B.linear()] = ra;
+      A.partial[B.linear()] = r2;
+      A.partial[nb + B.linear()] = ra;
     }
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(256) k_p_residual_mixed(Geo g, LevelPtrs<double> L, float* r32,
-                                                          float* e32, double* partial, double ih2) {
-  p_residual_mixed_body<D>(own_blk(), g, L, r32, e32, partial, ih2);
-}
-
 // Diagonal of the FP64 viscous operator of component d at face F:
 // m_d + (inv_re / h^2) * (2 mu_c on both cells + the edge viscosities, an edge
-// beyond a wall counted twice for the mirrored tangential neighbour). The
-// coefficients stay fixed through a time step's solves, so the diagonal is
-// formed once per step instead of in every defect-correction cycle.
+// beyond a wall counted twice for the mirrored tangential neighbour).
 template <int D, int d>
 __device__ __forceinline__ double v_diag64(const Geo& g, const LevelPtrs<double>& L,
                                            const int ci[3], long long F, double ir) {
@@ -144,27 +132,6 @@ __device__ __forceinline__ double v_diag64(const Geo& g, const LevelPtrs<double>
     dgV += (wp ? 2.0 : 1.0) * mep + (wm ? 2.0 : 1.0) * mem;
   }
   return L.m[d][F] + ir * dgV;
-}
-
-template <int D>
-__global__ void __launch_bounds__(256) k_v_diag(Geo g, LevelPtrs<double> L, Ptr3d diag,
-                                                double ir) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int k = blockIdx.z * blockDim.z + threadIdx.z;
-  if (i >= g.n[0] || j >= g.n[1] || k >= g.n[2]) return;
-  int ci[3] = {i, j, k};
-  long long F = gidx(g, i, j, k);
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    double v = 0.0;
-    if (g.per[d] || ci[d] != 0) {
-      if (d == 0) v = v_diag64<D, 0>(g, L, ci, F, ir);
-      else if (d == 1) v = v_diag64<D, 1>(g, L, ci, F, ir);
-      else v = v_diag64<D, (D == 3 ? 2 : 1)>(g, L, ci, F, ir);
-    }
-    diag.a[d][F] = v;
-  }
 }
 
 struct F32x3 {
@@ -196,100 +163,60 @@ __global__ void __launch_bounds__(256) k_v_idg32(Geo g, LevelPtrs<double> L, F32
   }
 }
 
-// FP64 viscous residual of component d at face F with the diagonal read from
-// `diag` (the same arithmetic as the FP64 residual kernel). INTERIOR: no
-// neighbour lies beyond a wall or across a periodic seam, so the offsets are
-// the plain strides and no flag is tested.
-template <int D, int d, bool INTERIOR, typename V>
-__device__ __forceinline__ double v_off64(const Geo& g, const LevelPtrs<double>& L,
-                                          const V* const vec[3], const int ci[3], long long F) {
+// (A u)_d at face F of a 2D grid, in the flux form of op64.cu: differences
+// first, so no diagonal is formed.
+template <int d, typename V>
+__device__ __forceinline__ double v_op2(const Geo& g, const VOpArgs& A, const V* const vec[3],
+                                        const int ci[3], long long F) {
+  constexpr int e = 1 - d;
   const V* __restrict__ ud = vec[d];
-  const long long od_p = INTERIOR ? g.st[d] : offp(g, d, ci[d]);
-  const long long od_m = INTERIOR ? -g.st[d] : offm(g, d, ci[d]);
-  double mcp = L.muc[F], mcm = L.muc[F + od_m];
-  double off = 2.0 * (mcp * (double)ud[F + od_p] + mcm * (double)ud[F + od_m]);
-#pragma unroll
-  for (int e = 0; e < D; ++e) {
-    if (e == d) continue;
-    const V* __restrict__ ue = vec[e];
-    const double* __restrict__ me = L.mue[edge_id(d, e)];
-    bool wp = false, wm = false;
-    if (!INTERIOR) {
-      bool pe = g.per[e] != 0;
-      wp = !pe && ci[e] == g.n[e] - 1;
-      wm = !pe && ci[e] == 0;
-    }
-    const long long oep = INTERIOR ? g.st[e] : offp(g, e, ci[e]);
-    const long long oem = INTERIOR ? -g.st[e] : offm(g, e, ci[e]);
-    long long Ep = F + oep;
-    double mep = me[Ep], mem = me[F];
-    double cp = (double)ue[Ep] - (double)ue[Ep + od_m];
-    double cm = (double)ue[F] - (double)ue[F + od_m];
-    double udp = 0.0, udm = 0.0;
-    if (!wp) udp = (double)ud[Ep];
-    if (!wm) udm = (double)ud[F + oem];
-    off += mep * (udp + cp) + mem * (udm - cm);
-  }
-  return off;
+  const V* __restrict__ ue = vec[e];
+  const double* __restrict__ me = A.mue[0];
+  const long long dp = offp(g, d, ci[d]), dm = offm(g, d, ci[d]);
+  const long long ep = offp(g, e, ci[e]), em = offm(g, e, ci[e]);
+  const bool wp = !g.per[e] && ci[e] == g.n[e] - 1, wm = !g.per[e] && ci[e] == 0;
+  const double u = (double)ud[F];
+  const double tp = A.muc[F] * ((double)ud[F + dp] - u), tm = A.muc[F + dm] * (u - (double)ud[F + dm]);
+  const double up = wp ? -u : (double)ud[F + ep], um = wm ? -u : (double)ud[F + em];
+  const double sp = me[F + ep] * ((up - u) + ((double)ue[F + ep] - (double)ue[F + ep + dm]));
+  const double sm = me[F] * ((u - um) + ((double)ue[F] - (double)ue[F + dm]));
+  return fma(-A.ir, fma(2.0, tp - tm, sp - sm), A.m[d][F] * u);
 }
 
-// The off-diagonal part of the FP64 viscous operator of component d at face
-// F applied to `vec` (FP64 or FP32 components, summed in FP64).
-template <int D, int d, bool INTERIOR>
-__device__ __forceinline__ double v_res64d(const Geo& g, const LevelPtrs<double>& L,
-                                           const double* __restrict__ diag, const int ci[3],
-                                           long long F, double ir) {
-  const double* const vec[3] = {L.u[0], L.u[1], L.u[2]};
-  double off = v_off64<D, d, INTERIOR, double>(g, L, vec, ci, F);
-  return L.uf[d][F] - diag[F] * L.u[d][F] + ir * off;
-}
-
-template <int D, bool INTERIOR>
-__device__ __forceinline__ double v_res_any(const Geo& g, const LevelPtrs<double>& L,
-                                            const Ptr3d& diag, int d, const int ci[3],
-                                            long long F, double ir) {
-  if (d == 0) return v_res64d<D, 0, INTERIOR>(g, L, diag.a[0], ci, F, ir);
-  if (d == 1) return v_res64d<D, 1, INTERIOR>(g, L, diag.a[1], ci, F, ir);
-  return v_res64d<D, (D == 3 ? 2 : 1), INTERIOR>(g, L, diag.a[D == 3 ? 2 : 1], ci, F, ir);
-}
-
-template <int D>
-__device__ __forceinline__ void v_residual_mixed_body(const Blk& B, Geo g, LevelPtrs<double> L,
-                                                      F32x3 r32, F32x3 e32, Ptr3d diag, double ir,
-                                                      double* partial, Ptr3d r64) {
+// FCG: w = A z on every unknown face (0 on the fixed wall faces) with partial
+// sums of z.q; else r = f - A u to FP32 (and FP64 when given), the FP32
+// correction zeroed, with partial sums of r^2.
+template <bool FCG>
+__global__ void __launch_bounds__(256) k_v_op2(Geo g, VOpArgs A) {
   __shared__ double sh[32];
+  const Blk B = own_blk();
   int i = B.x * blockDim.x + threadIdx.x;
   int j = B.y * blockDim.y + threadIdx.y;
-  int k = B.z * blockDim.z + threadIdx.z;
-  double r2 = 0.0;
-  if (i < g.n[0] && j < g.n[1] && k < g.n[2]) {
-    int ci[3] = {i, j, k};
-    long long F = gidx(g, i, j, k);
-    bool interior = true;
+  double acc = 0.0;
+  if (i < g.n[0] && j < g.n[1]) {
+    int ci[3] = {i, j, 0};
+    long long F = gidx(g, i, j, 0);
 #pragma unroll
-    for (int a = 0; a < D; ++a) interior = interior && ci[a] > 0 && ci[a] < g.n[a] - 1;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      double r = 0.0;
-      if (interior) r = v_res_any<D, true>(g, L, diag, d, ci, F, ir);
-      else if (g.per[d] || ci[d] != 0) r = v_res_any<D, false>(g, L, diag, d, ci, F, ir);
-      r32.a[d][F] = (float)r;
-      e32.a[d][F] = 0.0f;
-      if (r64.a[0]) r64.a[d][F] = r;
-      r2 += r * r;
+    for (int d = 0; d < 2; ++d) {
+      const bool wall = !g.per[d] && ci[d] == 0;
+      double v = 0.0;
+      if constexpr (FCG) {
+        if (!wall) v = d == 0 ? v_op2<0>(g, A, A.z, ci, F) : v_op2<1>(g, A, A.z, ci, F);
+        A.w[d][F] = v;
+        acc += (double)A.z[d][F] * A.q[d][F];
+      } else {
+        if (!wall) v = A.q[d][F] - (d == 0 ? v_op2<0>(g, A, A.u, ci, F) : v_op2<1>(g, A, A.u, ci, F));
+        A.r32[d][F] = (float)v;
+        A.e32[d][F] = 0.0f;
+        if (A.w[d]) A.w[d][F] = v;
+        acc += v * v;
+      }
     }
   }
-  if (partial) {
-    r2 = block_sum(r2, sh);
-    if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) partial[B.linear()] = r2;
+  if (A.partial) {
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) A.partial[B.linear()] = acc;
   }
-}
-
-template <int D>
-__global__ void __launch_bounds__(256, 3) k_v_residual_mixed(Geo g, LevelPtrs<double> L, F32x3 r32,
-                                                          F32x3 e32, Ptr3d diag, double ir,
-                                                          double* partial, Ptr3d r64) {
-  v_residual_mixed_body<D>(own_blk(), g, L, r32, e32, diag, ir, partial, r64);
 }
 
 // x += e over the unknowns of ncomp face components (ncomp = 0: cells)
@@ -326,13 +253,6 @@ __global__ void __launch_bounds__(256) k_convert(const Tin* __restrict__ in, Tou
 
 }  // namespace
 
-// three FP32 arrays to FP64 on every stored element
-__global__ void __launch_bounds__(256) k_convert3(F32x3 in, Ptr3d out, long long n) {
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-       q += (long long)gridDim.x * blockDim.x)
-    for (int d = 0; d < 3; ++d) out.a[d][q] = (double)in.a[d][q];
-}
-
 namespace {
 
 struct ConvList {
@@ -349,37 +269,54 @@ __global__ void __launch_bounds__(256) k_convert_list(ConvList L, long long elem
 
 }  // namespace
 
-int red_blocks_3d(int D, const Geo& g) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
-  return (int)(gr.x * gr.y * gr.z);
+// blocks of the FP64 passes (their partial results)
+int op_blocks(int D, const Geo& g, const OpShape& S) {
+  if (D == 3) return op_blocks(S);
+  dim3 gr = grd3(g.n[0], g.n[1], 1, blk3(2));
+  return (int)(gr.x * gr.y);
 }
 
-void launch_p_residual_mixed(int D, const Geo& g, const LevelPtrs<double>& L, float* r32,
-                             float* e32, double* partial, cudaStream_t s) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
-  const double ih2 = 1.0 / (g.h * g.h);
-  if (D == 3) k_p_residual_mixed<3><<<gr, b, 0, s>>>(g, L, r32, e32, partial, ih2);
-  else k_p_residual_mixed<2><<<gr, b, 0, s>>>(g, L, r32, e32, partial, ih2);
+void launch_p_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                             float* r32, float* e32, double* partial, cudaStream_t s) {
+  POpArgs a;
+  a.p = L.p;
+  a.f = L.pf;
+  for (int d = 0; d < 3; ++d) a.beta[d] = L.beta[d];
+  a.r32 = r32;
+  a.e32 = e32;
+  a.partial = partial;
+  a.ih2 = 1.0 / (g.h * g.h);
+  if (D == 3) launch_p_op(g, S, a, s);
+  else k_p_residual_mixed2<<<grd3(g.n[0], g.n[1], 1, blk3(2)), blk3(2), 0, s>>>(g, a);
 }
 
-void launch_v_residual_mixed(int D, const Geo& g, const LevelPtrs<double>& L, float* const r32[3],
-                             float* const e32[3], double* const diag[3], double inv_re,
-                             double* partial, cudaStream_t s, double* const r64[3]) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
-  F32x3 r, e;
-  Ptr3d dg, rr;
+namespace {
+VOpArgs v_op_args(const Geo& g, const LevelPtrs<double>& L, double inv_re, double* partial) {
+  VOpArgs a = {};
+  a.muc = L.muc;
   for (int d = 0; d < 3; ++d) {
-    r.a[d] = r32[d];
-    e.a[d] = e32[d];
-    dg.a[d] = diag[d];
-    rr.a[d] = r64 ? r64[d] : nullptr;
+    a.mue[d] = L.mue[d];
+    a.m[d] = L.m[d];
   }
-  double ir = inv_re / (g.h * g.h);
-  if (D == 3) k_v_residual_mixed<3><<<gr, b, 0, s>>>(g, L, r, e, dg, ir, partial, rr);
-  else k_v_residual_mixed<2><<<gr, b, 0, s>>>(g, L, r, e, dg, ir, partial, rr);
+  a.ir = inv_re / (g.h * g.h);
+  a.partial = partial;
+  return a;
+}
+}  // namespace
+
+void launch_v_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                             float* const r32[3], float* const e32[3], double inv_re,
+                             double* partial, cudaStream_t s, double* const r64[3]) {
+  VOpArgs a = v_op_args(g, L, inv_re, partial);
+  for (int d = 0; d < 3; ++d) {
+    a.u[d] = L.u[d];
+    a.q[d] = L.uf[d];
+    a.w[d] = r64 ? r64[d] : nullptr;
+    a.r32[d] = r32[d];
+    a.e32[d] = e32[d];
+  }
+  if (D == 3) launch_v_op(false, g, S, a, s);
+  else k_v_op2<false><<<grd3(g.n[0], g.n[1], 1, blk3(2)), blk3(2), 0, s>>>(g, a);
 }
 
 // ------------------------------------------------------------ flexible CG
@@ -391,72 +328,6 @@ void launch_v_residual_mixed(int D, const Geo& g, const LevelPtrs<double>& L, fl
 //   p = z + beta p,  q = w + beta q,  alpha = (p.r) / (p.q),
 //   x += alpha p,  r -= alpha q.
 // Scalars travel between the kernels in device memory (slots of `out`).
-// (z arrives in FP64: converting each FP32 neighbour at every use would put
-// about fifteen conversions per face on GB300's small FP64 pipe)
-template <int D, int d, bool INTERIOR>
-__device__ __forceinline__ double v_apply_z(const Geo& g, const LevelPtrs<double>& L,
-                                            const Ptr3d& z, const double* __restrict__ diag,
-                                            const int ci[3], long long F, double ir) {
-  const double* const vec[3] = {z.a[0], z.a[1], z.a[2]};
-  double off = v_off64<D, d, INTERIOR, double>(g, L, vec, ci, F);
-  return diag[F] * z.a[d][F] - ir * off;
-}
-
-template <int D, bool INTERIOR>
-__device__ __forceinline__ double v_apply_any(const Geo& g, const LevelPtrs<double>& L,
-                                              const Ptr3d& z, const Ptr3d& diag, int d,
-                                              const int ci[3], long long F, double ir) {
-  if (d == 0) return v_apply_z<D, 0, INTERIOR>(g, L, z, diag.a[0], ci, F, ir);
-  if (d == 1) return v_apply_z<D, 1, INTERIOR>(g, L, z, diag.a[1], ci, F, ir);
-  return v_apply_z<D, (D == 3 ? 2 : 1), INTERIOR>(g, L, z, diag.a[D == 3 ? 2 : 1], ci, F, ir);
-}
-
-__device__ __forceinline__ bool block_leader() {
-  return threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0;
-}
-
-// w = A z on every unknown face (0 on the fixed wall faces); partial sums of z.q.
-// GB300's FP64 rate bounds this kernel and the FP64 residual: their launch
-// bounds keep 4 and 3 blocks resident per SM (64 and 80 registers) so that
-// enough warps hide the FP64 pipe's and the loads' latency. The batched forms
-// hold a member's pointers in registers on top and keep 3 at 80 registers:
-// their spills (about 110 bytes a thread) cost less than the third block
-// gains (1 % of a 64-duct batch step).
-template <int D>
-__device__ __forceinline__ void fcg_apply_body(const Blk& B, Geo g, LevelPtrs<double> L, Ptr3d z,
-                                               Ptr3d diag, double ir, Ptr3d w, Ptr3d q,
-                                               double* partial) {
-  __shared__ double sh[32];
-  int i = B.x * blockDim.x + threadIdx.x;
-  int j = B.y * blockDim.y + threadIdx.y;
-  int k = B.z * blockDim.z + threadIdx.z;
-  double zq = 0.0;
-  if (i < g.n[0] && j < g.n[1] && k < g.n[2]) {
-    int ci[3] = {i, j, k};
-    long long F = gidx(g, i, j, k);
-    bool interior = true;
-#pragma unroll
-    for (int a = 0; a < D; ++a) interior = interior && ci[a] > 0 && ci[a] < g.n[a] - 1;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      double v = 0.0;
-      if (interior) v = v_apply_any<D, true>(g, L, z, diag, d, ci, F, ir);
-      else if (g.per[d] || ci[d] != 0) v = v_apply_any<D, false>(g, L, z, diag, d, ci, F, ir);
-      w.a[d][F] = v;
-      zq += z.a[d][F] * q.a[d][F];
-    }
-  }
-  zq = block_sum(zq, sh);
-  if (block_leader()) partial[B.linear()] = zq;
-}
-
-template <int D>
-__global__ void __launch_bounds__(256, 4) k_fcg_apply(Geo g, LevelPtrs<double> L, Ptr3d z,
-                                                   Ptr3d diag, double ir, Ptr3d w, Ptr3d q,
-                                                   double* partial) {
-  fcg_apply_body<D>(own_blk(), g, L, z, diag, ir, w, q, partial);
-}
-
 // The direction and update passes touch every stored element of the level
 // arrays (pads and fixed wall faces hold 0 in every vector, so they add
 // nothing): flat grid-stride loops over pairs of doubles.
@@ -464,7 +335,7 @@ constexpr int kFlatBlocks = 1216;   // 8 blocks of 256 threads per SM on 152 SMs
 
 // p = z + beta p, q = w + beta q; partial sums of p.q (first nb) and p.r (next nb)
 template <int D>
-__device__ __forceinline__ void fcg_dir_body(const Blk& B, long long npair, Ptr3d z, Ptr3d w,
+__device__ __forceinline__ void fcg_dir_body(const Blk& B, long long npair, F32x3 z, Ptr3d w,
                                              Ptr3d p, Ptr3d q, Ptr3d r,
                                              const double* __restrict__ out, int sl_zq, int sl_pq,
                                              double* partial) {
@@ -476,14 +347,16 @@ __device__ __forceinline__ void fcg_dir_body(const Blk& B, long long npair, Ptr3
   double pq = 0.0, pr = 0.0;
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    const double2* __restrict__ zz = reinterpret_cast<const double2*>(z.a[d]);
+    const float2* __restrict__ zz = reinterpret_cast<const float2*>(z.a[d]);
     const double2* __restrict__ ww = reinterpret_cast<const double2*>(w.a[d]);
     const double2* __restrict__ rr = reinterpret_cast<const double2*>(r.a[d]);
     double2* pp = reinterpret_cast<double2*>(p.a[d]);
     double2* qq = reinterpret_cast<double2*>(q.a[d]);
     for (long long k = B.x * (long long)blockDim.x + threadIdx.x; k < npair;
          k += (long long)B.gx * blockDim.x) {
-      double2 zv = zz[k], wv = ww[k], rv = rr[k], pv = zv, qv = wv;
+      const float2 zf = zz[k];
+      const double2 wv = ww[k], rv = rr[k];
+      double2 pv = make_double2((double)zf.x, (double)zf.y), qv = wv;
       if (!first) {
         const double2 po = pp[k], qo = qq[k];
         pv.x += beta * po.x;
@@ -506,7 +379,7 @@ __device__ __forceinline__ void fcg_dir_body(const Blk& B, long long npair, Ptr3
 }
 
 template <int D>
-__global__ void __launch_bounds__(256) k_fcg_dir(long long npair, Ptr3d z, Ptr3d w, Ptr3d p,
+__global__ void __launch_bounds__(256) k_fcg_dir(long long npair, F32x3 z, Ptr3d w, Ptr3d p,
                                                  Ptr3d q, Ptr3d r, const double* __restrict__ out,
                                                  int sl_zq, int sl_pq, double* partial) {
   fcg_dir_body<D>(own_blk(), npair, z, w, p, q, r, out, sl_zq, sl_pq, partial);
@@ -570,14 +443,17 @@ F32x3 f3(float* const a[3]) {
 }
 }  // namespace
 
-void launch_fcg_apply(int D, const Geo& g, const LevelPtrs<double>& L, double* const z[3],
-                      double* const diag[3], double inv_re, double* const w[3],
-                      double* const q[3], double* partial, cudaStream_t s) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
-  double ir = inv_re / (g.h * g.h);
-  if (D == 3) k_fcg_apply<3><<<gr, b, 0, s>>>(g, L, p3(z), p3(diag), ir, p3(w), p3(q), partial);
-  else k_fcg_apply<2><<<gr, b, 0, s>>>(g, L, p3(z), p3(diag), ir, p3(w), p3(q), partial);
+void launch_fcg_apply(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
+                      float* const z[3], double inv_re, double* const w[3], double* const q[3],
+                      double* partial, cudaStream_t s) {
+  VOpArgs a = v_op_args(g, L, inv_re, partial);
+  for (int d = 0; d < 3; ++d) {
+    a.z[d] = z[d];
+    a.q[d] = q[d];
+    a.w[d] = w[d];
+  }
+  if (D == 3) launch_v_op(true, g, S, a, s);
+  else k_v_op2<true><<<grd3(g.n[0], g.n[1], 1, blk3(2)), blk3(2), 0, s>>>(g, a);
 }
 
 // flat loops run over pairs: the level arrays hold an even number of
@@ -590,15 +466,15 @@ int fcg_flat_blocks(const Geo& g) {
   return (int)(nb < kFlatBlocks ? (nb < 1 ? 1 : nb) : kFlatBlocks);
 }
 
-void launch_fcg_dir(int D, const Geo& g, double* const z[3], double* const w[3], double* const p[3],
+void launch_fcg_dir(int D, const Geo& g, float* const z[3], double* const w[3], double* const p[3],
                     double* const q[3], double* const r[3], const double* out, int sl_zq,
                     int sl_pq, double* partial, cudaStream_t s) {
   const long long npair = flat_elems(g) / 2;
   const int nb = fcg_flat_blocks(g);
   if (D == 3)
-    k_fcg_dir<3><<<nb, 256, 0, s>>>(npair, p3(z), p3(w), p3(p), p3(q), p3(r), out, sl_zq, sl_pq, partial);
+    k_fcg_dir<3><<<nb, 256, 0, s>>>(npair, f3(z), p3(w), p3(p), p3(q), p3(r), out, sl_zq, sl_pq, partial);
   else
-    k_fcg_dir<2><<<nb, 256, 0, s>>>(npair, p3(z), p3(w), p3(p), p3(q), p3(r), out, sl_zq, sl_pq, partial);
+    k_fcg_dir<2><<<nb, 256, 0, s>>>(npair, f3(z), p3(w), p3(p), p3(q), p3(r), out, sl_zq, sl_pq, partial);
 }
 
 void launch_fcg_update(int D, const Geo& g, double* const x[3], double* const p[3],
@@ -613,17 +489,6 @@ void launch_fcg_update(int D, const Geo& g, double* const x[3], double* const p[
   else
     k_fcg_update<2><<<nb, 256, 0, s>>>(npair, p3(x), p3(p), p3(q), p3(r), f3(r32), f3(e32), out,
                                        sl_pq, sl_pr, partial);
-}
-
-void launch_v_diag(int D, const Geo& g, const LevelPtrs<double>& L, double* const diag[3],
-                   double inv_re, cudaStream_t s) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
-  Ptr3d dg;
-  for (int d = 0; d < 3; ++d) dg.a[d] = diag[d];
-  double ir = inv_re / (g.h * g.h);
-  if (D == 3) k_v_diag<3><<<gr, b, 0, s>>>(g, L, dg, ir);
-  else k_v_diag<2><<<gr, b, 0, s>>>(g, L, dg, ir);
 }
 
 void launch_add_correction(int D, const Geo& g, double* const x[3], float* const e[3], int ncomp,
@@ -642,16 +507,6 @@ void launch_add_correction(int D, const Geo& g, double* const x[3], float* const
 
 void launch_f32_to_f64(const float* in, double* out, long long n, cudaStream_t s) {
   k_convert<float, double><<<(unsigned)flat_convert_blocks(n), kBlock1D, 0, s>>>(in, out, n);
-}
-
-void launch_f32_to_f64_3(float* const in[3], double* const out[3], long long n, cudaStream_t s) {
-  F32x3 i;
-  Ptr3d o;
-  for (int d = 0; d < 3; ++d) {
-    i.a[d] = in[d];
-    o.a[d] = out[d];
-  }
-  k_convert3<<<(unsigned)flat_convert_blocks(n), kBlock1D, 0, s>>>(i, o, n);
 }
 
 void launch_f64_to_f32(const double* in, float* out, long long n, cudaStream_t s) {
@@ -694,29 +549,6 @@ void launch_coef_to_f32(int D, const Geo& g, const LevelPtrs<double>& L64,
 // The level-0 FP64 steps of the batched solves: the bodies above over a
 // persistent batch's work list, each with a member's own arrays, scalars and
 // the block decomposition of its single-instance launch.
-__global__ void __launch_bounds__(256, 3) kb_v_residual_mixed(BArgs A, int with_partial, int with_r64) {
-  for_items(A, [&](const BMember& M, const Blk& B) {
-    const Geo g = M.g[0];
-    F32x3 r, e;
-    Ptr3d dg, rr;
-    for (int d = 0; d < 3; ++d) {
-      r.a[d] = M.f[0].uf[d];
-      e.a[d] = M.f[0].u[d];
-      dg.a[d] = M.vdiag[d];
-      rr.a[d] = with_r64 ? M.d[0].ur[d] : nullptr;
-    }
-    v_residual_mixed_body<3>(B, g, M.d[0], r, e, dg, M.ir[0],
-                             with_partial ? M.sc.partial : nullptr, rr);
-  });
-}
-
-__global__ void __launch_bounds__(256) kb_p_residual_mixed(BArgs A, int with_partial) {
-  for_items(A, [&](const BMember& M, const Blk& B) {
-    p_residual_mixed_body<3>(B, M.g[0], M.d[0], M.f[0].pf, M.f[0].p,
-                             with_partial ? M.sc.partial : nullptr, M.ih2[0]);
-  });
-}
-
 __global__ void __launch_bounds__(256) kb_add_correction(BArgs A, int viscous) {
   for_items(A, [&](const BMember& M, const Blk& B) {
     Ptr3d x;
@@ -729,39 +561,12 @@ __global__ void __launch_bounds__(256) kb_add_correction(BArgs A, int viscous) {
   });
 }
 
-// z = the V-cycle's FP32 result in FP64, on every stored element
-__global__ void __launch_bounds__(256) kb_z_to_f64(BArgs A) {
-  for_items(A, [&](const BMember& M, const Blk& B) {
-    const long long n = flat_elems(M.g[0]);
-    for (int d = 0; d < 3; ++d) {
-      const float* __restrict__ in = M.f[0].u[d];
-      double* __restrict__ out = M.cg_z[d];
-      for (long long q = B.x * (long long)blockDim.x + threadIdx.x; q < n;
-           q += (long long)B.gx * blockDim.x)
-        out[q] = (double)in[q];
-    }
-  });
-}
-
-__global__ void __launch_bounds__(256, 3) kb_fcg_apply(BArgs A) {
-  for_items(A, [&](const BMember& M, const Blk& B) {
-    const Geo g = M.g[0];
-    Ptr3d z, dg, w, q;
-    for (int d = 0; d < 3; ++d) {
-      z.a[d] = M.cg_z[d];
-      dg.a[d] = M.vdiag[d];
-      w.a[d] = M.d[0].u2[d];
-      q.a[d] = M.cg_q[d];
-    }
-    fcg_apply_body<3>(B, g, M.d[0], z, dg, M.ir[0], w, q, M.sc.partial);
-  });
-}
-
 __global__ void __launch_bounds__(256) kb_fcg_dir(BArgs A, int sl_zq, int sl_pq) {
   for_items(A, [&](const BMember& M, const Blk& B) {
-    Ptr3d z, w, p, q, r;
+    F32x3 z;
+    Ptr3d w, p, q, r;
     for (int d = 0; d < 3; ++d) {
-      z.a[d] = M.cg_z[d];
+      z.a[d] = M.f[0].u[d];
       w.a[d] = M.d[0].u2[d];
       p.a[d] = M.cg_p[d];
       q.a[d] = M.cg_q[d];
@@ -795,20 +600,8 @@ int flat_convert_blocks(long long n) {
   return (int)(nb < 1 ? 1 : nb);
 }
 
-void launch_b_v_residual_mixed(const BArgs& A, bool partial, bool r64, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_v_residual_mixed<<<grid, blk3(3), 0, s>>>(A, partial ? 1 : 0, r64 ? 1 : 0);
-}
-void launch_b_p_residual_mixed(const BArgs& A, bool partial, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_p_residual_mixed<<<grid, blk3(3), 0, s>>>(A, partial ? 1 : 0);
-}
 void launch_b_add_correction(const BArgs& A, bool viscous, int grid, cudaStream_t s) {
   if (A.n > 0) kb_add_correction<<<grid, blk3(3), 0, s>>>(A, viscous ? 1 : 0);
-}
-void launch_b_z_to_f64(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_z_to_f64<<<grid, kBlock1D, 0, s>>>(A);
-}
-void launch_b_fcg_apply(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_fcg_apply<<<grid, blk3(3), 0, s>>>(A);
 }
 void launch_b_fcg_dir(const BArgs& A, int sl_zq, int sl_pq, int grid, cudaStream_t s) {
   if (A.n > 0) kb_fcg_dir<<<grid, 256, 0, s>>>(A, sl_zq, sl_pq);

@@ -92,10 +92,10 @@ size_t grid_pool_bytes(const bfibm_params& P, int* nlev = nullptr) {
   size_t bytes = 0;
   for (int l = 0; l < L; ++l) {
     size_t arr = (size_t)round_up(level_elems(g[l]) * 8, 256);
-    // level 0: velocity, density, force; mixed precision adds the FP64
-    // viscous diagonal and the flexible-CG vectors p, q and z
+    // level 0: velocity, density, force; mixed precision adds the
+    // flexible-CG vectors p and q
     int na = arrays_per_level(P.dim) + (l == 0 ? 3 * P.dim : 0) +
-             (l == 0 && P.precision == 1 ? 4 * P.dim : 0);
+             (l == 0 && P.precision == 1 ? 2 * P.dim : 0);
     bytes += arr * na;
     if (P.precision == 1)   // the level's arrays and the inverse viscous diagonals
       bytes += (size_t)round_up(level_elems(g[l]) * 4, 256) * (arrays_per_level(P.dim) + P.dim);
@@ -168,10 +168,9 @@ struct bfibm_ctx {
   int D = 0, L = 0;
   Level lev[kMaxLevels];
   double* uvel[3] = {nullptr, nullptr, nullptr};
-  double* vdiag[3] = {nullptr, nullptr, nullptr};   // FP64 viscous diagonal (mixed precision)
+  OpShape op{};                                     // blocks of the level-0 FP64 passes (mixed)
   double* cg_p[3] = {nullptr, nullptr, nullptr};    // flexible-CG direction and A times it
   double* cg_q[3] = {nullptr, nullptr, nullptr};
-  double* cg_z[3] = {nullptr, nullptr, nullptr};    // the preconditioned residual in FP64
   double* rho[3] = {nullptr, nullptr, nullptr};
   double* frc[3] = {nullptr, nullptr, nullptr};
   double* G_dev = nullptr;
@@ -416,11 +415,10 @@ void fill_member(const bfibm_ctx* c, BMember& B) {
   }
   B.L = c->L;
   B.inv_re = c->P.inv_re;
+  B.op = c->op;
   for (int d = 0; d < 3; ++d) {
-    B.vdiag[d] = c->vdiag[d];
     B.cg_p[d] = c->cg_p[d];
     B.cg_q[d] = c->cg_q[d];
-    B.cg_z[d] = c->cg_z[d];
   }
   B.sc = c->sc;
   B.cycles = c->dev_cycles;
@@ -734,7 +732,7 @@ bfibm_status solve_p_mixed(bfibm_ctx* c, int ncycles, int* used) {
   double* one[3] = {L0.d.pf, nullptr, nullptr};
   bool tol = ncycles <= 0;
   const int inner = c->inner;
-  int nb = red_blocks_3d(c->D, L0.g);
+  int nb = op_blocks(c->D, L0.g, c->op);
   if (tol || c->collect_stats) launch_norm2(c->D, L0.g, one, 0, c->sc, SL_PF, s);
   int vmax = tol ? c->P.max_cycles : ncycles;
   int maxc = dc_iterations(vmax, inner);
@@ -743,7 +741,7 @@ bfibm_status solve_p_mixed(bfibm_ctx* c, int ncycles, int* used) {
   float* es[3] = {L0.f.p, nullptr, nullptr};
   if (tol && c->capturing) {
     cudaMemsetAsync(c->dev_cycles + 1, 0, sizeof(int), s);
-    launch_p_residual_mixed(c->D, L0.g, L0.d, L0.f.pf, L0.f.p, nullptr, s);
+    launch_p_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.pf, L0.f.p, nullptr, s);
     c->loop_inner[1] = inner;
     bfibm_status cs = capture_while(c, 1, [&](cudaGraphConditionalHandle h) {
       cudaStream_t b = c->stream;
@@ -752,7 +750,7 @@ bfibm_status solve_p_mixed(bfibm_ctx* c, int ncycles, int* used) {
       es[0] = L0.f.p;
       launch_add_correction(c->D, L0.g, xs, es, 0, b);
       launch_sub_mean(c->D, L0.g, L0.d.p, c->sc, b);
-      launch_p_residual_mixed(c->D, L0.g, L0.d, L0.f.pf, L0.f.p, c->sc.partial, b);
+      launch_p_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.pf, L0.f.p, c->sc.partial, b);
       launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_PR, 1.0, b);
       if (c->P.div_tol > 0.0) launch_finalize_max(c->sc.partial + nb, nb, c->sc.out, SL_PRMAX, b);
       launch_tol_check(h, c->sc.out, SL_PF, SL_PR, c->P.rtol, maxc, c->dev_cycles + 1,
@@ -764,7 +762,7 @@ bfibm_status solve_p_mixed(bfibm_ctx* c, int ncycles, int* used) {
   }
   int k = 0, vdone = 0;
   for (k = 1; k <= maxc; ++k) {
-    launch_p_residual_mixed(c->D, L0.g, L0.d, L0.f.pf, L0.f.p, tol ? c->sc.partial : nullptr, s);
+    launch_p_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.pf, L0.f.p, tol ? c->sc.partial : nullptr, s);
     if (tol) {
       launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_PR, 1.0, s);
       launch_finalize_max(c->sc.partial + nb, nb, c->sc.out, SL_PRMAX, s);
@@ -784,7 +782,7 @@ bfibm_status solve_p_mixed(bfibm_ctx* c, int ncycles, int* used) {
     launch_sub_mean(c->D, L0.g, L0.d.p, c->sc, s);
   }
   if (c->collect_stats || tol) {
-    launch_p_residual_mixed(c->D, L0.g, L0.d, L0.f.pf, L0.f.p, c->sc.partial, s);
+    launch_p_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.pf, L0.f.p, c->sc.partial, s);
     launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_PR, 1.0, s);
   }
   *used = vdone;
@@ -796,20 +794,20 @@ bfibm_status solve_v_mixed(bfibm_ctx* c, int ncycles, int* used) {
   cudaStream_t s = c->stream;
   bool tol = ncycles <= 0;
   const int inner = c->inner;
-  int nb = red_blocks_3d(c->D, L0.g);
+  int nb = op_blocks(c->D, L0.g, c->op);
   if (tol || c->collect_stats) launch_norm2(c->D, L0.g, L0.d.uf, c->D, c->sc, SL_VF, s);
   int vmax = tol ? c->P.max_cycles : ncycles;
   int maxc = dc_iterations(vmax, inner);
   bfibm_status st = tol ? BFIBM_ENOCONV : BFIBM_OK;
   if (tol && c->capturing) {
     cudaMemsetAsync(c->dev_cycles, 0, sizeof(int), s);
-    launch_v_residual_mixed(c->D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re, nullptr, s);
+    launch_v_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re, nullptr, s);
     c->loop_inner[0] = inner;
     bfibm_status cs = capture_while(c, 0, [&](cudaGraphConditionalHandle h) {
       cudaStream_t b = c->stream;
       for (int q = 0; q < inner; ++q) vcycle_v32(c, 0);
       launch_add_correction(c->D, L0.g, L0.d.u, L0.f.u, c->D, b);
-      launch_v_residual_mixed(c->D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re, c->sc.partial, b);
+      launch_v_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re, c->sc.partial, b);
       launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, b);
       launch_tol_check(h, c->sc.out, SL_VF, SL_VR, c->P.rtol, maxc, c->dev_cycles,
                        c->loop_total, c->counters + 4, b);
@@ -819,7 +817,7 @@ bfibm_status solve_v_mixed(bfibm_ctx* c, int ncycles, int* used) {
   }
   int k = 0, vdone = 0;
   for (k = 1; k <= maxc; ++k) {
-    launch_v_residual_mixed(c->D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re,
+    launch_v_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re,
                             tol ? c->sc.partial : nullptr, s);
     if (tol) {
       launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, s);
@@ -837,7 +835,7 @@ bfibm_status solve_v_mixed(bfibm_ctx* c, int ncycles, int* used) {
     launch_add_correction(c->D, L0.g, L0.d.u, L0.f.u, c->D, s);
   }
   if (c->collect_stats || tol) {
-    launch_v_residual_mixed(c->D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re, c->sc.partial, s);
+    launch_v_residual_mixed(c->D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re, c->sc.partial, s);
     launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, s);
   }
   *used = vdone;
@@ -855,7 +853,7 @@ bfibm_status solve_v_fcg(bfibm_ctx* c, int ncycles, int* used) {
   const int D = c->D;
   const bool tol = ncycles <= 0;
   const int inner = c->inner;
-  const int nb = red_blocks_3d(D, L0.g);
+  const int nb = op_blocks(D, L0.g, c->op);
   const int nbf = fcg_flat_blocks(L0.g);
   double* w[3] = {L0.d.u2[0], L0.d.u2[1], L0.d.u2[2]};
   double* r[3] = {L0.d.ur[0], L0.d.ur[1], L0.d.ur[2]};
@@ -863,18 +861,15 @@ bfibm_status solve_v_fcg(bfibm_ctx* c, int ncycles, int* used) {
   const int maxc = dc_iterations(tol ? c->P.max_cycles : ncycles, inner);
   // r = f - A x in FP64 (and as the FP32 right-hand side), the first
   // direction flagged by p.q = 0
-  launch_v_residual_mixed(D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re, c->sc.partial,
+  launch_v_residual_mixed(D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re, c->sc.partial,
                           s, r);
   launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, s);
   CK(cudaMemsetAsync(c->sc.out + SL_PQ, 0, sizeof(double), s));
   auto iteration = [&](cudaStream_t b, int nv) {
     for (int q = 0; q < nv; ++q) vcycle_v32(c, 0);
-    if (D == 3) launch_f32_to_f64_3(L0.f.u, c->cg_z, level_elems(L0.g), b);
-    else
-      for (int d = 0; d < D; ++d) launch_f32_to_f64(L0.f.u[d], c->cg_z[d], level_elems(L0.g), b);
-    launch_fcg_apply(D, L0.g, L0.d, c->cg_z, c->vdiag, c->P.inv_re, w, c->cg_q, c->sc.partial, b);
+    launch_fcg_apply(D, L0.g, c->op, L0.d, L0.f.u, c->P.inv_re, w, c->cg_q, c->sc.partial, b);
     launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_ZQ, 1.0, b);
-    launch_fcg_dir(D, L0.g, c->cg_z, w, c->cg_p, c->cg_q, r, c->sc.out, SL_ZQ, SL_PQ,
+    launch_fcg_dir(D, L0.g, L0.f.u, w, c->cg_p, c->cg_q, r, c->sc.out, SL_ZQ, SL_PQ,
                    c->sc.partial, b);
     launch_finalize_sum(c->sc.partial, nbf, c->sc.out, SL_PQ, 1.0, b);
     launch_finalize_sum(c->sc.partial + nbf, nbf, c->sc.out, SL_PRR, 1.0, b);
@@ -891,7 +886,7 @@ bfibm_status solve_v_fcg(bfibm_ctx* c, int ncycles, int* used) {
                        c->counters + 4, c->stream);
     });
     if (cs == BFIBM_OK) {   // the true FP64 residual of the final iterate, checked
-      launch_v_residual_mixed(D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re,
+      launch_v_residual_mixed(D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re,
                               c->sc.partial, s);
       launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, s);
       launch_res_check(c->sc.out, SL_VF, SL_VR, kTrueResidualSlack * c->P.rtol, c->counters + 4,
@@ -923,7 +918,7 @@ bfibm_status solve_v_fcg(bfibm_ctx* c, int ncycles, int* used) {
     if ((fn > 0.0 ? rn / fn : 0.0) <= c->P.rtol) st = BFIBM_OK;
   }
   if (c->collect_stats || tol) {   // the true FP64 residual of the final iterate
-    launch_v_residual_mixed(D, L0.g, L0.d, L0.f.uf, L0.f.u, c->vdiag, c->P.inv_re,
+    launch_v_residual_mixed(D, L0.g, c->op, L0.d, L0.f.uf, L0.f.u, c->P.inv_re,
                             c->sc.partial, s);
     launch_finalize_sum(c->sc.partial, nb, c->sc.out, SL_VR, 1.0, s);
   }
@@ -972,7 +967,6 @@ void build_coefficients(bfibm_ctx* c) {
                          c->stream);
   }
   if (c->P.precision == 1) {
-    launch_v_diag(c->D, L0.g, L0.d, c->vdiag, c->P.inv_re, c->stream);
     for (int l = 0; l < c->L; ++l) {
       launch_coef_to_f32(c->D, c->lev[l].g, c->lev[l].d, c->lev[l].f, c->stream);
       const double h = c->lev[l].g.h;
@@ -1279,8 +1273,8 @@ struct Persist {
   cudaStream_t tstream[kMaxLevels] = {};
   cudaEvent_t tfork[kMaxLevels] = {}, tjoin[kMaxLevels] = {};
   // level 0, every member
-  PList a3, ared, aflat, aconv;      // 3D, cell reductions, flat CG passes, conversions
-  PList fin3, finred, finflat;       // one item per member, gx = its producer's blocks
+  PList a3, aop, ared, aflat;        // 3D, FP64 operator passes, cell reductions, flat CG passes
+  PList finop, finred, finflat;       // one item per member, gx = its producer's blocks
   bool masked = false;               // queuing the body of a device loop
   cudaStream_t stream = nullptr, aux = nullptr;
   cudaEvent_t fork = nullptr, done = nullptr;
@@ -1695,16 +1689,18 @@ bfibm_status persist_build(Persist& P, bool tune) {
   ok &= make_items(nm, all, [&](int m) { return dim3(fcg_flat_blocks(lev(m, 0)), 1, 1); }, v);
   PK(upload(P, v, P.aflat));
   ok &= make_items(nm, all, [&](int m) {
-    return dim3(flat_convert_blocks(level_elems(lev(m, 0))), 1, 1);
+    const OpShape& S = P.mem[m]->op;
+    return dim3(S.nx * S.ny, S.nc, 1);
   }, v);
-  PK(upload(P, v, P.aconv));
+  PK(upload(P, v, P.aop));
+  P.aop.grid = std::min(P.aop.n, 2 * device_sms());   // two blocks resident per SM
   auto one_per = [&](auto nb_of) {
     v.clear();
     for (int m = 0; m < nm; ++m)
       v.push_back(BItem{m, 0, 0, 0, (unsigned short)nb_of(m), 1, 1});
   };
-  one_per([&](int m) { return red_blocks_3d(3, lev(m, 0)); });
-  PK(upload(P, v, P.fin3));
+  one_per([&](int m) { return op_blocks(P.mem[m]->op); });
+  PK(upload(P, v, P.finop));
   one_per([&](int m) { return red_grid_of(cells_of(lev(m, 0))); });
   PK(upload(P, v, P.finred));
   one_per([&](int m) { return fcg_flat_blocks(lev(m, 0)); });
@@ -1871,15 +1867,14 @@ bfibm_status b_solve_v(Persist& P) {
   launch_b_norm2(bargs(P, P.ared, 0), true, P.ared.grid, s);
   launch_b_finalize(bargs(P, P.finred, 0), 0, SL_VF, false, false, s);
   if (P.krylov) {
-    launch_b_v_residual_mixed(bargs(P, P.a3, 0), true, true, P.a3.grid, s);
-    launch_b_finalize(bargs(P, P.fin3, 0), 0, SL_VR, false, false, s);
+    launch_b_v_residual_mixed(bargs(P, P.aop, 0), true, true, P.aop.grid, s);
+    launch_b_finalize(bargs(P, P.finop, 0), 0, SL_VR, false, false, s);
     launch_b_begin(P.tab, nm, P.act, 0, SL_PQ, s);
     bfibm_status st = p_capture_while(P, 0, [&](cudaGraphConditionalHandle h) {
       cudaStream_t b = P.stream;
       for (int q = 0; q < P.inner; ++q) b_vcycle(P, 0, true);
-      launch_b_z_to_f64(bargs(P, P.aconv, 0), P.aconv.grid, b);
-      launch_b_fcg_apply(bargs(P, P.a3, 0), P.a3.grid, b);
-      launch_b_finalize(bargs(P, P.fin3, 0), 0, SL_ZQ, false, false, b);
+      launch_b_fcg_apply(bargs(P, P.aop, 0), P.aop.grid, b);
+      launch_b_finalize(bargs(P, P.finop, 0), 0, SL_ZQ, false, false, b);
       launch_b_fcg_dir(bargs(P, P.aflat, 0), SL_ZQ, SL_PQ, P.aflat.grid, b);
       launch_b_finalize(bargs(P, P.finflat, 0), 0, SL_PQ, false, false, b);
       launch_b_finalize(bargs(P, P.finflat, 0), 1, SL_PRR, false, false, b);
@@ -1889,19 +1884,19 @@ bfibm_status b_solve_v(Persist& P) {
     });
     if (st != BFIBM_OK) return st;
     // the true FP64 residual of every member's final iterate, checked
-    launch_b_v_residual_mixed(bargs(P, P.a3, 0), true, false, P.a3.grid, s);
-    launch_b_finalize(bargs(P, P.fin3, 0), 0, SL_VR, false, false, s);
+    launch_b_v_residual_mixed(bargs(P, P.aop, 0), true, false, P.aop.grid, s);
+    launch_b_finalize(bargs(P, P.finop, 0), 0, SL_VR, false, false, s);
     launch_b_res_check(P.tab, nm, SL_VF, SL_VR, kTrueResidualSlack, s);
     return BFIBM_OK;
   }
   launch_b_begin(P.tab, nm, P.act, 0, -1, s);
-  launch_b_v_residual_mixed(bargs(P, P.a3, 0), false, false, P.a3.grid, s);
+  launch_b_v_residual_mixed(bargs(P, P.aop, 0), false, false, P.aop.grid, s);
   return p_capture_while(P, 0, [&](cudaGraphConditionalHandle h) {
     cudaStream_t b = P.stream;
     for (int q = 0; q < P.inner; ++q) b_vcycle(P, 0, true);
     launch_b_add_correction(bargs(P, P.a3, 0), true, P.a3.grid, b);
-    launch_b_v_residual_mixed(bargs(P, P.a3, 0), true, false, P.a3.grid, b);
-    launch_b_finalize(bargs(P, P.fin3, 0), 0, SL_VR, false, false, b);
+    launch_b_v_residual_mixed(bargs(P, P.aop, 0), true, false, P.aop.grid, b);
+    launch_b_finalize(bargs(P, P.finop, 0), 0, SL_VR, false, false, b);
     launch_b_tol_check(h, P.tab, nm, P.act, 0, SL_VF, SL_VR, -1, P.iters, b, P.unroll == 0);
   });
 }
@@ -1914,7 +1909,7 @@ bfibm_status b_solve_p(Persist& P) {
   launch_b_norm2(bargs(P, P.ared, 0), false, P.ared.grid, s);
   launch_b_finalize(bargs(P, P.finred, 0), 0, SL_PF, false, false, s);
   launch_b_begin(P.tab, nm, P.act, 1, -1, s);
-  launch_b_p_residual_mixed(bargs(P, P.a3, 0), false, P.a3.grid, s);
+  launch_b_p_residual_mixed(bargs(P, P.aop, 0), false, P.aop.grid, s);
   return p_capture_while(P, 1, [&](cudaGraphConditionalHandle h) {
     cudaStream_t b = P.stream;
     for (int q = 0; q < P.inner; ++q) b_vcycle(P, 0, false);
@@ -1922,9 +1917,9 @@ bfibm_status b_solve_p(Persist& P) {
     launch_b_partial_sum_p(bargs(P, P.ared, 0), P.ared.grid, b);
     launch_b_finalize(bargs(P, P.finred, 0), 0, 0, false, true, b);
     launch_b_sub_scalar_p(bargs(P, P.a3, 0), P.a3.grid, b);
-    launch_b_p_residual_mixed(bargs(P, P.a3, 0), true, P.a3.grid, b);
-    launch_b_finalize(bargs(P, P.fin3, 0), 0, SL_PR, false, false, b);
-    launch_b_finalize(bargs(P, P.fin3, 0), 1, SL_PRMAX, true, false, b);
+    launch_b_p_residual_mixed(bargs(P, P.aop, 0), true, P.aop.grid, b);
+    launch_b_finalize(bargs(P, P.finop, 0), 0, SL_PR, false, false, b);
+    launch_b_finalize(bargs(P, P.finop, 0), 1, SL_PRMAX, true, false, b);
     launch_b_tol_check(h, P.tab, nm, P.act, 1, SL_PF, SL_PR, SL_PRMAX, P.iters, b,
                        P.unroll == 0);
   });
@@ -2014,6 +2009,7 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
   Geo geos[kMaxLevels];
   c->L = build_levels(*p, geos);
   for (int l = 0; l < c->L; ++l) c->lev[l].g = geos[l];
+  if (p->precision == 1 && c->D == 3) c->op = op_shape(c->lev[0].g);
   if (stream) {
     c->stream = (cudaStream_t)stream;
   } else {
@@ -2061,10 +2057,8 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
         c->rho[a] = take(Lv.g);
         c->frc[a] = take(Lv.g);
         if (p->precision == 1) {
-          c->vdiag[a] = take(Lv.g);
           c->cg_p[a] = take(Lv.g);
           c->cg_q[a] = take(Lv.g);
-          c->cg_z[a] = take(Lv.g);
         }
       }
   }
@@ -2100,7 +2094,7 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
   c->sc.out = (double*)cur;
   cur += 256;
   // remaining scalar room
-  c->partial_cap = std::max<long long>(4 * kRedBlocks, 2LL * red_blocks_3d(D, c->lev[0].g) + 64);
+  c->partial_cap = std::max<long long>(4 * kRedBlocks, 2LL * op_blocks(D, c->lev[0].g, c->op) + 64);
   if (cudaMalloc((void**)&c->sc.partial, sizeof(double) * c->partial_cap) != cudaSuccess ||
       cudaMalloc((void**)&c->step_dev, sizeof(long long)) != cudaSuccess ||
       cudaMalloc((void**)&c->counters, sizeof(int) * kCounters) != cudaSuccess ||
