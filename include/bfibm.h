@@ -276,12 +276,13 @@ bfibm_status bfibm_body_force(bfibm_ctx* c, double* G);
    default 2e9; 0 tests the barrier once without waiting. A sweep whose wait
    runs out drains its copies in flight, stops and raises
    bfibm_stats.wait_timeouts; the step then reports BFIBM_ETIMEOUT. Short
-   limits exist to exercise that path), BFIBM_OPT_TAIL (3D mixed precision:
-   the FP32 V-cycle levels of at most this many cells, down to and with the
-   FP64 coarsest solve, run in one launch per V-cycle, a cluster of 8 thread
-   blocks with a cluster barrier between phases and in-place red-black sweeps;
-   default 8192, 0 keeps one launch per sweep, residual and transfer; the same
-   results to the bit either way). */
+   limits exist to exercise that path), BFIBM_OPT_TAIL (closed ducts: the
+   V-cycle levels of at most this many cells, down to and with the FP64
+   coarsest solve, run in one launch per V-cycle where they fit the shared
+   memory of a cluster of 16 thread blocks, with a cluster barrier between
+   phases and in-place red-black sweeps; default 32768 in mixed precision, 8192
+   in FP64; 0 keeps one launch per sweep, residual and transfer; the same
+   results either way, to the bit in mixed precision, to rounding in FP64). */
 enum {
   BFIBM_OPT_STATS = 0,
   BFIBM_OPT_GRAPH = 1,
@@ -426,10 +427,10 @@ void bfibm_batch_destroy(bfibm_batch* b);
    same while k covers the iterations the slowest member needs
    (a member not done after k iterations stops there without being counted as
    unconverged). It serves a profiler that cannot see kernels inside
-   conditional graph nodes. BFIBM_BATCH_TAIL (default 4096): the levels of at
+   conditional graph nodes. BFIBM_BATCH_TAIL (default 32768): the levels of at
    most this many cells, down to and with each member's coarsest solve, run
-   in the coarse-level kernel of BFIBM_OPT_TAIL with one thread block per
-   member, on a branch of the graph beside the other members' launches (0:
+   in the cluster kernel of BFIBM_OPT_TAIL, each member's cluster as large as
+   lets the members run side by side, on a branch of the graph beside the other members' launches (0:
    one launch per level and phase throughout); the members' own
    BFIBM_OPT_TAIL does not apply in the batch, and the results are the same
    to the bit. Every option drops the current plan. */

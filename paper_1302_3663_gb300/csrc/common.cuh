@@ -45,7 +45,8 @@ struct LevelPtrs {
   T* mue[3];     // mu on edges: xy, xz, yz
   T* p2;         // second buffer of p for out-of-place sweeps
   T* u2[3];      // second buffers of u
-  T* idg[3];     // FP32 sweeps: 1 / diagonal of the viscous operator of component d
+  T* idg[3];     // 1 / diagonal of the viscous operator of component d
+  T* pdg;        // FP64: 1 / (sum of beta) of the pressure operator
 };
 
 struct Ptr3d {
@@ -123,6 +124,27 @@ struct Scalars {
   double* out;       // 16 finalized scalars
 };
 
+// -------------------------------------------------------- the cluster V-cycle
+// One level's slab of one CTA: extents, strides (elements) and the offsets of
+// its arrays in shared memory. An array is planes of two colours of R rows of
+// RS elements; point (i, r) of local plane lp sits at
+//   lp PS + ((i + r + plane) & 1) CP + r RS + i / 2.
+// Planes 1 .. npl are owned, 0 and npl + 1 are halos. Arrays without a halo
+// plane start later: their offsets are shifted so that lp indexes them too.
+struct ClLv {
+  int n0, R, nS, s0, sR;
+  int RS, CP, PS, nh;
+  unsigned mnh, mR, ms0, msR;   // ceil(2^32 / d) of nh, R, s0, sR: quotients by a high product
+  int C;                     // CTAs that share the level (1: the cluster's first alone)
+  int pc, na, last;          // planes per CTA, CTAs that own planes, planes of the last of them
+  int k0, npl;               // this CTA: the first owned plane, owned planes
+  int lo, hi, nlo;           // CTAs below and above (-1: a wall), planes of the one below
+  int per0, perR, perS;
+  int st1, st2;              // strides of the global arrays: row, plane
+  int fs;                    // right-hand sides and inverse diagonals are in shared memory
+  int u[3], f[3], g[3], c, e[3];
+};
+
 // ------------------------------------------------------- batched launches
 // The block a kernel body works on: its coordinates and the extent of the
 // grid it belongs to. A single-instance kernel passes its own blockIdx and
@@ -164,7 +186,10 @@ struct BMember {
   double dscale, div_tol;   // the pressure loop's second test: dscale max |r_p| <= div_tol
   int coarse_sweeps;
   int nu1, nu2;             // sweeps before and after the coarse-grid correction
-  int tail;                 // first level of the coarse-level cluster kernel (L: none)
+  int tail;                 // first level of the cluster V-cycle (L: none)
+  double* cmat[2];          // the coarsest solve as a matrix of ncm rows (0: none): pressure,
+  int ncm[2];               // viscous
+  ClLv cl[2][2][kMaxLevels];   // the cluster V-cycle's slabs: from the tail, the coarsest alone
   double ir[kMaxLevels];    // inv_re / h^2 per level and 1 / h^2, formed on the host (IEEE
   double ih2[kMaxLevels];   // division, the same bits as on the device) so that no thread
                             // divides in FP64
@@ -359,20 +384,6 @@ void launch_b_begin(const BMember* tab, int nm, int* act, int which, int zero_sl
 // test of the single-instance loop (||r||/||f|| from out[sr], out[sf]; with
 // smax >= 0 also dscale out[smax] <= div_tol); a member that stops leaves the
 // mask; the loop runs again while any member is active.
-// The coarse levels of an FP32 V-cycle in one launch (stencil.cu): one
-// cluster of kTailCtas CTAs per listed member runs its levels tail .. L - 1
-// (tail from the member table): nu1 in-place red-black sweeps per level,
-// residual and restriction down to the coarsest level, the FP64 coarse solve
-// there (with its conversions), prolongation and nu2 sweeps back up, with a
-// cluster barrier between phases. Same arithmetic, point for point, as the
-// launches it replaces. viscous: the viscous components, else the pressure;
-// act (may be null) masks members; smem: the largest tail_smem of the members;
-// ctas 1 gives each member one CTA (a batch's members then run side by side).
-constexpr int kTailCtas = 8;
-void launch_tail(bool viscous, const BMember* tab, const int* list, int nlist, const int* act,
-                 size_t smem, cudaStream_t s, int ctas = kTailCtas);
-size_t tail_smem(const Geo& coarsest, bool viscous);
-cudaError_t tail_set_smem();
 // iters[which] counts the loop's iterations; use_h false: no loop node to
 // steer (an unrolled loop), the masks alone decide.
 void launch_b_tol_check(cudaGraphConditionalHandle h, const BMember* tab, int nm, int* act,
@@ -414,6 +425,32 @@ void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int bx, size_t sm
 // its own buffer (items: flat blocks over the level's elements)
 void launch_b_copy_back(const BArgs& A, int K, int grid, cudaStream_t s);
 
+// ------------------------------------------------------------------ cluster.cu
+// The coarse levels of a V-cycle in one launch: one cluster of C CTAs per
+// listed member runs its levels from its tail level (or the coarsest alone) to
+// L - 1: nu1 red-black sweeps per level, residual and restriction down, the
+// coarsest solve (FP64), prolongation and nu2 sweeps up. fp64: the FP64 arrays
+// throughout, else the FP32 V-cycle with its FP64 coarsest level. act (may be
+// null) masks members; smem: the largest cl_bytes of the members.
+// per: whether x (3D: or y) is periodic in any listed member
+void launch_cluster(int D, bool fp64, bool viscous, bool per, const BMember* tab, const int* list,
+                    int nlist, const int* act, bool coarse_only, int C, size_t smem, cudaStream_t s);
+// shared memory of a CTA for levels from .. L - 1 (0: they do not fit); nd: the
+// rows of the coarsest solve's matrix (0: none; [pressure, viscous] below)
+// lv (may be null) receives the layouts
+size_t cl_bytes(int D, bool fp64, bool viscous, const Geo* g, int L, int from, int C, int nd,
+                ClLv* lv = nullptr);
+// the first level of at most `cells` cells from which a cluster of C CTAs can
+// run the rest of the cycle (L: none, or an open duct)
+int cl_first_level(int D, bool fp64, const Geo* g, int L, long long cells, int C, const int nd[2]);
+// the coarsest solve as a matrix: its rows (0: kept as sweeps), and the matrix
+// for the level's current coefficients
+int cl_matrix_rows(int D, bool viscous, const Geo& g);
+void launch_coarse_matrix(int D, bool viscous, const Geo& g, const LevelPtrs<double>& L, int sweeps,
+                          double inv_re, double* B, int n, cudaStream_t s);
+int cl_max_ctas();   // the largest cluster this device schedules: 16 or 8
+cudaError_t cl_setup();
+
 // ---------------------------------------------------------------- smooth_tma.cu
 // 3D FP32 red-black sweeps with TMA-staged inputs. Kind K: 0..2 viscous
 // component, 3 pressure; coef = inv_re / h^2 (viscous) or h^2 (pressure);
@@ -441,6 +478,8 @@ bool tma_chosen(int K, const Geo& g);
 bool tma_plan_of(int K, const Geo& g, int out[5]);
 
 // FP64-only grid stages.
+// L.idg and L.pdg from the level's coefficients
+void launch_idg64(int D, const Geo& g, const LevelPtrs<double>& L, double inv_re, cudaStream_t s);
 void launch_coef_fine(int D, const Geo& g, double* const rho[3], double* beta[3], double* m[3],
                       double msc, cudaStream_t s);
 void launch_coef_restrict(int D, const Geo& gf, const Geo& gc, const LevelPtrs<double>& F,

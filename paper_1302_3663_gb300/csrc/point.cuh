@@ -1,9 +1,8 @@
 // Point updates of the one-pass red-black sweeps (Sec. 3.5), shared by the
-// sweep kernels (smooth.cu) and the coarse-level cluster kernel (stencil.cu).
-// COH = true reads every array the sweeps write (the iterates and right-hand
-// sides) through L2 (ld.global.cg): a kernel that updates them in place and
-// reads them back after a cluster barrier must not take them from the
-// read-only cache. The arithmetic does not depend on COH.
+// sweep kernels (smooth.cu), and the expressions that the cluster V-cycle
+// (cluster.cu) shares with the per-level launches.
+// COH = true reads through L2 (ld.global.cg) what other CTAs of a cluster
+// wrote in the same launch. The arithmetic does not depend on it.
 #pragma once
 
 #include "common.cuh"
@@ -15,6 +14,43 @@ template <bool COH, typename T>
 __device__ __forceinline__ T ldm(const T* p) {
   if constexpr (COH) return __ldcg(p);
   else return *p;
+}
+
+// Roundings written out, so that every kernel that computes one of these
+// expressions gives the same bits whatever the compiler would contract.
+__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float pfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double pfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float psub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double psub(double a, double b) { return __dsub_rn(a, b); }
+
+// The viscous residual in flux form: differences first, so no diagonal is
+// formed (the V-cycles' FP32 residual, and the FP64 one of the cluster V-cycle).
+//   t = mu_c (u(+d) - u) - mu_c(-d) (u - u(-d))
+//   V = 2 t + sum_e mu_e(+e) [(u(+e) - u) + (u_e(F+e) - u_e(F+e-d))]
+//               - mu_e [(u - u(-e)) + (u_e(F) - u_e(F-d))]
+//   r = f - m u + ir V
+template <typename T>
+__device__ __forceinline__ T vr_normal(T mcp, T up, T u, T mcm, T um) {
+  return pmul(T(2), pfma(mcp, psub(up, u), -pmul(mcm, psub(u, um))));
+}
+template <typename T>
+__device__ __forceinline__ T vr_edge(T V, T u, T mep, T up, T uEp, T uEpm, T mem, T um, T uF,
+                                     T uFm) {
+  const T a = padd(psub(up, u), psub(uEp, uEpm)), b = padd(psub(u, um), psub(uF, uFm));
+  return padd(V, pfma(mep, a, -pmul(mem, b)));
+}
+template <typename T>
+__device__ __forceinline__ T vr_final(T f, T m, T u, T ir, T V) {
+  return pfma(ir, V, pfma(-m, u, f));
+}
+// the pressure residual from p_terms' sums
+template <typename T>
+__device__ __forceinline__ T pr_final(T f, T num, T dg, T p, T ih2) {
+  return pfma(-pfma(-dg, p, num), ih2, f);
 }
 
 // edge array of the (d, e) pair: xy 0, xz 1, yz 2
@@ -55,7 +91,7 @@ __device__ __forceinline__ void make_pt(const Geo& g, const int ci[3], Pt& q) {
 // Pressure: the update from the iterate's current neighbours (the red
 // points' old black neighbours, or the black points' new red ones). Neighbours
 // are summed axis 0, 1, 2, lower then upper, as in the two-kernel sweep.
-template <int D, typename T, bool COH = false>
+template <int D, typename T>
 __device__ __forceinline__ T p_red(const LevelPtrs<T>& L, const Pt& q, T h2) {
   T num = T(0), dg = T(0);
 #pragma unroll
@@ -63,23 +99,23 @@ __device__ __forceinline__ T p_red(const LevelPtrs<T>& L, const Pt& q, T h2) {
     const T* __restrict__ b = L.beta[a];
     if (!q.wm[a]) {
       T bb = b[q.F];
-      if constexpr (sizeof(T) == 4) px_acc(num, dg, bb, ldm<COH>(L.p + q.F + q.om[a]));
+      if constexpr (sizeof(T) == 4) px_acc(num, dg, bb, L.p[q.F + q.om[a]]);
       else {
-        num += bb * ldm<COH>(L.p + q.F + q.om[a]);
+        num += bb * L.p[q.F + q.om[a]];
         dg += bb;
       }
     }
     if (!q.wp[a]) {
       T bb = b[q.F + q.op[a]];
-      if constexpr (sizeof(T) == 4) px_acc(num, dg, bb, ldm<COH>(L.p + q.F + q.op[a]));
+      if constexpr (sizeof(T) == 4) px_acc(num, dg, bb, L.p[q.F + q.op[a]]);
       else {
-        num += bb * ldm<COH>(L.p + q.F + q.op[a]);
+        num += bb * L.p[q.F + q.op[a]];
         dg += bb;
       }
     }
   }
-  if constexpr (sizeof(T) == 4) return px_final(num, dg, h2, ldm<COH>(L.pf + q.F));
-  else return (num - h2 * ldm<COH>(L.pf + q.F)) / dg;
+  if constexpr (sizeof(T) == 4) return px_final(num, dg, h2, L.pf[q.F]);
+  else return (num - h2 * L.pf[q.F]) / dg;
 }
 
 // ---------------------------------------------------------------------------
@@ -96,7 +132,7 @@ struct VC {
   T cross, diag;       // diag: the diagonal (FP64) or its inverse (FP32)
 };
 
-template <int D, int d, typename T, bool COH = false>
+template <int D, int d, typename T>
 __device__ __forceinline__ void v_coef(const LevelPtrs<T>& L, const Pt& q, T ir, VC<D, d, T>& v) {
   const int F = q.F, od_m = q.om[d];
   T mcp = L.muc[F], mcm = L.muc[F + od_m];
@@ -113,8 +149,8 @@ __device__ __forceinline__ void v_coef(const LevelPtrs<T>& L, const Pt& q, T ir,
     const int Ep = F + q.op[e];
     T mep = me[Ep], mem = me[F];
     if constexpr (kIdg<T>)
-      v.cross = vx_cross(v.cross, mep, ldm<COH>(ue + Ep), ldm<COH>(ue + Ep + od_m), mem,
-                         ldm<COH>(ue + F), ldm<COH>(ue + F + od_m));
+      v.cross = vx_cross(v.cross, mep, ue[Ep], ue[Ep + od_m], mem,
+                         ue[F], ue[F + od_m]);
     else
       v.cross += mep * (ue[Ep] - ue[Ep + od_m]) - mem * (ue[F] - ue[F + od_m]);
     v.cep[k] = mep;
@@ -132,23 +168,23 @@ __device__ __forceinline__ T v_solve(T num, T diag) {
   else return num / diag;
 }
 
-template <int D, int d, typename T, bool COH = false>
+template <int D, int d, typename T>
 __device__ __forceinline__ T v_red(const LevelPtrs<T>& L, const Pt& q, T ir) {
   VC<D, d, T> v;
-  v_coef<D, d, T, COH>(L, q, ir, v);
+  v_coef<D, d, T>(L, q, ir, v);
   const T* __restrict__ ud = L.u[d];
   if constexpr (kIdg<T>) {
-    float off = vx_off(v.cross, v.cdp, ldm<COH>(ud + q.F + q.op[d]), v.cdm,
-                       ldm<COH>(ud + q.F + q.om[d]));
+    float off = vx_off(v.cross, v.cdp, ud[q.F + q.op[d]], v.cdm,
+                       ud[q.F + q.om[d]]);
     int k = 0;
 #pragma unroll
     for (int e = 0; e < D; ++e) {
       if (e == d) continue;
-      if (!q.wp[e]) off = vx_acc(off, v.cep[k], ldm<COH>(ud + q.F + q.op[e]));
-      if (!q.wm[e]) off = vx_acc(off, v.cem[k], ldm<COH>(ud + q.F + q.om[e]));
+      if (!q.wp[e]) off = vx_acc(off, v.cep[k], ud[q.F + q.op[e]]);
+      if (!q.wm[e]) off = vx_acc(off, v.cem[k], ud[q.F + q.om[e]]);
       ++k;
     }
-    return vx_final(ldm<COH>(L.uf[d] + q.F), ir, off, v.diag);
+    return vx_final(L.uf[d][q.F], ir, off, v.diag);
   } else {
     T off = v.cross + v.cdp * ud[q.F + q.op[d]] + v.cdm * ud[q.F + q.om[d]];
     int k = 0;

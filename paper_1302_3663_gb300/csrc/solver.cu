@@ -86,6 +86,19 @@ int build_levels(const bfibm_params& P, Geo out[kMaxLevels]) {
   return L;
 }
 
+// The levels with FP64 inverse diagonals: every level of an FP64 context, the
+// coarsest one in mixed precision.
+bool has_idg64(const bfibm_params& P, int l, int L) { return P.precision == 0 || l == L - 1; }
+
+// Rows of the coarsest solve's matrix (0: none). Solves to a tolerance run tens
+// of V-cycles on one set of coefficients. A fixed count of at least two gains
+// while the columns run side by side in one wave (their build then takes as long
+// as one solve by sweeps).
+int matrix_rows(const bfibm_params& P, bool V, const Geo& g) {
+  const int n = cl_matrix_rows(P.dim, V, g), vc = V ? P.vc_visc : P.vc_p;
+  return vc <= 0 || (vc >= 2 && n <= 384) ? n : 0;
+}
+
 size_t grid_pool_bytes(const bfibm_params& P, int* nlev = nullptr) {
   Geo g[kMaxLevels];
   int L = build_levels(P, g);
@@ -95,7 +108,11 @@ size_t grid_pool_bytes(const bfibm_params& P, int* nlev = nullptr) {
     // level 0: velocity, density, force; mixed precision adds the
     // flexible-CG vectors p and q
     int na = arrays_per_level(P.dim) + (l == 0 ? 3 * P.dim : 0) +
-             (l == 0 && P.precision == 1 ? 2 * P.dim : 0);
+             (l == 0 && P.precision == 1 ? 2 * P.dim : 0) +
+             (has_idg64(P, l, L) ? P.dim + 1 : 0);
+    if (l == L - 1)
+      for (int V = 0; V < 2; ++V)
+        bytes += (size_t)round_up(8LL * matrix_rows(P, V, g[l]) * matrix_rows(P, V, g[l]), 256);
     bytes += arr * na;
     if (P.precision == 1)   // the level's arrays and the inverse viscous diagonals
       bytes += (size_t)round_up(level_elems(g[l]) * 4, 256) * (arrays_per_level(P.dim) + P.dim);
@@ -161,6 +178,15 @@ const char* validate(const bfibm_params* p) {
 
 constexpr int kCounters = 8;
 
+// Levels of at most this many cells run in the cluster V-cycle (cluster.cu)
+// where they fit its shared memory: FP32 and FP64 cycles. Time per step with
+// the line on either side of a level: FP32, a 24x24x48 level (27,648 cells)
+// 26.7 -> 21.2 ms on the 48x48x96 duct, 34.3 -> 31.0 on 96x96x192; a 32x32x64
+// level (65,536) 50.9 -> 52.1 on 128x128x256. FP64, 16x16x32 and 128x64 levels
+// 2D 256x128 1.71 -> 1.60 ms, 256x128 itself 1.60 -> 1.76; a 24^3 level 2.15 ->
+// 2.30 on 48^3.
+constexpr long long kTailCells32 = 32768, kTailCells64 = 8192;
+
 }  // namespace
 
 struct bfibm_ctx {
@@ -215,9 +241,13 @@ struct bfibm_ctx {
   long long version = 0;          // changes whenever the step graph is dropped: a batch plan
                                   // built on this context is then rebuilt
   long long partial_cap = 0;      // doubles in sc.partial
-  long long tail_cells = 8192;    // BFIBM_OPT_TAIL: FP32 V-cycle levels of at most this many
-                                  // cells run in the coarse-level cluster kernel (0: none)
+  long long tail_cells = kTailCells32;   // BFIBM_OPT_TAIL: V-cycle levels of at most this many
+                                  // cells run in the cluster V-cycle (0: none)
   int tail_lev = kMaxLevels;      // the first of them (L: none)
+  size_t cl_smem[2][2] = {};      // its shared memory: [from the tail, the coarsest level alone]
+                                  // [pressure, viscous] (0: it does not fit)
+  double* cmat[2] = {nullptr, nullptr};   // the coarsest solve as a matrix: pressure, viscous
+  int ncm[2] = {0, 0};
   BMember* self_tab = nullptr;    // this context as the one member of that kernel's table
   int* self_list = nullptr;       // {0}
   std::string err;
@@ -335,11 +365,38 @@ void prolong_faces(bfibm_ctx* c, const Geo& gf, const Geo& gc, T* const ec[3], T
   for (int d = 0; d < c->D; ++d) launch_prolong_face<T>(c->D, d, gf, gc, ec[d], xf[d], c->stream);
 }
 
+// whether an axis the cluster kernel does not split into slabs is periodic
+bool cluster_per(const bfibm_ctx* c) {
+  return c->P.periodic[0] || (c->D == 3 && c->P.periodic[1]);
+}
+
+// The rest of a V-cycle from the tail level on in one cluster launch.
+bool cluster_cycle(bfibm_ctx* c, int l, bool V) {
+  if (l != c->tail_lev) return false;
+  launch_cluster(c->D, c->P.precision == 0, V, cluster_per(c), c->self_tab, c->self_list, 1, nullptr,
+                 false, cl_max_ctas(), c->cl_smem[0][V], c->stream);
+  return true;
+}
+
+// The coarsest solve on the level's FP64 arrays: the cluster kernel where the
+// slabs fit, else one block (open ducts, levels too large).
+void coarse_solve(bfibm_ctx* c, bool V) {
+  Level& Lv = c->lev[c->L - 1];
+  if (c->cl_smem[1][V])
+    launch_cluster(c->D, true, V, cluster_per(c), c->self_tab, c->self_list, 1, nullptr, true,
+                   cl_max_ctas(), c->cl_smem[1][V], c->stream);
+  else if (V)
+    launch_coarse_v<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->P.inv_re, c->stream);
+  else
+    launch_coarse_p<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->stream);
+}
+
 void vcycle_p(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
+  if (cluster_cycle(c, l, false)) return;
   if (l == c->L - 1) {
-    launch_coarse_p<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, s);
+    coarse_solve(c, false);
     return;
   }
   smooth_p(c, l, c->P.nu1);
@@ -354,8 +411,9 @@ void vcycle_p(bfibm_ctx* c, int l) {
 void vcycle_v(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
+  if (cluster_cycle(c, l, true)) return;
   if (l == c->L - 1) {
-    launch_coarse_v<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->P.inv_re, s);
+    coarse_solve(c, true);
     return;
   }
   smooth_v(c, l, c->P.nu1);
@@ -396,17 +454,19 @@ inline int dc_iterations(int vcycles, int inner) { return (vcycles + inner - 1) 
 
 long long cells_of(const Geo& g) { return (long long)g.n[0] * g.n[1] * g.n[2]; }
 
-// First level of the coarse-level cluster kernel: the first level of at most
-// tail_cells cells (3D mixed precision, closed duct), else L.
-int tail_level(const bfibm_ctx* c) {
-  if (c->D != 3 || c->P.precision != 1 || c->tail_cells <= 0 || c->P.open_flow) return c->L;
-  for (int l = 0; l < c->L; ++l)
-    if (cells_of(c->lev[l].g) <= c->tail_cells) return l;
-  return c->L;
+// the context's levels as one array
+struct Geos {
+  Geo g[kMaxLevels];
+};
+Geos geos_of(const bfibm_ctx* c) {
+  Geos q{};
+  for (int l = 0; l < c->L; ++l) q.g[l] = c->lev[l].g;
+  return q;
 }
 
 // The context as a member of a batched kernel's table.
-void fill_member(const bfibm_ctx* c, BMember& B) {
+// `tail`: the first level of its cluster V-cycle, with clusters of C CTAs.
+void fill_member(const bfibm_ctx* c, BMember& B, int tail, int C) {
   std::memset(&B, 0, sizeof(B));
   for (int l = 0; l < c->L; ++l) {
     B.g[l] = c->lev[l].g;
@@ -431,7 +491,17 @@ void fill_member(const bfibm_ctx* c, BMember& B) {
   B.coarse_sweeps = c->P.coarse_sweeps;
   B.nu1 = c->P.nu1;
   B.nu2 = c->P.nu2;
-  B.tail = c->tail_lev;
+  B.tail = tail;
+  const Geos q = geos_of(c);
+  for (int V = 0; V < 2; ++V) {
+    const bool fp64 = c->P.precision == 0;
+    if (tail < c->L) cl_bytes(c->D, fp64, V, q.g, c->L, tail, C, c->ncm[V], B.cl[0][V]);
+    if (!c->P.open_flow) cl_bytes(c->D, fp64, V, q.g, c->L, c->L - 1, C, c->ncm[V], B.cl[1][V]);
+  }
+  for (int V = 0; V < 2; ++V) {
+    B.cmat[V] = c->cmat[V];
+    B.ncm[V] = c->ncm[V];
+  }
   for (int l = 0; l < c->L; ++l) {
     const double h = c->lev[l].g.h;
     B.ir[l] = c->P.inv_re / (h * h);
@@ -441,10 +511,17 @@ void fill_member(const bfibm_ctx* c, BMember& B) {
 
 // the context's own one-member table, with its current settings
 cudaError_t upload_self(bfibm_ctx* c) {
-  c->tail_lev = tail_level(c);
+  const Geos q = geos_of(c);
+  const bool fp64 = c->P.precision == 0;
+  const int C = cl_max_ctas();
+  c->tail_lev = cl_first_level(c->D, fp64, q.g, c->L, c->tail_cells, C, c->ncm);
+  for (int V = 0; V < 2; ++V) {
+    c->cl_smem[0][V] = c->tail_lev < c->L ? cl_bytes(c->D, fp64, V, q.g, c->L, c->tail_lev, C, c->ncm[V]) : 0;
+    c->cl_smem[1][V] = c->P.open_flow ? 0 : cl_bytes(c->D, fp64, V, q.g, c->L, c->L - 1, C, c->ncm[V]);
+  }
   if (!c->self_tab) return cudaSuccess;
   BMember B;
-  fill_member(c, B);
+  fill_member(c, B, c->tail_lev, C);
   cudaError_t e = cudaMemcpyAsync(c->self_tab, &B, sizeof(B), cudaMemcpyHostToDevice, c->stream);
   return e == cudaSuccess ? cudaStreamSynchronize(c->stream) : e;
 }
@@ -671,16 +748,12 @@ void smooth_v32(bfibm_ctx* c, int l, int n) {
 void vcycle_p32(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
-  if (l == c->tail_lev) {
-    launch_tail(false, c->self_tab, c->self_list, 1, nullptr,
-                tail_smem(c->lev[c->L - 1].g, false), s);
-    return;
-  }
+  if (cluster_cycle(c, l, false)) return;
   if (l == c->L - 1) {
     long long n = level_elems(Lv.g);
     launch_f32_to_f64(Lv.f.pf, Lv.d.pf, n, s);
     cudaMemsetAsync(Lv.d.p, 0, n * sizeof(double), s);
-    launch_coarse_p<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, s);
+    coarse_solve(c, false);
     launch_f64_to_f32(Lv.d.p, Lv.f.p, n, s);
     return;
   }
@@ -696,18 +769,14 @@ void vcycle_p32(bfibm_ctx* c, int l) {
 void vcycle_v32(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
-  if (l == c->tail_lev) {
-    launch_tail(true, c->self_tab, c->self_list, 1, nullptr,
-                tail_smem(c->lev[c->L - 1].g, true), s);
-    return;
-  }
+  if (cluster_cycle(c, l, true)) return;
   if (l == c->L - 1) {
     long long n = level_elems(Lv.g);
     for (int d = 0; d < c->D; ++d) {
       launch_f32_to_f64(Lv.f.uf[d], Lv.d.uf[d], n, s);
       cudaMemsetAsync(Lv.d.u[d], 0, n * sizeof(double), s);
     }
-    launch_coarse_v<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->P.inv_re, s);
+    coarse_solve(c, true);
     for (int d = 0; d < c->D; ++d) launch_f64_to_f32(Lv.d.u[d], Lv.f.u[d], n, s);
     return;
   }
@@ -956,6 +1025,19 @@ void stage_interp_advance(bfibm_ctx* c) {
 }
 void stage_springs(bfibm_ctx* c) { launch_springs(c->D, c->lev[0].g, c->N, c->S, c->stream); }
 
+// The FP64 inverse diagonals of a level and, on the coarsest one, the matrices
+// of its solve, from the level's coefficients.
+void inverse_diagonals(bfibm_ctx* c, int l) {
+  const Level& Lv = c->lev[l];
+  if (!Lv.d.pdg) return;
+  launch_idg64(c->D, Lv.g, Lv.d, c->P.inv_re, c->stream);
+  if (l == c->L - 1)
+    for (int V = 0; V < 2; ++V)
+      if (c->ncm[V])
+        launch_coarse_matrix(c->D, V, Lv.g, Lv.d, c->P.coarse_sweeps, c->P.inv_re, c->cmat[V],
+                             c->ncm[V], c->stream);
+}
+
 void build_coefficients(bfibm_ctx* c) {
   Level& L0 = c->lev[0];
   launch_coef_fine(c->D, L0.g, c->rho, L0.d.beta, L0.d.m, c->P.sigma / c->P.dt, c->stream);
@@ -966,6 +1048,7 @@ void build_coefficients(bfibm_ctx* c) {
     launch_coef_restrict(c->D, c->lev[l - 1].g, c->lev[l].g, c->lev[l - 1].d, c->lev[l].d, gam,
                          c->stream);
   }
+  for (int l = 0; l < c->L; ++l) inverse_diagonals(c, l);
   if (c->P.precision == 1) {
     for (int l = 0; l < c->L; ++l) {
       launch_coef_to_f32(c->D, c->lev[l].g, c->lev[l].d, c->lev[l].f, c->stream);
@@ -1180,6 +1263,12 @@ bfibm_status copy_field(bfibm_ctx* c, int which, int comp, int level, void* ext,
     CK(cudaMemcpy2DAsync(ext, row, p, pitch, row, rows, kind, c->stream));
   else
     CK(cudaMemcpy2DAsync(p, pitch, ext, row, row, rows, kind, c->stream));
+  // the inverse diagonals follow their coefficients
+  if (!to_ext &&
+      (which == BFIBM_F_BETA || which == BFIBM_F_M || which == BFIBM_F_MUC || which == BFIBM_F_MUE)) {
+    inverse_diagonals(c, level);
+    CK(cudaGetLastError());
+  }
   CK(cudaStreamSynchronize(c->stream));
   return BFIBM_OK;
 }
@@ -1254,7 +1343,7 @@ struct Persist {
   int depth = 0;                     // levels of the deepest member
   int nu1 = 2, nu2 = 2, inner = 1, krylov = 0;
   int unroll = 0;                    // > 0: each solve loop unrolled to this many iterations
-  long long tail_cells = 4096;       // levels of at most this many cells: the coarse-level kernel
+  long long tail_cells = kTailCells32;   // levels of at most this many cells: the cluster V-cycle
   std::vector<int> ptail;            // each member's first level in that kernel (L: none)
   // per level l: the members that smooth on l (l below their coarsest level)
   PList swv[kMaxLevels], swp[kMaxLevels];   // ring-sweep blocks (viscous, pressure shape)
@@ -1265,8 +1354,12 @@ struct Persist {
   PList fl[kMaxLevels];   // flat blocks over the elements of l: copies after odd sweep counts
   PList co[kMaxLevels];   // one item per member whose coarsest level is l
   size_t co_smem[kMaxLevels][2] = {};
-  int* tail[kMaxLevels] = {};        // members whose coarse-level cluster kernel starts on l
+  bool per = false;                  // x or y periodic in a member
+  int C = 1;                         // CTAs per cluster of the cluster V-cycle
+  int* tail[kMaxLevels] = {};        // members whose cluster V-cycle starts on l
   int ntail[kMaxLevels] = {};
+  int* cco[kMaxLevels] = {};         // members whose coarsest level l runs in it alone
+  int ncco[kMaxLevels] = {};
   size_t tail_smem[kMaxLevels][2] = {};
   // that kernel runs on a branch of its own, beside the other members' work on
   // the same and deeper levels
@@ -1599,18 +1692,26 @@ bfibm_status persist_build(Persist& P, bool tune) {
   std::vector<BMember> host(nm);
   P.depth = 0;
   P.ptail.assign(nm, 0);
+  // the batch's own threshold, and clusters small enough that the members' run
+  // side by side in one wave; at least as large as every coarsest level that
+  // runs there needs (a member's results do not depend on the cluster's size)
+  P.C = 1;
+  while (2 * P.C * nm <= device_sms() && 2 * P.C <= cl_max_ctas()) P.C *= 2;
   for (int m = 0; m < nm; ++m) {
     const bfibm_ctx* c = P.mem[m];
-    fill_member(c, host[m]);
-    // the batch's own threshold: each member's kernel has one CTA here
-    int t = c->L;
-    for (int l = 0; P.tail_cells > 0 && l < c->L; ++l)
-      if (cells_of(c->lev[l].g) <= P.tail_cells) {
-        t = l;
-        break;
-      }
-    host[m].tail = P.ptail[m] = t;
+    const Geos q = geos_of(c);
+    for (int V = 0; V < 2; ++V)
+      while (c->cl_smem[1][V] && P.C < cl_max_ctas() &&
+             !cl_bytes(3, false, V, q.g, c->L, c->L - 1, P.C, c->ncm[V]))
+        P.C *= 2;
+  }
+  for (int m = 0; m < nm; ++m) {
+    const bfibm_ctx* c = P.mem[m];
+    const Geos q = geos_of(c);
+    P.ptail[m] = cl_first_level(3, false, q.g, c->L, P.tail_cells, P.C, c->ncm);
+    fill_member(c, host[m], P.ptail[m], P.C);
     P.depth = std::max(P.depth, c->L);
+    P.per = P.per || cluster_per(c);
   }
   PK(cudaMalloc((void**)&P.tab, nm * sizeof(BMember)));
   P.allocs.push_back(P.tab);
@@ -1622,7 +1723,6 @@ bfibm_status persist_build(Persist& P, bool tune) {
   P.allocs.push_back(P.iters);
   PK(cudaMemset(P.iters, 0, 2 * sizeof(long long)));
   PK(b_coarse_set_smem());
-  PK(tail_set_smem());
   std::vector<BItem> v;
   bool ok = true;   // every grid within the items' 16-bit block coordinates
   auto lev = [&](int m, int l) -> const Geo& { return P.mem[m]->lev[l].g; };
@@ -1650,24 +1750,37 @@ bfibm_status persist_build(Persist& P, bool tune) {
       return dim3(flat_convert_blocks(level_elems(lev(m, l))), 1, 1);
     }, v);
     PK(upload(P, v, P.fl[l]));
+    // a coarsest level outside the tail: alone in the cluster kernel where its
+    // slabs fit, else in one block (the pressure and viscous slabs of a level
+    // are told apart by launch_b_level's callers through cl_smem)
     auto coarse_here = [&](int m) { return tail_of(m) >= P.mem[m]->L && l == P.mem[m]->L - 1; };
-    ok &= make_items(nm, coarse_here, [&](int) { return dim3(1, 1, 1); }, v);
+    auto fits = [&](int m) { return P.mem[m]->cl_smem[1][0] && P.mem[m]->cl_smem[1][1]; };
+    ok &= make_items(nm, [&](int m) { return coarse_here(m) && !fits(m); },
+                     [&](int) { return dim3(1, 1, 1); }, v);
     PK(upload(P, v, P.co[l]));
-    std::vector<int> tl;
-    for (int m = 0; m < nm; ++m)
-      if (tail_of(m) == l) tl.push_back(m);
-    P.ntail[l] = (int)tl.size();
-    if (!tl.empty()) {
-      PK(cudaMalloc((void**)&P.tail[l], tl.size() * sizeof(int)));
-      P.allocs.push_back(P.tail[l]);
-      PK(cudaMemcpy(P.tail[l], tl.data(), tl.size() * sizeof(int), cudaMemcpyHostToDevice));
-    }
+    auto members = [&](auto use, int*& dev, int& n) -> cudaError_t {
+      std::vector<int> tl;
+      for (int m = 0; m < nm; ++m)
+        if (use(m)) tl.push_back(m);
+      n = (int)tl.size();
+      if (tl.empty()) return cudaSuccess;
+      cudaError_t e = cudaMalloc((void**)&dev, tl.size() * sizeof(int));
+      if (e != cudaSuccess) return e;
+      P.allocs.push_back(dev);
+      return cudaMemcpy(dev, tl.data(), tl.size() * sizeof(int), cudaMemcpyHostToDevice);
+    };
+    // (a member without a tail has its level count there, another member's level)
+    auto tail_here = [&](int m) { return tail_of(m) == l && l < P.mem[m]->L; };
+    PK(members(tail_here, P.tail[l], P.ntail[l]));
+    PK(members([&](int m) { return coarse_here(m) && fits(m); }, P.cco[l], P.ncco[l]));
     for (int vis = 0; vis < 2; ++vis) {
       size_t mx = 0, mt = 0;
       for (int m = 0; m < nm; ++m) {
-        const Geo& gc = lev(m, P.mem[m]->L - 1);
-        if (coarse_here(m)) mx = std::max(mx, b_coarse_smem(gc, vis != 0));
-        if (tail_of(m) == l) mt = std::max(mt, tail_smem(gc, vis != 0));
+        const bfibm_ctx* c = P.mem[m];
+        const Geos q = geos_of(c);
+        if (coarse_here(m) && !fits(m)) mx = std::max(mx, b_coarse_smem(lev(m, c->L - 1), vis != 0));
+        if (tail_here(m) || (coarse_here(m) && fits(m)))
+          mt = std::max(mt, cl_bytes(3, false, vis != 0, q.g, c->L, l, P.C, c->ncm[vis]));
       }
       P.co_smem[l][vis] = mx;
       P.tail_smem[l][vis] = mt;
@@ -1766,8 +1879,8 @@ void b_vcycle(Persist& P, int l, bool V) {
   if (P.ntail[l]) {   // forked: joined again at the end of this level
     cudaEventRecord(P.tfork[l], s);
     cudaStreamWaitEvent(P.tstream[l], P.tfork[l], 0);
-    launch_tail(V, P.tab, P.tail[l], P.ntail[l], P.masked ? P.act : nullptr,
-                P.tail_smem[l][V ? 1 : 0], P.tstream[l], 1);
+    launch_cluster(3, false, V, P.per, P.tab, P.tail[l], P.ntail[l], P.masked ? P.act : nullptr, false,
+                   P.C, P.tail_smem[l][V ? 1 : 0], P.tstream[l]);
     cudaEventRecord(P.tjoin[l], P.tstream[l]);
   }
   b_level(P, l, V);
@@ -1779,6 +1892,8 @@ void b_vcycle(Persist& P, int l, bool V) {
 void b_level(Persist& P, int l, bool V) {
   cudaStream_t s = P.stream;
   if (P.co[l].n) launch_b_coarse(bargs(P, P.co[l], l), V, P.co_smem[l][V ? 1 : 0], s);
+  launch_cluster(3, false, V, P.per, P.tab, P.cco[l], P.ncco[l], P.masked ? P.act : nullptr, true, P.C,
+                 P.tail_smem[l][V ? 1 : 0], s);
   if (!P.en[l].n) return;
   b_smooth(P, l, P.nu1, V);
   if (V) {
@@ -2006,6 +2121,7 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
   c->version = next_version();
   c->P = *p;
   c->D = p->dim;
+  c->tail_cells = p->precision == 1 ? kTailCells32 : kTailCells64;
   Geo geos[kMaxLevels];
   c->L = build_levels(*p, geos);
   for (int l = 0; l < c->L; ++l) c->lev[l].g = geos[l];
@@ -2051,6 +2167,16 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
     }
     d.muc = take(Lv.g);
     for (int e = 0; e < E; ++e) d.mue[e] = take(Lv.g);
+    if (has_idg64(*p, l, c->L)) {
+      for (int a = 0; a < D; ++a) d.idg[a] = take(Lv.g);
+      d.pdg = take(Lv.g);
+    }
+    if (l == c->L - 1)
+      for (int V = 0; V < 2; ++V) {
+        const long long n = c->ncm[V] = matrix_rows(*p, V, Lv.g);
+        c->cmat[V] = n ? (double*)cur : nullptr;
+        cur += round_up(8 * n * n, 256);
+      }
     if (l == 0)
       for (int a = 0; a < D; ++a) {
         c->uvel[a] = take(Lv.g);
@@ -2143,12 +2269,12 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
     }
   }
   if (coarse_set_smem() != cudaSuccess || fused_set_carveout() != cudaSuccess ||
-      tail_set_smem() != cudaSuccess) {
+      cl_setup() != cudaSuccess) {
     cudaGetLastError();
     bfibm_destroy(c);
     return BFIBM_ECUDA;
   }
-  if (p->precision == 1 && D == 3) {
+  if (!p->open_flow) {
     static const int zero = 0;
     if (cudaMalloc((void**)&c->self_tab, sizeof(BMember)) != cudaSuccess ||
         cudaMalloc((void**)&c->self_list, sizeof(int)) != cudaSuccess ||
@@ -2829,7 +2955,7 @@ struct bfibm_batch {
   int persistent = 0;    // BFIBM_BATCH_PERSISTENT
   int tune = 1;          // BFIBM_BATCH_TUNE
   int unroll = 0;        // BFIBM_BATCH_UNROLL
-  long long tail = 4096; // BFIBM_BATCH_TAIL
+  long long tail = kTailCells32;   // BFIBM_BATCH_TAIL
   Persist* ps = nullptr; // the plan of the last persistent step
   long long builds = 0;  // plans built
   std::string err;

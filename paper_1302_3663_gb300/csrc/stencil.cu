@@ -14,6 +14,7 @@
 
 #include "common.cuh"
 #include "point.cuh"
+#include "transfer.cuh"
 
 namespace bf {
 
@@ -117,7 +118,7 @@ __device__ __forceinline__ void decode(const Geo& g, long long idx, int& i, int&
 // beta_nb p_nb over the existing neighbours, dg = sum of beta_nb; then
 // (A p)(c) = (num - dg p(c)) / h^2. No flux crosses a wall.
 // ---------------------------------------------------------------------------
-template <int D, typename T, bool COH = false>
+template <int D, typename T>
 __device__ __forceinline__ void p_terms(const Geo& g, const LevelPtrs<T>& L, const int ci[3],
                                         long long c, T& num, T& dg) {
   num = T(0);
@@ -128,18 +129,18 @@ __device__ __forceinline__ void p_terms(const Geo& g, const LevelPtrs<T>& L, con
     if (ci[a] > 0 || g.per[a]) {
       long long cm = c + offm(g, a, ci[a]);
       T bb = b[c];
-      num += bb * ldm<COH>(L.p + cm);
-      dg += bb;
+      num = pfma(bb, L.p[cm], num);
+      dg = padd(dg, bb);
     }
     if (ci[a] < g.n[a] - 1 || g.per[a]) {
       long long cp = c + offp(g, a, ci[a]);
       T bb = b[cp];
-      num += bb * ldm<COH>(L.p + cp);
-      dg += bb;
+      num = pfma(bb, L.p[cp], num);
+      dg = padd(dg, bb);
     } else if (is_open(g, a)) {
       // the outflow face, pressure held there: the homogeneous ghost -p
       // (the held value is in the right-hand side)
-      dg += T(2) * b[c + st_of(g, a)];
+      dg = pfma(T(2), b[c + st_of(g, a)], dg);
     }
   }
 }
@@ -161,12 +162,12 @@ __global__ void __launch_bounds__(256) k_p_rbgs(Geo g, LevelPtrs<T> L, int colou
 }
 
 // ih2 = (T)(1 / h^2), formed once on the host
-template <int D, typename T, bool COH = false>
+template <int D, typename T>
 __device__ __forceinline__ void p_residual_at(const Geo& g, const LevelPtrs<T>& L,
                                               const int ci[3], long long c, T ih2) {
   T num, dg;
-  p_terms<D, T, COH>(g, L, ci, c, num, dg);
-  L.pr[c] = ldm<COH>(L.pf + c) - (num - dg * ldm<COH>(L.p + c)) * ih2;
+  p_terms<D, T>(g, L, ci, c, num, dg);
+  L.pr[c] = pr_final(L.pf[c], num, dg, L.p[c], ih2);
 }
 
 template <int D, typename T>
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(256) k_p_residual(Geo g, LevelPtrs<T> L, T ih2
 // that edge contributes its cross term only.
 // q: the point's neighbour offsets and wall flags (make_pt), formed once per
 // point and shared by the components of a residual.
-template <int D, int d, typename T, bool COH = false>
+template <int D, int d, typename T>
 __device__ __forceinline__ void v_terms_q(const Geo& g, const LevelPtrs<T>& L, const int ci[3],
                                           const Pt& q, T& off, T& dgV) {
   const T* __restrict__ ud = L.u[d];
@@ -208,7 +209,7 @@ __device__ __forceinline__ void v_terms_q(const Geo& g, const LevelPtrs<T>& L, c
   const int od_m = q.om[d];
   const int od_p = outflow ? od_m : q.op[d];
   T mcp = outflow ? L.muc[F + od_m] : L.muc[F], mcm = L.muc[F + od_m];
-  off = T(2) * (mcp * ldm<COH>(ud + F + od_p) + mcm * ldm<COH>(ud + F + od_m));
+  off = T(2) * (mcp * ud[F + od_p] + mcm * ud[F + od_m]);
   dgV = T(2) * (mcp + mcm);
 #pragma unroll
   for (int e = 0; e < D; ++e) {
@@ -220,22 +221,22 @@ __device__ __forceinline__ void v_terms_q(const Geo& g, const LevelPtrs<T>& L, c
     bool neu = wp && e == g.open;   // beyond the outflow: even ghost, no weight
     const int Ep = F + q.op[e];     // e-face index ci[e] + 1
     T mep = me[Ep], mem = me[F];
-    T cp = outflow ? T(0) : ldm<COH>(ue + Ep) - ldm<COH>(ue + Ep + od_m);
-    T cm = outflow ? T(0) : ldm<COH>(ue + F) - ldm<COH>(ue + F + od_m);
+    T cp = outflow ? T(0) : ue[Ep] - ue[Ep + od_m];
+    T cm = outflow ? T(0) : ue[F] - ue[F + od_m];
     T udp = T(0), udm = T(0);
-    if (!wp) udp = ldm<COH>(ud + Ep);
-    if (!wm) udm = ldm<COH>(ud + F + q.om[e]);
+    if (!wp) udp = ud[Ep];
+    if (!wm) udm = ud[F + q.om[e]];
     off += mep * (udp + cp) + mem * (udm - cm);
     dgV += (neu ? T(0) : (wp ? T(2) : T(1))) * mep + (wm ? T(2) : T(1)) * mem;
   }
 }
 
-template <int D, int d, typename T, bool COH = false>
+template <int D, int d, typename T>
 __device__ __forceinline__ void v_terms(const Geo& g, const LevelPtrs<T>& L, const int ci[3],
                                         long long F, T& off, T& dgV) {
   Pt q;
   make_pt<D>(g, ci, q);
-  v_terms_q<D, d, T, COH>(g, L, ci, q, off, dgV);
+  v_terms_q<D, d, T>(g, L, ci, q, off, dgV);
 }
 
 template <int D, int d, typename T>
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_v_rbgs(Geo g, LevelPtrs<T> L, int colou
   L.u[d][F] = (L.uf[d][F] + ir * off) / (L.m[d][F] + ir * dgV);
 }
 
-template <int D, int d, typename T, bool COH = false>
+template <int D, int d, typename T>
 __device__ __forceinline__ void v_residual_point(const Geo& g, const LevelPtrs<T>& L,
                                                  const int ci[3], const Pt& q, T ir) {
   const int F = q.F;
@@ -267,9 +268,25 @@ __device__ __forceinline__ void v_residual_point(const Geo& g, const LevelPtrs<T
     L.ur[d][F] = T(0);
     return;
   }
-  T off, dgV;
-  v_terms_q<D, d, T, COH>(g, L, ci, q, off, dgV);
-  L.ur[d][F] = ldm<COH>(L.uf[d] + F) - (L.m[d][F] + ir * dgV) * ldm<COH>(L.u[d] + F) + ir * off;
+  if constexpr (sizeof(T) == 4) {   // the FP32 V-cycles run in closed ducts only
+    const T* __restrict__ ud = L.u[d];
+    const T u = ud[F];
+    T V = vr_normal(L.muc[F], ud[F + q.op[d]], u, L.muc[F + q.om[d]], ud[F + q.om[d]]);
+#pragma unroll
+    for (int e = 0; e < D; ++e) {
+      if (e == d) continue;
+      const T* __restrict__ ue = L.u[e];
+      const T* __restrict__ me = L.mue[edge_id(d, e)];
+      const int Ep = F + q.op[e];
+      const T up = q.wp[e] ? -u : ud[Ep], um = q.wm[e] ? -u : ud[F + q.om[e]];
+      V = vr_edge(V, u, me[Ep], up, ue[Ep], ue[Ep + q.om[d]], me[F], um, ue[F], ue[F + q.om[d]]);
+    }
+    L.ur[d][F] = vr_final(L.uf[d][F], L.m[d][F], u, ir, V);
+  } else {
+    T off, dgV;
+    v_terms_q<D, d, T>(g, L, ci, q, off, dgV);
+    L.ur[d][F] = L.uf[d][F] - (L.m[d][F] + ir * dgV) * L.u[d][F] + ir * off;
+  }
 }
 
 template <int D, typename T>
@@ -292,32 +309,6 @@ __global__ void __launch_bounds__(256) k_v_residual(Geo g, LevelPtrs<T> L, T ir)
   v_residual_body<D, T>(own_blk(), g, L, ir);
 }
 
-// ---------------------------------------------------------------------------
-// Grid transfers (Sec. 3.5).
-// Cell-centred restriction: mean of the 2^D children. Face restriction along
-// its own axis: (1/4, 1/2, 1/4) on the faces 2I-1, 2I, 2I+1; across the other
-// axes the mean of the two children. Both zero the coarse iterate.
-// ---------------------------------------------------------------------------
-template <int D, typename T, bool COH = false>
-__device__ __forceinline__ void restrict_cell_at(const Geo& gf, const Geo& gc,
-                                                 const T* __restrict__ rf, T* __restrict__ fc,
-                                                 T* __restrict__ xc, int I, int J, int K) {
-  long long f0 = gidx(gf, 2 * I, 2 * J, D == 3 ? 2 * K : 0);
-  long long sy = gf.st[1], sz = gf.st[2];
-  T s = ldm<COH>(rf + f0) + ldm<COH>(rf + f0 + 1);
-  s += ldm<COH>(rf + f0 + sy);
-  s += ldm<COH>(rf + f0 + sy + 1);
-  if constexpr (D == 3) {
-    s += ldm<COH>(rf + f0 + sz);
-    s += ldm<COH>(rf + f0 + sz + 1);
-    s += ldm<COH>(rf + f0 + sz + sy);
-    s += ldm<COH>(rf + f0 + sz + sy + 1);
-  }
-  long long c = gidx(gc, I, J, K);
-  fc[c] = s * (D == 3 ? T(0.125) : T(0.25));
-  xc[c] = T(0);
-}
-
 template <int D, typename T>
 __device__ __forceinline__ void restrict_cell_body(const Blk& B, Geo gf, Geo gc,
                                                    const T* __restrict__ rf, T* __restrict__ fc,
@@ -333,45 +324,6 @@ template <int D, typename T>
 __global__ void __launch_bounds__(256) k_restrict_cell(Geo gf, Geo gc, const T* __restrict__ rf,
                                                        T* __restrict__ fc, T* __restrict__ xc) {
   restrict_cell_body<D, T>(own_blk(), gf, gc, rf, fc, xc);
-}
-
-// one coarse face C (a stored face along d, a cell across it)
-template <int D, int d, typename T, bool COH = false>
-__device__ __forceinline__ void restrict_face_at(const Geo& gf, const Geo& gc,
-                                                 const T* __restrict__ rf, T* __restrict__ fc,
-                                                 T* __restrict__ xc, const int C[3]) {
-  long long c = gidx(gc, C[0], C[1], C[2]);
-  xc[c] = T(0);
-  bool wallface = !gc.per[d] && (C[d] == 0 || (C[d] == gc.n[d] && d != gc.open));
-  if (wallface) {
-    fc[c] = T(0);
-    return;
-  }
-  constexpr int ta = (d == 0) ? 1 : 0;
-  constexpr int tb = (D == 3) ? ((d == 2) ? 1 : 2) : -1;
-  int nf = gf.n[d];
-  int f[3] = {0, 0, 0};
-  T s = T(0);
-#pragma unroll
-  for (int t2 = 0; t2 < (D == 3 ? 2 : 1); ++t2) {
-#pragma unroll
-    for (int t1 = 0; t1 < 2; ++t1) {
-      f[ta] = 2 * C[ta] + t1;
-      if constexpr (tb >= 0) f[tb] = 2 * C[tb] + t2;
-      T along = T(0);
-#pragma unroll
-      for (int o = -1; o <= 1; ++o) {
-        int q = 2 * C[d] + o;
-        if (gf.per[d]) q = q < 0 ? q + nf : (q >= nf ? q - nf : q);
-        if (d == gf.open && q > nf) q = nf - 1;   // even ghost beyond the outflow
-        f[d] = q;
-        T w = (o == 0) ? T(0.5) : T(0.25);
-        along += w * ldm<COH>(rf + gidx(gf, f[0], f[1], f[2]));
-      }
-      s += along;
-    }
-  }
-  fc[c] = s * (D == 3 ? T(0.25) : T(0.5));
 }
 
 template <int D, int d, typename T>
@@ -423,99 +375,6 @@ __global__ void __launch_bounds__(256) k_restrict_face3(Geo gf, Geo gc, Faces3<T
   restrict_face3_body<T>(own_blk(), gf, gc, rf, fc, xc);
 }
 
-// 1D prolongation weights. Cell-centred axis: 3/4 on the parent, 1/4 on the
-// next coarse cell toward the child; beyond a wall the mirror ghost
-// (sign `mirror`) folds that 1/4 into the parent. Face axis: the coincident
-// coarse face, or the mean of the two coarse faces around a midway face.
-// The weights are exact binary fractions in any precision.
-template <typename T>
-__device__ __forceinline__ int prol_cell_1d(int i, int nc, int per, int mirror_lo, int mirror_hi,
-                                            int idx[2], T w[2]) {
-  int I = i >> 1;
-  int J = I + ((i & 1) ? 1 : -1);
-  idx[0] = I;
-  w[0] = T(0.75);
-  w[1] = T(0);
-  if (per) {
-    idx[1] = J < 0 ? J + nc : (J >= nc ? J - nc : J);
-    w[1] = T(0.25);
-    return 2;
-  }
-  if (J < 0 || J >= nc) {
-    const int mirror = J < 0 ? mirror_lo : mirror_hi;
-    w[0] = mirror > 0 ? T(1) : T(0.5);
-    idx[1] = I;   // weight 0: any valid index
-    return 1;
-  }
-  idx[1] = J;
-  w[1] = T(0.25);
-  return 2;
-}
-template <typename T>
-__device__ __forceinline__ int prol_face_1d(int i, int nc, int per, int idx[2], T w[2]) {
-  int I = i >> 1;
-  w[1] = T(0);
-  if ((i & 1) == 0) {
-    idx[0] = I;   // a fine face index is below 2 nc, so I < nc
-    idx[1] = I;   // weight 0: any valid index
-    w[0] = T(1);
-    return 1;
-  }
-  idx[0] = I;
-  w[0] = T(0.5);
-  idx[1] = (per && I + 1 == nc) ? 0 : I + 1;
-  w[1] = T(0.5);
-  return 2;
-}
-
-// Roundings of the prolongation written out, so that every form of it (one
-// point per thread, two points per thread, the coarse-level cluster kernel)
-// gives the same bits whatever the compiler would contract.
-__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float pfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double pfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
-
-// separable tensor-product sum: x-rows first, then y, then z, each pair of
-// terms as w1 t1 + (w0 t0) with one rounding of the product and one of the
-// fused sum. Every axis takes two terms; a missing term has weight 0 and a
-// valid index, and adding its exact zero leaves the sum unchanged, so the
-// loops unroll fully and the index and weight arrays stay in registers.
-template <typename T, bool COH = false>
-__device__ __forceinline__ T prol_sum(const Geo& gc, const T* __restrict__ ec, const int idx[3][2],
-                                      const T w[3][2]) {
-  T col[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    T row[2];
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      long long r = gidx(gc, 0, idx[1][b], idx[2][c]);
-      row[b] = pfma(w[0][1], ldm<COH>(ec + r + idx[0][1]), pmul(w[0][0], ldm<COH>(ec + r + idx[0][0])));
-    }
-    col[c] = pfma(w[1][1], row[1], pmul(w[1][0], row[0]));
-  }
-  return pfma(w[2][1], col[1], pmul(w[2][0], col[0]));
-}
-
-// the coarse correction added at one fine cell fi
-template <int D, typename T, bool COH = false>
-__device__ __forceinline__ void prolong_cell_at(const Geo& gf, const Geo& gc,
-                                                const T* __restrict__ ec, T* __restrict__ xf,
-                                                const int fi[3]) {
-  int idx[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-  T w[3][2] = {{T(1), T(0)}, {T(1), T(0)}, {T(1), T(0)}};
-  // the pressure correction mirrors evenly at walls and the inflow, oddly at
-  // the outflow, where the pressure is held
-#pragma unroll
-  for (int a = 0; a < D; ++a)
-    prol_cell_1d<T>(fi[a], gc.n[a], gc.per[a], +1, a == gc.open ? -1 : +1, idx[a], w[a]);
-  const long long x = gidx(gf, fi[0], fi[1], fi[2]);
-  xf[x] = padd(ldm<COH>(xf + x), prol_sum<T, COH>(gc, ec, idx, w));
-}
-
 template <int D, typename T>
 __device__ __forceinline__ void prolong_cell_body(const Blk& B, Geo gf, Geo gc,
                                                   const T* __restrict__ ec, T* __restrict__ xf) {
@@ -531,24 +390,6 @@ template <int D, typename T>
 __global__ void __launch_bounds__(256) k_prolong_cell(Geo gf, Geo gc, const T* __restrict__ ec,
                                                       T* __restrict__ xf) {
   prolong_cell_body<D, T>(own_blk(), gf, gc, ec, xf);
-}
-
-// the coarse correction added at one fine face fi of component d (not a wall face)
-template <int D, int d, typename T, bool COH = false>
-__device__ __forceinline__ void prolong_face_at(const Geo& gf, const Geo& gc,
-                                                const T* __restrict__ ec, T* __restrict__ xf,
-                                                const int fi[3]) {
-  int idx[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-  T w[3][2] = {{T(1), T(0)}, {T(1), T(0)}, {T(1), T(0)}};
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    if (a == d)
-      prol_face_1d<T>(fi[a], gc.n[a], gc.per[a], idx[a], w[a]);
-    else   // tangential velocity: odd at walls and the inflow, even beyond the outflow
-      prol_cell_1d<T>(fi[a], gc.n[a], gc.per[a], -1, a == gc.open ? +1 : -1, idx[a], w[a]);
-  }
-  const long long x = gidx(gf, fi[0], fi[1], fi[2]);
-  xf[x] = padd(ldm<COH>(xf + x), prol_sum<T, COH>(gc, ec, idx, w));
 }
 
 template <int D, int d, typename T>
@@ -876,6 +717,40 @@ template <int D, typename T>
 __global__ void __launch_bounds__(1024) k_coarse_v(Geo g, LevelPtrs<T> Lg, int sweeps, T ir,
                                                    long long nel, int use_smem) {
   coarse_v_body<D, T>(own_blk(), g, Lg, sweeps, ir, nel, use_smem);
+}
+
+// 1 / diagonal of both FP64 operators on every unknown of a level (0 on the
+// fixed wall faces), formed once when the coefficients change: an FP64
+// division and the diagonal's sums cost as much as the rest of an update.
+template <int D, int d>
+__device__ __forceinline__ void idg64_point(const Geo& g, const LevelPtrs<double>& L,
+                                            const int ci[3], long long F, double ir) {
+  if (beyond_outflow<d>(g, ci)) return;
+  double v = 0.0;
+  if (g.per[d] || ci[d] != 0) {
+    double off, dgV;
+    v_terms<D, d, double>(g, L, ci, F, off, dgV);
+    v = 1.0 / (L.m[d][F] + ir * dgV);
+  }
+  L.idg[d][F] = v;
+}
+template <int D>
+__global__ void __launch_bounds__(256) k_idg64(Geo g, LevelPtrs<double> L, double ir) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int j = blockIdx.y * blockDim.y + threadIdx.y;
+  int k = blockIdx.z * blockDim.z + threadIdx.z;
+  if (i >= g.n[0] + (g.open == 0) || j >= g.n[1] + (g.open == 1) || k >= g.n[2] + (g.open == 2))
+    return;
+  const int ci[3] = {i, j, k};
+  const long long F = gidx(g, i, j, k);
+  idg64_point<D, 0>(g, L, ci, F, ir);
+  idg64_point<D, 1>(g, L, ci, F, ir);
+  if constexpr (D == 3) idg64_point<D, 2>(g, L, ci, F, ir);
+  if (i < g.n[0] && j < g.n[1] && k < g.n[2]) {
+    double num, dg;
+    p_terms<D, double>(g, L, ci, F, num, dg);
+    L.pdg[F] = 1.0 / dg;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1592,240 +1467,6 @@ __global__ void kb_res_check(const BMember* __restrict__ tab, int nm, int sf, in
 }
 
 
-// ===========================================================================
-// Coarse-level V-cycle in one launch (one cluster per member). The levels
-// below a few thousand cells cost a launch per sweep, residual, transfer and
-// conversion, each a few microseconds of mostly idle GPU; here one cluster of
-// kTailCtas CTAs runs them all, phase after phase, with a cluster barrier
-// (release / acquire) between phases. Sweeps are in place: all red points of
-// a component, a barrier, all black points. The red update reads the old
-// black neighbours and the black update the new red ones, as in the one-pass
-// sweeps, with the same point function (v_red / p_red), so the bits are those
-// of the launches it replaces. Every array a phase writes is read back through
-// L2 (the COH point functions), never through the read-only cache.
-// ===========================================================================
-// the barrier between phases: the cluster's (release / acquire at cluster
-// scope), or the block's when the member has one CTA
-template <int C>
-__device__ __forceinline__ void tail_sync() {
-  if constexpr (C == 1) {
-    __syncthreads();
-  } else {
-    asm volatile("barrier.cluster.arrive.release;\n\t"
-                 "barrier.cluster.wait.acquire;" ::: "memory");
-  }
-}
-
-// one colour of viscous component d on level g, in place
-template <int d>
-__device__ __forceinline__ void tail_v_colour(const Geo& g, const LevelPtrs<float>& L, float ir,
-                                              int colour, int t0, int T) {
-  const int nh = (g.n[0] + 1) >> 1;
-  const int npts = nh * g.n[1] * g.n[2];
-  for (int q = t0; q < npts; q += T) {
-    const int ih = q % nh, r = q / nh;
-    const int j = r % g.n[1], k = r / g.n[1];
-    const int i = 2 * ih + ((j + k + colour) & 1);
-    if (i >= g.n[0]) continue;
-    const int ci[3] = {i, j, k};
-    if (!g.per[d] && ci[d] == 0) continue;   // the wall face stays 0
-    Pt pt;
-    make_pt<3>(g, ci, pt);
-    L.u[d][pt.F] = v_red<3, d, float, true>(L, pt, ir);
-  }
-}
-
-__device__ __forceinline__ void tail_p_colour(const Geo& g, const LevelPtrs<float>& L, float h2,
-                                              int colour, int t0, int T) {
-  const int nh = (g.n[0] + 1) >> 1;
-  const int npts = nh * g.n[1] * g.n[2];
-  for (int q = t0; q < npts; q += T) {
-    const int ih = q % nh, r = q / nh;
-    const int j = r % g.n[1], k = r / g.n[1];
-    const int i = 2 * ih + ((j + k + colour) & 1);
-    if (i >= g.n[0]) continue;
-    const int ci[3] = {i, j, k};
-    Pt pt;
-    make_pt<3>(g, ci, pt);
-    L.p[pt.F] = p_red<3, float, true>(L, pt, h2);
-  }
-}
-
-template <bool V, int C>
-__device__ __forceinline__ void tail_smooth(const BMember& M, int l, int n, int t0, int T) {
-  const Geo g = M.g[l];
-  const LevelPtrs<float> L = M.f[l];
-  for (int it = 0; it < n; ++it) {
-    if (V) {
-      const float ir = (float)M.ir[l];
-      for (int c = 0; c < 2; ++c) {
-        tail_v_colour<0>(g, L, ir, c, t0, T);
-        tail_sync<C>();
-      }
-      for (int c = 0; c < 2; ++c) {
-        tail_v_colour<1>(g, L, ir, c, t0, T);
-        tail_sync<C>();
-      }
-      for (int c = 0; c < 2; ++c) {
-        tail_v_colour<2>(g, L, ir, c, t0, T);
-        tail_sync<C>();
-      }
-    } else {
-      const float h2 = (float)(g.h * g.h);
-      for (int c = 0; c < 2; ++c) {
-        tail_p_colour(g, L, h2, c, t0, T);
-        tail_sync<C>();
-      }
-    }
-  }
-}
-
-// residual on level l, restricted to level l + 1 (whose iterate it zeroes)
-template <bool V, int C>
-__device__ __forceinline__ void tail_down(const BMember& M, int l, int t0, int T) {
-  const Geo g = M.g[l], gc = M.g[l + 1];
-  const LevelPtrs<float> L = M.f[l], Lc = M.f[l + 1];
-  const int ncell = g.n[0] * g.n[1] * g.n[2];
-  const float ir = (float)M.ir[l];
-  for (int q = t0; q < ncell; q += T) {
-    const int ci[3] = {q % g.n[0], (q / g.n[0]) % g.n[1], q / (g.n[0] * g.n[1])};
-    Pt pt;
-    make_pt<3>(g, ci, pt);
-    if (V) {
-      v_residual_point<3, 0, float, true>(g, L, ci, pt, ir);
-      v_residual_point<3, 1, float, true>(g, L, ci, pt, ir);
-      v_residual_point<3, 2, float, true>(g, L, ci, pt, ir);
-    } else {
-      p_residual_at<3, float, true>(g, L, ci, pt.F, (float)M.ih2[l]);
-    }
-  }
-  tail_sync<C>();
-  if (V) {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      // along d the stored faces (walls included), across d the cells
-      const int e0 = d == 0 ? gc.s[0] : gc.n[0], e1 = d == 1 ? gc.s[1] : gc.n[1],
-                e2 = d == 2 ? gc.s[2] : gc.n[2];
-      for (int q = t0; q < e0 * e1 * e2; q += T) {
-        const int cc[3] = {q % e0, (q / e0) % e1, q / (e0 * e1)};
-        if (d == 0) restrict_face_at<3, 0, float, true>(g, gc, L.ur[0], Lc.uf[0], Lc.u[0], cc);
-        else if (d == 1) restrict_face_at<3, 1, float, true>(g, gc, L.ur[1], Lc.uf[1], Lc.u[1], cc);
-        else restrict_face_at<3, 2, float, true>(g, gc, L.ur[2], Lc.uf[2], Lc.u[2], cc);
-      }
-    }
-  } else {
-    const int nc = gc.n[0] * gc.n[1] * gc.n[2];
-    for (int q = t0; q < nc; q += T)
-      restrict_cell_at<3, float, true>(g, gc, L.pr, Lc.pf, Lc.p, q % gc.n[0],
-                                       (q / gc.n[0]) % gc.n[1], q / (gc.n[0] * gc.n[1]));
-  }
-  tail_sync<C>();
-}
-
-// the correction of level l + 1 prolonged onto level l
-template <bool V, int C>
-__device__ __forceinline__ void tail_up(const BMember& M, int l, int t0, int T) {
-  const Geo g = M.g[l], gc = M.g[l + 1];
-  const LevelPtrs<float> L = M.f[l], Lc = M.f[l + 1];
-  const int ncell = g.n[0] * g.n[1] * g.n[2];
-  for (int q = t0; q < ncell; q += T) {
-    const int fi[3] = {q % g.n[0], (q / g.n[0]) % g.n[1], q / (g.n[0] * g.n[1])};
-    if (V) {
-      if (g.per[0] || fi[0] != 0) prolong_face_at<3, 0, float, true>(g, gc, Lc.u[0], L.u[0], fi);
-      if (g.per[1] || fi[1] != 0) prolong_face_at<3, 1, float, true>(g, gc, Lc.u[1], L.u[1], fi);
-      if (g.per[2] || fi[2] != 0) prolong_face_at<3, 2, float, true>(g, gc, Lc.u[2], L.u[2], fi);
-    } else {
-      prolong_cell_at<3, float, true>(g, gc, Lc.p, L.p, fi);
-    }
-  }
-  tail_sync<C>();
-}
-
-// the coarsest level, on the cluster's first CTA: as kb_coarse
-template <bool V, int C>
-__device__ __forceinline__ void tail_coarse(const BMember& M, int rank) {
-  const int l = M.L - 1;
-  if (rank == 0) {
-    const Geo g = M.g[l];
-    const LevelPtrs<double> Ld = M.d[l];
-    const LevelPtrs<float> Lf = M.f[l];
-    const long long nel = g.st[2] * g.s[2];
-    for (long long q = threadIdx.x; q < nel; q += blockDim.x) {
-      if (V) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          Ld.uf[d][q] = (double)__ldcg(Lf.uf[d] + q);
-          Ld.u[d][q] = 0.0;
-        }
-      } else {
-        Ld.pf[q] = (double)__ldcg(Lf.pf + q);
-        Ld.p[q] = 0.0;
-      }
-    }
-    __syncthreads();
-    const int use = coarse_bytes(3, g, (int)sizeof(double), V) <= kCoarseSmemMax;
-    const Blk B{0, 0, 0, 1, 1, 1};
-    if (V) coarse_v_body<3, double>(B, g, Ld, M.coarse_sweeps, M.ir[l], nel, use);
-    else coarse_p_body<3, double>(B, g, Ld, M.coarse_sweeps, nel, use);
-    __syncthreads();
-    for (long long q = threadIdx.x; q < nel; q += blockDim.x) {
-      if (V) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) Lf.u[d][q] = (float)Ld.u[d][q];
-      } else {
-        Lf.p[q] = (float)Ld.p[q];
-      }
-    }
-  }
-  tail_sync<C>();
-}
-
-// one member per C CTAs (a cluster when C > 1)
-template <bool V, int C>
-__device__ __forceinline__ void tail_run(const BMember* __restrict__ tab,
-                                         const int* __restrict__ list, int nlist,
-                                         const int* __restrict__ act) {
-  const int item = blockIdx.x / C;
-  if (item >= nlist) return;
-  const int m = list[item];
-  if (act && !act[m]) return;               // all C CTAs leave together
-  const BMember& M = tab[m];
-  const int rank = blockIdx.x % C;
-  const int t0 = rank * blockDim.x + threadIdx.x, T = C * blockDim.x;
-  const int ls = M.tail, lc = M.L - 1;
-  for (int l = ls; l < lc; ++l) {
-    tail_smooth<V, C>(M, l, M.nu1, t0, T);
-    tail_down<V, C>(M, l, t0, T);
-  }
-  tail_coarse<V, C>(M, rank);
-  for (int l = lc - 1; l >= ls; --l) {
-    tail_up<V, C>(M, l, t0, T);
-    tail_smooth<V, C>(M, l, M.nu2, t0, T);
-  }
-}
-
-// Threads per CTA: the pressure's coarsest solve sums the right-hand side's
-// mean over 1024 threads, as the one-block coarse kernel does (the same order,
-// the same bits); the viscous kernel has no block reduction and takes 512
-// threads, so that each may hold 128 registers.
-template <bool V>
-constexpr int kTailThreads = V ? 512 : 1024;
-
-template <bool V>
-__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads<V>)
-    k_tail(const BMember* __restrict__ tab, const int* __restrict__ list, int nlist,
-           const int* __restrict__ act) {
-  tail_run<V, kTailCtas>(tab, list, nlist, act);
-}
-
-// one CTA per member: many members side by side in one wave
-template <bool V>
-__global__ void __launch_bounds__(kTailThreads<V>) k_tail1(const BMember* __restrict__ tab,
-                                                           const int* __restrict__ list,
-                                                           int nlist, const int* __restrict__ act) {
-  tail_run<V, 1>(tab, list, nlist, act);
-}
-
 }  // namespace
 
 // ===========================================================================
@@ -2045,6 +1686,14 @@ void launch_coef_restrict(int D, const Geo& gf, const Geo& gc, const LevelPtrs<d
   else k_coef_restrict<2><<<gr, b, 0, s>>>(gf, gc, F, C, gamma);
 }
 
+void launch_idg64(int D, const Geo& g, const LevelPtrs<double>& L, double inv_re, cudaStream_t s) {
+  dim3 b = blk3(D);
+  dim3 gr = grd3(ext(g, 0, true), ext(g, 1, true), ext(g, 2, true), b);
+  const double ir = inv_re / (g.h * g.h);
+  if (D == 3) k_idg64<3><<<gr, b, 0, s>>>(g, L, ir);
+  else k_idg64<2><<<gr, b, 0, s>>>(g, L, ir);
+}
+
 void launch_adv_rhs(int D, const Geo& g, double* const uvel[3], double* const rho[3],
                     double* const frc[3], const LevelPtrs<double>& L0, double c_force,
                     int flow_axis, const double* G_dev, cudaStream_t s) {
@@ -2229,32 +1878,6 @@ void launch_b_tol_check(cudaGraphConditionalHandle h, const BMember* tab, int nm
 void launch_b_res_check(const BMember* tab, int nm, int sf, int sr, double slack,
                         cudaStream_t s) {
   if (nm > 0) kb_res_check<<<(nm + 255) / 256, 256, 0, s>>>(tab, nm, sf, sr, slack);
-}
-
-size_t tail_smem(const Geo& coarsest, bool viscous) { return b_coarse_smem(coarsest, viscous); }
-
-cudaError_t tail_set_smem() {
-  cudaError_t e = cudaSuccess;
-  for (const void* f : {(const void*)k_tail<true>, (const void*)k_tail<false>,
-                        (const void*)k_tail1<true>, (const void*)k_tail1<false>})
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kCoarseSmemMax);
-  return e;
-}
-
-void launch_tail(bool viscous, const BMember* tab, const int* list, int nlist, const int* act,
-                 size_t smem, cudaStream_t s, int ctas) {
-  if (nlist <= 0) return;
-  if (ctas == 1) {
-    if (viscous) k_tail1<true><<<nlist, kTailThreads<true>, smem, s>>>(tab, list, nlist, act);
-    else k_tail1<false><<<nlist, kTailThreads<false>, smem, s>>>(tab, list, nlist, act);
-  } else {
-    if (viscous)
-      k_tail<true><<<nlist * kTailCtas, kTailThreads<true>, smem, s>>>(tab, list, nlist, act);
-    else
-      k_tail<false><<<nlist * kTailCtas, kTailThreads<false>, smem, s>>>(tab, list, nlist, act);
-  }
 }
 
 }  // namespace bf
