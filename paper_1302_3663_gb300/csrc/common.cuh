@@ -310,6 +310,9 @@ void launch_p_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelP
 void launch_v_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelPtrs<double>& L,
                              float* const r32[3], float* const e32[3], double inv_re,
                              double* partial, cudaStream_t s, double* const r64[3] = nullptr);
+// L.ur = L.uf - A L.u in FP64 (3D, closed)
+void launch_v_residual_op(const Geo& g, const OpShape& S, const LevelPtrs<double>& L, double inv_re,
+                          cudaStream_t s);
 // Flexible CG around the FP32 V-cycle: z is the V-cycle's FP32 result;
 // w = A z in FP64 with partial z.q;
 // p = z + beta p, q = w + beta q with partials p.q, p.r (2 nb entries);

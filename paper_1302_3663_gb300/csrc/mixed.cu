@@ -319,6 +319,17 @@ void launch_v_residual_mixed(int D, const Geo& g, const OpShape& S, const LevelP
   else k_v_op2<false><<<grd3(g.n[0], g.n[1], 1, blk3(2)), blk3(2), 0, s>>>(g, a);
 }
 
+void launch_v_residual_op(const Geo& g, const OpShape& S, const LevelPtrs<double>& L, double inv_re,
+                          cudaStream_t s) {
+  VOpArgs a = v_op_args(g, L, inv_re, nullptr);
+  for (int d = 0; d < 3; ++d) {
+    a.u[d] = L.u[d];
+    a.q[d] = L.uf[d];
+    a.w[d] = L.ur[d];
+  }
+  launch_v_op(false, g, S, a, s);
+}
+
 // ------------------------------------------------------------ flexible CG
 // Flexible conjugate gradients for the viscous solve, in FP64 around the
 // FP32 V-cycle as preconditioner M (the viscous operator A is symmetric

@@ -109,8 +109,8 @@ __device__ __forceinline__ double op_u(const Geo& g, const T* __restrict__ u, co
 // mu_de ((u_d - u_d(-e)) + (u_e - u_e(-d))) on edges,
 //   V_d = 2 (t_d - t_d(-d)) + sum_e (s_de(+e) - s_de),   (A u)_d = m_d u_d - ir V_d.
 // FCG: u is the FP32 correction z; w = A z, partial sums of z.q.
-// else: r = f - A u to FP32 (and r64 when given), the FP32 correction zeroed,
-// partial sums of r^2.
+// else: r = f - A u to FP32 and the FP32 correction zeroed (when given), to w
+// (when given), partial sums of r^2.
 template <bool FCG>
 __device__ __forceinline__ void v_op_body(const Blk& B, const Geo& g, const OpShape& S,
                                           const VOpArgs& a) {
@@ -212,8 +212,10 @@ __device__ __forceinline__ void v_op_body(const Blk& B, const Geo& g, const OpSh
             acc = fma(up[d], qF[d], acc);
           } else {
             const double r = wall ? 0.0 : qF[d] - Au;
-            a.r32[d][F] = (float)r;
-            a.e32[d][F] = 0.f;
+            if (a.r32[d]) {
+              a.r32[d][F] = (float)r;
+              a.e32[d][F] = 0.f;
+            }
             if (a.w[d]) a.w[d][F] = r;
             acc = fma(r, r, acc);
           }

@@ -26,6 +26,7 @@ struct Level {
   Geo g;
   LevelPtrs<double> d;   // FP64 arrays
   LevelPtrs<float> f;    // FP32 arrays of the mixed-precision V-cycles
+  OpShape op{};          // FP64 contexts: the residual pass's blocks (nx 0: face by face)
 };
 
 int edge_count(int D) { return D == 3 ? 3 : 1; }
@@ -408,6 +409,13 @@ void vcycle_p(bfibm_ctx* c, int l) {
   smooth_p(c, l, c->P.nu2);
 }
 
+// the FP64 viscous residual of a level
+void residual_v(bfibm_ctx* c, int l) {
+  const Level& Lv = c->lev[l];
+  if (Lv.op.nx) launch_v_residual_op(Lv.g, Lv.op, Lv.d, c->P.inv_re, c->stream);
+  else launch_v_residual<double>(c->D, Lv.g, Lv.d, c->P.inv_re, c->stream);
+}
+
 void vcycle_v(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
@@ -417,7 +425,7 @@ void vcycle_v(bfibm_ctx* c, int l) {
     return;
   }
   smooth_v(c, l, c->P.nu1);
-  launch_v_residual<double>(c->D, Lv.g, Lv.d, c->P.inv_re, s);
+  residual_v(c, l);
   Level& Lc = c->lev[l + 1];
   restrict_faces(c, Lv.g, Lc.g, Lv.d.ur, Lc.d.uf, Lc.d.u);
   vcycle_v(c, l + 1);
@@ -649,7 +657,7 @@ bfibm_status solve_v(bfibm_ctx* c, int ncycles, int* used) {
   if (!tol) {
     for (int k = 0; k < ncycles; ++k) vcycle_v(c, 0);
     if (c->collect_stats) {
-      launch_v_residual<double>(c->D, L0.g, L0.d, c->P.inv_re, s);
+      residual_v(c, 0);
       launch_norm2(c->D, L0.g, L0.d.ur, c->D, c->sc, SL_VR, s);
     }
     *used = ncycles;
@@ -660,7 +668,7 @@ bfibm_status solve_v(bfibm_ctx* c, int ncycles, int* used) {
     c->loop_inner[0] = 1;
     bfibm_status cs = capture_while(c, 0, [&](cudaGraphConditionalHandle h) {
       vcycle_v(c, 0);
-      launch_v_residual<double>(c->D, L0.g, L0.d, c->P.inv_re, c->stream);
+      residual_v(c, 0);
       launch_norm2(c->D, L0.g, L0.d.ur, c->D, c->sc, SL_VR, c->stream);
       launch_tol_check(h, c->sc.out, SL_VF, SL_VR, c->P.rtol, c->P.max_cycles, c->dev_cycles,
                        c->loop_total, c->counters + 4, c->stream);
@@ -672,7 +680,7 @@ bfibm_status solve_v(bfibm_ctx* c, int ncycles, int* used) {
   int k = 0;
   for (k = 1; k <= c->P.max_cycles; ++k) {
     vcycle_v(c, 0);
-    launch_v_residual<double>(c->D, L0.g, L0.d, c->P.inv_re, s);
+    residual_v(c, 0);
     launch_norm2(c->D, L0.g, L0.d.ur, c->D, c->sc, SL_VR, s);
     bfibm_status rs = read_scalars(c);
     if (rs != BFIBM_OK) return rs;
@@ -2126,6 +2134,10 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
   c->L = build_levels(*p, geos);
   for (int l = 0; l < c->L; ++l) c->lev[l].g = geos[l];
   if (p->precision == 1 && c->D == 3) c->op = op_shape(c->lev[0].g);
+  if (p->precision == 0 && c->D == 3 && !p->open_flow)
+    for (int l = 0; l < c->L; ++l)   // smaller levels: a launch's latency hides the difference
+      if ((long long)c->lev[l].g.n[0] * c->lev[l].g.n[1] * c->lev[l].g.n[2] >= 1 << 15)
+        c->lev[l].op = op_shape(c->lev[l].g);
   if (stream) {
     c->stream = (cudaStream_t)stream;
   } else {

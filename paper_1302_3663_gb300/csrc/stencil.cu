@@ -145,20 +145,41 @@ __device__ __forceinline__ void p_terms(const Geo& g, const LevelPtrs<T>& L, con
   }
 }
 
-template <int D, typename T>
-__global__ void __launch_bounds__(256) k_p_rbgs(Geo g, LevelPtrs<T> L, int colour) {
-  int ih = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int k = blockIdx.z * blockDim.z + threadIdx.z;
-  if (j >= g.n[1] || k >= g.n[2]) return;
-  int i = 2 * ih + ((j + k + colour) & 1);
-  if (i >= g.n[0]) return;
-  int ci[3] = {i, j, k};
-  long long c = gidx(g, i, j, k);
-  T num, dg;
-  p_terms<D, T>(g, L, ci, c, num, dg);
-  T h2 = (T)(g.h * g.h);
-  L.p[c] = (num - h2 * L.pf[c]) / dg;
+// The colour kernels: one thread per point of the colour, a plane's rows
+// numbered without gaps along blockIdx.x (an FP64 instruction costs the same
+// for one lane as for 32, and a row seldom fills whole warps), planes along
+// blockIdx.y. nh: points per row, mnh = ceil(2^32 / nh).
+// INV: multiply by the inverse diagonal (L.idg, L.pdg) instead of forming the
+// diagonal and dividing. The sweeps are bound by the FP64 rate: about 20
+// operations per viscous point instead of 40, 8 instead of 26 for the pressure.
+// Three sweeps of both systems on a 101x75x130 grid: 1165 -> 669 us.
+// f(i, j, k) for the thread's points of e0 x e1 x e2 of one colour
+template <class F>
+__device__ __forceinline__ void colour_points(int nh, unsigned mnh, int e0, int e1, int e2,
+                                              int colour, F&& f) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  int j = nh == 1 ? q : (int)__umulhi((unsigned)q, mnh);
+  if (j * nh > q) --j;   // the high product exceeds the quotient by one at most
+  if (j >= e1) return;
+  const int ih = q - j * nh;
+  for (int k = blockIdx.y; k < e2; k += gridDim.y) {
+    const int i = 2 * ih + ((j + k + colour) & 1);
+    if (i < e0) f(i, j, k);
+  }
+}
+
+template <int D, typename T, bool INV>
+__global__ void __launch_bounds__(256) k_p_rbgs(Geo g, LevelPtrs<T> L, int colour, int nh,
+                                                unsigned mnh) {
+  const T h2 = (T)(g.h * g.h);
+  colour_points(nh, mnh, g.n[0], g.n[1], g.n[2], colour, [&](int i, int j, int k) {
+    const int ci[3] = {i, j, k};
+    const long long c = gidx(g, i, j, k);
+    T num, dg;
+    p_terms<D, T>(g, L, ci, c, num, dg);
+    if constexpr (INV) L.p[c] = pmul(pfma(-h2, L.pf[c], num), L.pdg[c]);
+    else L.p[c] = (num - h2 * L.pf[c]) / dg;
+  });
 }
 
 // ih2 = (T)(1 / h^2), formed once on the host
@@ -239,23 +260,21 @@ __device__ __forceinline__ void v_terms(const Geo& g, const LevelPtrs<T>& L, con
   v_terms_q<D, d, T>(g, L, ci, q, off, dgV);
 }
 
-template <int D, int d, typename T>
-__global__ void __launch_bounds__(256) k_v_rbgs(Geo g, LevelPtrs<T> L, int colour, T ir) {
-  int ih = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int k = blockIdx.z * blockDim.z + threadIdx.z;
+template <int D, int d, typename T, bool INV>
+__global__ void __launch_bounds__(256) k_v_rbgs(Geo g, LevelPtrs<T> L, int colour, T ir, int nh,
+                                                unsigned mnh) {
   // the faces of component d: along an open axis d the outflow face n too
   const int e0 = g.n[0] + (d == 0 && g.open == 0), e1 = g.n[1] + (d == 1 && g.open == 1),
             e2 = g.n[2] + (d == 2 && g.open == 2);
-  if (j >= e1 || k >= e2) return;
-  int i = 2 * ih + ((j + k + colour) & 1);
-  if (i >= e0) return;
-  int ci[3] = {i, j, k};
-  if (!g.per[d] && ci[d] == 0) return;   // wall face
-  long long F = gidx(g, i, j, k);
-  T off, dgV;
-  v_terms<D, d, T>(g, L, ci, F, off, dgV);
-  L.u[d][F] = (L.uf[d][F] + ir * off) / (L.m[d][F] + ir * dgV);
+  colour_points(nh, mnh, e0, e1, e2, colour, [&](int i, int j, int k) {
+    const int ci[3] = {i, j, k};
+    if (!g.per[d] && ci[d] == 0) return;   // wall face
+    const long long F = gidx(g, i, j, k);
+    T off, dgV;
+    v_terms<D, d, T>(g, L, ci, F, off, dgV);
+    if constexpr (INV) L.u[d][F] = pmul(pfma(ir, off, L.uf[d][F]), L.idg[d][F]);
+    else L.u[d][F] = (L.uf[d][F] + ir * off) / (L.m[d][F] + ir * dgV);
+  });
 }
 
 template <int D, int d, typename T>
@@ -1472,12 +1491,30 @@ __global__ void kb_res_check(const BMember* __restrict__ tab, int nm, int sf, in
 // ===========================================================================
 // launchers
 // ===========================================================================
+namespace {
+// the launch of a colour kernel over rows of e0 points, e1 rows, e2 planes
+struct ColourGrid {
+  dim3 grid, block;
+  int nh;
+  unsigned mnh;
+};
+ColourGrid colour_grid(int e0, int e1, int e2) {
+  ColourGrid c;
+  c.nh = (e0 + 1) / 2;
+  c.mnh = (unsigned)((0x100000000ull + (unsigned long long)c.nh - 1) / (unsigned long long)c.nh);
+  const long long np = (long long)c.nh * e1;
+  c.block = dim3((unsigned)(np < 256 ? (np + 31) / 32 * 32 : 256));
+  c.grid = dim3((unsigned)((np + c.block.x - 1) / c.block.x), (unsigned)(e2 < 65535 ? e2 : 65535));
+  return c;
+}
+}  // namespace
+
 template <typename T>
 void launch_p_rbgs(int D, const Geo& g, const LevelPtrs<T>& L, int colour, cudaStream_t s) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3((g.n[0] + 1) / 2, g.n[1], g.n[2], b);
-  if (D == 3) k_p_rbgs<3, T><<<gr, b, 0, s>>>(g, L, colour);
-  else k_p_rbgs<2, T><<<gr, b, 0, s>>>(g, L, colour);
+  const ColourGrid c = colour_grid(g.n[0], g.n[1], g.n[2]);
+  auto run = [&](auto k) { k<<<c.grid, c.block, 0, s>>>(g, L, colour, c.nh, c.mnh); };
+  if (D == 3) L.pdg ? run(k_p_rbgs<3, T, true>) : run(k_p_rbgs<3, T, false>);
+  else L.pdg ? run(k_p_rbgs<2, T, true>) : run(k_p_rbgs<2, T, false>);
 }
 
 template <typename T>
@@ -1492,16 +1529,17 @@ void launch_p_residual(int D, const Geo& g, const LevelPtrs<T>& L, cudaStream_t 
 template <typename T>
 void launch_v_rbgs(int D, const Geo& g, const LevelPtrs<T>& L, int d, int colour, double inv_re,
                    cudaStream_t s) {
-  dim3 b = blk3(D);
-  dim3 gr = grd3((ext(g, 0, d == 0) + 1) / 2, ext(g, 1, d == 1), ext(g, 2, d == 2), b);
-  T ir = (T)(inv_re / (g.h * g.h));
+  const ColourGrid c = colour_grid(ext(g, 0, d == 0), ext(g, 1, d == 1), ext(g, 2, d == 2));
+  const T ir = (T)(inv_re / (g.h * g.h));
+  auto run = [&](auto k) { k<<<c.grid, c.block, 0, s>>>(g, L, colour, ir, c.nh, c.mnh); };
+  const bool inv = L.idg[d] != nullptr;
   if (D == 3) {
-    if (d == 0) k_v_rbgs<3, 0, T><<<gr, b, 0, s>>>(g, L, colour, ir);
-    else if (d == 1) k_v_rbgs<3, 1, T><<<gr, b, 0, s>>>(g, L, colour, ir);
-    else k_v_rbgs<3, 2, T><<<gr, b, 0, s>>>(g, L, colour, ir);
+    if (d == 0) inv ? run(k_v_rbgs<3, 0, T, true>) : run(k_v_rbgs<3, 0, T, false>);
+    else if (d == 1) inv ? run(k_v_rbgs<3, 1, T, true>) : run(k_v_rbgs<3, 1, T, false>);
+    else inv ? run(k_v_rbgs<3, 2, T, true>) : run(k_v_rbgs<3, 2, T, false>);
   } else {
-    if (d == 0) k_v_rbgs<2, 0, T><<<gr, b, 0, s>>>(g, L, colour, ir);
-    else k_v_rbgs<2, 1, T><<<gr, b, 0, s>>>(g, L, colour, ir);
+    if (d == 0) inv ? run(k_v_rbgs<2, 0, T, true>) : run(k_v_rbgs<2, 0, T, false>);
+    else inv ? run(k_v_rbgs<2, 1, T, true>) : run(k_v_rbgs<2, 1, T, false>);
   }
 }
 

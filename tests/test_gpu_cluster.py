@@ -64,3 +64,18 @@ def test_coefficients_set_on_the_coarsest_level_are_used():
         return u
     assert np.array_equal(run(1.0), run(1.0))
     assert not np.array_equal(run(1.0), run(50.0))
+
+
+@pytest.mark.parametrize("n,per", GRIDS + [((66, 6, 4), (0, 0, 1)), ((6, 130), (0, 1))])
+def test_fp64_sweeps_with_inverse_diagonals(n, per):
+    # an FP64 context multiplies by stored inverse diagonals, a mixed-precision one (whose finest
+    # level stores none) divides: three sweeps of some 25 roundings each, diagonally dominant
+    out = []
+    for precision in (0, 1):
+        c = context(n, per, 8, precision=precision)
+        c.smooth_viscous(0, 3)
+        c.smooth_pressure(0, 3)
+        out.append([c.get_field("ut", d) for d in range(c.dim)] + [c.get_field("p")])
+        c.close()
+    for a, b in zip(*out):
+        assert np.abs(a - b).max() <= 1e-13 * np.abs(b).max()
