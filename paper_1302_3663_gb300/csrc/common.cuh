@@ -289,6 +289,7 @@ int ring_fill_kc(int D, int K, const Geo& g, int TY, int NP, int BX, int waves);
 // (red, black) pair of a row, TY rows per block plus two ring rows, KC planes
 // per chunk; same arithmetic as the one-pass sweep
 bool pair_eligible(int D, const Geo& g, int TY);
+int pair_threads(int n0, int TY);   // threads of its block
 void launch_v_rb_pair(const Geo& g, const LevelPtrs<float>& L, int d, float* out, double inv_re,
                       cudaStream_t s, int TY, int KC);
 // the pair sweep of the 3D FP32 pressure (same eligibility and shapes)
@@ -417,12 +418,13 @@ void launch_b_sweep(const BArgs& A, int K, int TY, int KC, int NP, int bx, size_
 const void* b_sweep_kernel(int K, int NP);
 size_t b_sweep_smem(int NP, int TY, int W);
 // the pair sweep of viscous component d over a work list of pair-eligible
-// members sharing the streaming axis' periodicity (perz); one block of
-// bx x (TY + 2) threads per item; smem: 4 (TY + 2) W floats, W the widest row
-void launch_b_pair(const BArgs& A, int d, bool perz, int TY, int KC, int bx, size_t smem,
+// members sharing the streaming axis' periodicity (perz); one block of `block`
+// threads (the widest row's pair_threads) per item; smem: 4 (TY + 2) W floats,
+// W the widest row
+void launch_b_pair(const BArgs& A, int d, bool perz, int TY, int KC, int block, size_t smem,
                    cudaStream_t s);
 // the same for the pressure
-void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int bx, size_t smem,
+void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int block, size_t smem,
                     cudaStream_t s);
 // after an odd count of sweeps: the current iterate of kind K copied back to
 // its own buffer (items: flat blocks over the level's elements)

@@ -427,8 +427,33 @@ __device__ __forceinline__ float psolve(const PSet& c, float ir, float up_d, flo
   return vx_final(c.uf, ir, off, c.idg);
 }
 
+// The pair of a thread: row r of the block's TY + 2 (0 and TY + 1: ring rows),
+// points x0 and x0 + 1. Rows of one parity lie side by side, first the even
+// ones, then (from a multiple of 32 threads) the odd ones, without gaps: the
+// red element of a pair depends on the row's parity, which is thus the same
+// in every lane of a warp, and rows of any length fill the warps. A warp per
+// 32 pairs of one row left a quarter of the lanes idle at 48, 96 and 144
+// points and room for 3 to 6 rows where 5 to 18 fit (finest viscous sweep of a
+// component, best of the tuner's shapes: 96x96x192 25.7 -> 22.1 us, 144x144x288
+// 98.9 (ring sweep) -> 60.3, 160x160x320 129.6 -> 87, 128x128x256 44.2 -> 43.6).
+struct PairLane {
+  int r, x0;
+  bool ok;
+};
+__device__ __forceinline__ PairLane pair_lane(int n0, int TY) {
+  const int np = n0 >> 1, nr = TY + 2, ne = (nr + 1) >> 1;
+  const int pad = (ne * np + 31) & ~31;
+  const int half = (int)threadIdx.x >= pad ? 1 : 0, q = threadIdx.x - (half ? pad : 0);
+  const int rr = q / np;
+  PairLane l;
+  l.r = 2 * rr + half;
+  l.x0 = 2 * (q - rr * np);
+  l.ok = l.r < nr;
+  return l;
+}
+
 template <int d, bool PERZ>
-__device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<float> L,
+__device__ __forceinline__ void v_rb_pair_body(const Blk& B, const Geo& g, const LevelPtrs<float>& L,
                                                float* __restrict__ out, int TY, int KC, float ir) {
   constexpr int e1 = d == 0 ? 1 : 0, e2 = d == 2 ? 1 : 2;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -436,20 +461,21 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int W = n0;                        // ring row pitch
   const int plane = (TY + 2) * W;
-  const int x0 = 2 * threadIdx.x, r = threadIdx.y;
+  const PairLane pl = pair_lane(n0, TY);
+  const int x0 = pl.x0, r = pl.r;
   const int j0 = B.x * TY;
   const int k0 = B.y * KC, k1 = min(k0 + KC, n2);
   const int j = j0 - 1 + r;
-  const bool lane_ok = x0 < n0;
+  const bool lane_ok = pl.ok;
   const bool rowvalid = lane_ok && j >= 0 && j < n1;
   const bool own = rowvalid && r >= 1 && r <= TY;
   const int st1 = (int)g.st[1], st2 = (int)g.st[2];
-  const int xl = x0 > 0 ? x0 - 1 : 0;     // left of the pair (clamped at the wall: zero weight)
+  const int dl = x0 > 0 ? -1 : 0;         // left of the pair (clamped at the wall: zero weight)
+  const int rb = r * W + x0;              // the pair in a ring plane
   // wall flags of the row and of the two x positions
   const bool wpy = j == n1 - 1, wmy = j == 0;
   const bool wmx0 = x0 == 0, wpx1 = x0 + 1 == n0 - 1;
-  for (int q = threadIdx.y * blockDim.x + threadIdx.x; q < 4 * plane; q += blockDim.x * blockDim.y)
-    ring[q] = 0.f;
+  for (int q = threadIdx.x; q < 4 * plane; q += blockDim.x) ring[q] = 0.f;
   const float* __restrict__ ud = L.u[d];
   const float* __restrict__ ua = L.u[e1];
   const float* __restrict__ ub = L.u[e2];
@@ -471,7 +497,7 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
     PRow q;
     const int o = oy + kz * st2;
     q.v = ldp(a, o);
-    q.l = left ? __ldg(a + o - x0 + xl) : 0.f;
+    q.l = left ? __ldg(a + o + dl) : 0.f;
     q.r = right ? __ldg(a + o + 2) : 0.f;
     return q;
   };
@@ -560,7 +586,7 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
       PRow UDx = UDc;
       const int ox = oy0 + kw * st2;
       if constexpr (PAR == 1) UDx.r = __ldg(ud + ox + 2);
-      else UDx.l = __ldg(ud + ox - x0 + xl);
+      else UDx.l = __ldg(ud + ox + dl);
       PSet c0, c1;
       if constexpr (d == 0) {
         // e1 = y: mu_xy at F, F + y; u_y at F, F + y (and x - 1)
@@ -619,14 +645,14 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
       np_[2] = pe<PAR>(UDp);
       nm_[2] = pe<PAR>(UDm);
       redv = psolve(PAR ? c1 : c0, ir, np_[d], nm_[d], np_[e1], nm_[e1], np_[e2], nm_[e2]);
-      const bool wall_red = (d == 0 && x0 + PAR == 0) || (d == 1 && j == 0) ||
+      const bool wall_red = (d == 0 && PAR == 0 && wmx0) || (d == 1 && wmy) ||
                             (d == 2 && !PERZ && kw == 0);
       if (wall_red) redv = 0.f;
       blk = PAR ? c0 : c1;
     }
     if (lane_ok) {
       const float2 rv = PAR ? make_float2(0.f, redv) : make_float2(redv, 0.f);
-      *reinterpret_cast<float2*>(ring + sk * plane + r * W + x0) = rv;
+      *reinterpret_cast<float2*>(ring + sk * plane + rb) = rv;
     }
     __syncthreads();
     // the black point (element PAR) of plane k - 1 on the block's own rows;
@@ -635,17 +661,16 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
     if (own && kb >= k0 && kb < k1) {
       const int kbw = pz(kb);
       const int s_m = (sk + 2) & 3, s_0 = (sk + 3) & 3;   // planes k - 2, k - 1 (k: sk)
-      const int xb = x0 + PAR;
-      const float* R0 = ring + s_0 * plane + r * W;
+      const float* R0 = ring + s_0 * plane + rb + PAR;
       float np_[3], nm_[3];
-      np_[0] = xb + 1 < n0 ? R0[xb + 1] : 0.f;
-      nm_[0] = xb > 0 ? R0[xb - 1] : 0.f;
-      np_[1] = R0[W + xb];
-      nm_[1] = R0[-W + xb];
-      np_[2] = ring[sk * plane + r * W + xb];
-      nm_[2] = ring[s_m * plane + r * W + xb];
+      np_[0] = PAR == 0 || !wpx1 ? R0[1] : 0.f;
+      nm_[0] = PAR == 1 || !wmx0 ? R0[-1] : 0.f;
+      np_[1] = R0[W];
+      nm_[1] = R0[-W];
+      np_[2] = ring[sk * plane + rb + PAR];
+      nm_[2] = ring[s_m * plane + rb + PAR];
       float bv = psolve(keep, ir, np_[d], nm_[d], np_[e1], nm_[e1], np_[e2], nm_[e2]);
-      const bool wall_blk = (d == 0 && xb == 0) || (d == 1 && j == 0) ||
+      const bool wall_blk = (d == 0 && PAR == 0 && wmx0) || (d == 1 && wmy) ||
                             (d == 2 && !PERZ && kbw == 0);
       if (wall_blk) bv = 0.f;
       const float2 o = PAR ? make_float2(red_prev, bv) : make_float2(bv, red_prev);
@@ -710,7 +735,8 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
 }
 
 template <int d, bool PERZ>
-__global__ void __launch_bounds__(512, 2) k_v_rb_pair(Geo g, LevelPtrs<float> L,
+__global__ void __launch_bounds__(512, 2) k_v_rb_pair(const __grid_constant__ Geo g,
+                                                   const __grid_constant__ LevelPtrs<float> L,
                                                    float* __restrict__ out, int TY, int KC,
                                                    float ir) {
   v_rb_pair_body<d, PERZ>(own_blk(), g, L, out, TY, KC, ir);
@@ -743,8 +769,8 @@ __global__ void __launch_bounds__(1024) kb_sweep(BArgs A, int TY, int KC) {
 
 // Batched pair sweep of viscous component d: block b does item b of the list
 // (one block per item, so no work-list loop adds registers to a kernel at its
-// limit); the block is as wide as the widest member's row needs, and the lanes
-// past a narrower member's row only take part in the barriers.
+// limit); the block is as large as the widest member's rows need, and the
+// threads a narrower member has no pairs for only take part in the barriers.
 template <int d, bool PERZ>
 __global__ void __launch_bounds__(512, 2) kb_pair(BArgs A, int TY, int KC) {
   const BItem it = A.items[blockIdx.x];
@@ -788,19 +814,20 @@ __device__ __forceinline__ void p_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const int W = n0;
   const int plane = (TY + 2) * W;
-  const int x0 = 2 * threadIdx.x, r = threadIdx.y;
+  const PairLane pl = pair_lane(n0, TY);
+  const int x0 = pl.x0, r = pl.r;
   const int j0 = B.x * TY;
   const int k0 = B.y * KC, k1 = min(k0 + KC, n2);
   const int j = j0 - 1 + r;
-  const bool lane_ok = x0 < n0;
+  const bool lane_ok = pl.ok;
   const bool rowvalid = lane_ok && j >= 0 && j < n1;
   const bool own = rowvalid && r >= 1 && r <= TY;
   const int st1 = (int)g.st[1], st2 = (int)g.st[2];
-  const int xl = x0 > 0 ? x0 - 1 : 0;
+  const int dl = x0 > 0 ? -1 : 0;
+  const int rb = r * W + x0;
   const bool wpy = j == n1 - 1, wmy = j == 0;
   const bool wmx0 = x0 == 0, wpx1 = x0 + 1 == n0 - 1;
-  for (int q = threadIdx.y * blockDim.x + threadIdx.x; q < 4 * plane; q += blockDim.x * blockDim.y)
-    ring[q] = 0.f;
+  for (int q = threadIdx.x; q < 4 * plane; q += blockDim.x) ring[q] = 0.f;
   const float* __restrict__ pp = L.p;
   const float* __restrict__ bx = L.beta[0];
   const float* __restrict__ by = L.beta[1];
@@ -851,7 +878,7 @@ __device__ __forceinline__ void p_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
       const int oz = kw * st2;
       // p of this row (queued) with the value left (red at x0 + 1) or right (red at x0)
       const float2 P0 = Pc;
-      const float Pl = PAR ? 0.f : __ldg(pp + oy0 + oz - x0 + xl);
+      const float Pl = PAR ? 0.f : __ldg(pp + oy0 + oz + dl);
       const float Pr = PAR ? __ldg(pp + oy0 + oz + 2) : 0.f;
       const float2 PYm = ldp(pp, oym + oz), PYp = ldp(pp, oyp + oz);
       const float2 BX = ldp(bx, oy0 + oz);
@@ -897,7 +924,7 @@ __device__ __forceinline__ void p_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
     }
     if (lane_ok) {
       const float2 rv = PAR ? make_float2(0.f, redv) : make_float2(redv, 0.f);
-      *reinterpret_cast<float2*>(ring + sk * plane + r * W + x0) = rv;
+      *reinterpret_cast<float2*>(ring + sk * plane + rb) = rv;
     }
     __syncthreads();
     // the black point (element PAR) of plane k - 1 on the block's own rows;
@@ -906,15 +933,14 @@ __device__ __forceinline__ void p_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
     if (own && kb >= k0 && kb < k1) {
       const int kbw = pz(kb);
       const int s_m = (sk + 2) & 3, s_0 = (sk + 3) & 3;
-      const int xb = x0 + PAR;
-      const float* R0 = ring + s_0 * plane + r * W;
+      const float* R0 = ring + s_0 * plane + rb + PAR;
       float nb[6];
-      nb[0] = xb > 0 ? R0[xb - 1] : 0.f;
-      nb[1] = xb + 1 < n0 ? R0[xb + 1] : 0.f;
-      nb[2] = R0[-W + xb];
-      nb[3] = R0[W + xb];
-      nb[4] = ring[s_m * plane + r * W + xb];
-      nb[5] = ring[sk * plane + r * W + xb];
+      nb[0] = PAR == 1 || !wmx0 ? R0[-1] : 0.f;
+      nb[1] = PAR == 0 || !wpx1 ? R0[1] : 0.f;
+      nb[2] = R0[-W];
+      nb[3] = R0[W];
+      nb[4] = ring[s_m * plane + rb + PAR];
+      nb[5] = ring[sk * plane + rb + PAR];
       const float bv = ppsolve(keep, h2, nb);
       const float2 o = PAR ? make_float2(red_prev, bv) : make_float2(bv, red_prev);
       *reinterpret_cast<float2*>(out + oy0 + kbw * st2) = o;
@@ -1046,13 +1072,17 @@ void launch_v_rb_fused(int D, const Geo& g, const LevelPtrs<T>& L, int d, T* out
   }
 }
 
-// Pair sweep: blocks of (pairs of a row rounded up to 32) x (TY + 2) threads
-// over (row tiles, plane chunks); 3D, walls in x and y, an even row of at
-// most 256 points.
+// Threads of a pair-sweep block on rows of n0 points (see pair_lane).
+int pair_threads(int n0, int TY) {
+  const int np = n0 / 2, nr = TY + 2, ne = (nr + 1) / 2;
+  return (ne * np + 31) / 32 * 32 + ((nr - ne) * np + 31) / 32 * 32;
+}
+
+// Pair sweep: blocks of at most 512 threads over (row tiles, plane chunks); 3D,
+// walls in x and y, an even row of at most 256 points.
 bool pair_eligible(int D, const Geo& g, int TY) {
   if (D != 3 || g.per[0] || g.per[1] || (g.n[0] & 1) || g.n[0] < 4 || g.n[0] > 256) return false;
-  const int bx = ((g.n[0] / 2 + 31) / 32) * 32;
-  return TY >= 1 && TY <= g.n[1] && bx * (TY + 2) <= 512;
+  return TY >= 1 && TY <= g.n[1] && pair_threads(g.n[0], TY) <= 512;
 }
 
 const void* pair_kernel(int d, bool perz) {
@@ -1067,9 +1097,8 @@ size_t pair_smem(const Geo& g, int TY) { return (size_t)4 * (TY + 2) * g.n[0] * 
 
 void launch_v_rb_pair(const Geo& g, const LevelPtrs<float>& L, int d, float* out, double inv_re,
                       cudaStream_t s, int TY, int KC) {
-  const int bx = ((g.n[0] / 2 + 31) / 32) * 32;
   if (KC < 1) KC = 1;
-  dim3 block(bx, TY + 2, 1);
+  const int block = pair_threads(g.n[0], TY);
   dim3 grid((g.n[1] + TY - 1) / TY, (g.n[2] + KC - 1) / KC, 1);
   const float ir = (float)(inv_re / (g.h * g.h));
   const size_t sm = pair_smem(g, TY);
@@ -1090,9 +1119,8 @@ const void* p_pair_kernel(bool perz) {
 
 void launch_p_rb_pair(const Geo& g, const LevelPtrs<float>& L, float* out, cudaStream_t s, int TY,
                       int KC) {
-  const int bx = ((g.n[0] / 2 + 31) / 32) * 32;
   if (KC < 1) KC = 1;
-  dim3 block(bx, TY + 2, 1);
+  const int block = pair_threads(g.n[0], TY);
   dim3 grid((g.n[1] + TY - 1) / TY, (g.n[2] + KC - 1) / KC, 1);
   const float h2 = (float)(g.h * g.h);
   const size_t sm = pair_smem(g, TY);
@@ -1100,10 +1128,9 @@ void launch_p_rb_pair(const Geo& g, const LevelPtrs<float>& L, float* out, cudaS
   else k_p_rb_pair<false><<<grid, block, sm, s>>>(g, L, out, TY, KC, h2);
 }
 
-void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int bx, size_t smem,
+void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int block, size_t smem,
                     cudaStream_t s) {
   if (A.n <= 0) return;
-  const dim3 block(bx, TY + 2, 1);
   if (perz) kb_ppair<true><<<A.n, block, smem, s>>>(A, TY, KC);
   else kb_ppair<false><<<A.n, block, smem, s>>>(A, TY, KC);
 }
@@ -1113,9 +1140,9 @@ void launch_b_ppair(const BArgs& A, bool perz, int TY, int KC, int bx, size_t sm
 int pair_fill_kc(const Geo& g, int d, int TY, int waves) {
   if (!pair_eligible(3, g, TY)) return 0;
   const void* fn = d == 3 ? p_pair_kernel(g.per[2] != 0) : pair_kernel(d, g.per[2] != 0);
-  const int bx = ((g.n[0] / 2 + 31) / 32) * 32;
   int bps = 0, dev = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, bx * (TY + 2), pair_smem(g, TY)) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, pair_threads(g.n[0], TY),
+                                                    pair_smem(g, TY)) !=
           cudaSuccess ||
       cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -1239,10 +1266,9 @@ void launch_b_sweep(const BArgs& A, int K, int TY, int KC, int NP, int bx, size_
   cudaLaunchKernel(b_sweep_kernel(K, NP == 2 ? 2 : 1), dim3(grid), block, args, smem, s);
 }
 
-void launch_b_pair(const BArgs& A, int d, bool perz, int TY, int KC, int bx, size_t smem,
+void launch_b_pair(const BArgs& A, int d, bool perz, int TY, int KC, int block, size_t smem,
                    cudaStream_t s) {
   if (A.n <= 0) return;
-  const dim3 block(bx, TY + 2, 1);
   if (perz) {
     if (d == 0) kb_pair<0, true><<<A.n, block, smem, s>>>(A, TY, KC);
     else if (d == 1) kb_pair<1, true><<<A.n, block, smem, s>>>(A, TY, KC);

@@ -718,7 +718,7 @@ cudaError_t tma_autotune(int D, const Geo& g, const LevelPtrs<float>& L, int K, 
   }
   // the pair sweep (viscous components and pressure): tile rows and chunk planes
   if (search && status == cudaSuccess) {
-    for (int pTY : {2, 4, 6, 8, 10, 14}) {
+    for (int pTY : {2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 18}) {
       if (!pair_eligible(D, g, pTY)) continue;
       int kcs_pair[5] = {8, 16, 32, pair_fill_kc(g, K, pTY, 1), pair_fill_kc(g, K, pTY, 2)};
       for (int ci = 0; ci < 5; ++ci) {

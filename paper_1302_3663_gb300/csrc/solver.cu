@@ -1338,6 +1338,7 @@ struct PShape {   // a batched sweep: rows, chunk planes, planes per phase, thre
   int all = 0;    // 1: one block per item; 0: the resident blocks stride over the items
   int kern = 0;   // 0 the ring sweep, 1 the pair sweep (viscous; one block per item)
   int perz = 0;   // the pair sweep: the streaming axis is periodic in every member
+  int threads = 0;   // the pair sweep: threads of a block
   size_t smem = 0;
   int grid = 0;
 };
@@ -1461,7 +1462,10 @@ cudaError_t sweep_list(Persist& P, int l, int K, PShape& sh, PList& L) {
     if (p_smooths(P, m, l))
       W = std::max(W, sh.kern ? P.mem[m]->lev[l].g.n[0] : P.mem[m]->lev[l].g.s[0]);
   sh.smem = sh.kern ? (size_t)4 * (sh.TY + 2) * W * sizeof(float) : b_sweep_smem(sh.NP, sh.TY, W);
-  if (sh.kern) sh.all = 1;
+  if (sh.kern) {
+    sh.all = 1;
+    sh.threads = pair_threads(W, sh.TY);
+  }
   std::vector<BItem> v;
   make_items(nm, [&](int m) { return p_smooths(P, m, l); },
              [&](int m) {
@@ -1512,10 +1516,10 @@ PShape default_shape(const Persist& P, int l) {
   long long KC = tiles / (3LL * device_sms());
   sh.KC = (int)std::max(4LL, std::min(16LL, KC));
   // the pair sweep where every member smoothing here can take it and the
-  // level holds at least 2^19 cells in all, in the shape the tuner picks on
-  // such levels of uneven ducts: six tile rows (fewer where the rows are
-  // wide), 16-plane chunks, one block per item
-  int bxu = 0, perz = -1;
+  // level holds at least 2^19 cells in all: as many tile rows as the block
+  // holds of the widest member's rows (at most 14), 16-plane chunks, one block
+  // per item
+  int bxu = 0, wid = 2, perz = -1;
   long long cells = 0;
   bool pair_ok = true;
   for (size_t m = 0; pair_ok && m < P.mem.size(); ++m) {
@@ -1525,9 +1529,11 @@ PShape default_shape(const Persist& P, int l) {
               (perz < 0 || perz == g.per[2]);
     perz = g.per[2];
     bxu = std::max(bxu, (g.n[0] / 2 + 31) / 32 * 32);
+    wid = std::max(wid, g.n[0]);
     cells += (long long)g.n[0] * g.n[1] * g.n[2];
   }
-  const int pTY = std::min({6, bxu > 0 ? 512 / bxu - 2 : 0, nR});
+  int pTY = std::min(14, nR);
+  while (pTY >= 1 && pair_threads(wid, pTY) > 512) --pTY;
   if (pair_ok && perz >= 0 && cells >= (1LL << 19) && pTY >= 1) {
     sh.kern = 1;
     sh.perz = perz;
@@ -1601,7 +1607,7 @@ cudaError_t tune_level(Persist& P, int l, int K) {
         }
   // the pair sweep (viscous): where every member smoothing on the level can
   // take it, with one block width (the widest row's) for all
-  int bxu = 0, n1min = 1 << 30, perz = -1;
+  int bxu = 0, wid = 2, n1min = 1 << 30, perz = -1;
   bool pair_ok = st == cudaSuccess;
   for (size_t m = 0; pair_ok && m < P.mem.size(); ++m) {
     if (!p_smooths(P, (int)m, l)) continue;
@@ -1610,12 +1616,13 @@ cudaError_t tune_level(Persist& P, int l, int K) {
               (perz < 0 || perz == g.per[2]);
     perz = g.per[2];
     bxu = std::max(bxu, (g.n[0] / 2 + 31) / 32 * 32);
+    wid = std::max(wid, g.n[0]);
     n1min = std::min(n1min, g.n[1]);
   }
   if (pair_ok && perz >= 0)
-    for (int TY : {2, 4, 6, 8, 10, 14})
+    for (int TY : {2, 3, 4, 5, 6, 8, 10, 14, 18})
       for (int KC : {4, 8, 16, 32}) {
-        if (TY > n1min || bxu * (TY + 2) > 512) continue;
+        if (TY > n1min || pair_threads(wid, TY) > 512) continue;
         PShape sh = best;
         sh.kern = 1;
         sh.perz = perz;
@@ -1631,8 +1638,9 @@ cudaError_t tune_level(Persist& P, int l, int K) {
         for (int round = 0; round < 3 && st == cudaSuccess; ++round) {
           cudaEventRecord(e0, P.stream);
           for (int r = 0; r < 3; ++r) {
-            if (K == 3) launch_b_ppair(A, sh.perz != 0, sh.TY, sh.KC, sh.bx, sh.smem, P.stream);
-            else launch_b_pair(A, K, sh.perz != 0, sh.TY, sh.KC, sh.bx, sh.smem, P.stream);
+            if (K == 3) launch_b_ppair(A, sh.perz != 0, sh.TY, sh.KC, sh.threads, sh.smem,
+                                       P.stream);
+            else launch_b_pair(A, K, sh.perz != 0, sh.TY, sh.KC, sh.threads, sh.smem, P.stream);
           }
           cudaEventRecord(e1, P.stream);
           st = cudaEventSynchronize(e1);
@@ -1857,8 +1865,8 @@ void b_smooth(Persist& P, int l, int n, bool V) {
       for (int d = 0; d < 3; ++d) {
         const PShape& sh = P.shv[l];
         if (sh.kern)
-          launch_b_pair(bargs(P, P.swv[l], l, cur), d, sh.perz != 0, sh.TY, sh.KC, sh.bx, sh.smem,
-                        P.stream);
+          launch_b_pair(bargs(P, P.swv[l], l, cur), d, sh.perz != 0, sh.TY, sh.KC, sh.threads,
+                        sh.smem, P.stream);
         else
           launch_b_sweep(bargs(P, P.swv[l], l, cur), d, sh.TY, sh.KC, sh.NP, sh.bx, sh.smem,
                          sh.grid, P.stream);
@@ -1867,7 +1875,7 @@ void b_smooth(Persist& P, int l, int n, bool V) {
     } else {
       const PShape& sh = P.shp[l];
       if (sh.kern)
-        launch_b_ppair(bargs(P, P.swp[l], l, cur), sh.perz != 0, sh.TY, sh.KC, sh.bx, sh.smem,
+        launch_b_ppair(bargs(P, P.swp[l], l, cur), sh.perz != 0, sh.TY, sh.KC, sh.threads, sh.smem,
                        P.stream);
       else
         launch_b_sweep(bargs(P, P.swp[l], l, cur), 3, sh.TY, sh.KC, sh.NP, sh.bx, sh.smem,
@@ -3161,13 +3169,14 @@ bfibm_status bfibm_batch_set_sweep_shape(bfibm_batch* b, int level, int kind,
     return BFIBM_EINVAL;
   }
   if (sh.kern) {   // the pair sweep: every member eligible, one row width
-    bool ok = sh.NP == 1 && sh.bx * (sh.TY + 2) <= 512;
+    bool ok = sh.NP == 1;
     int perz = -1;
     for (size_t m = 0; ok && m < P.mem.size(); ++m) {
       if (!p_smooths(P, (int)m, level)) continue;
       const Geo& g = P.mem[m]->lev[level].g;
       ok = !g.per[0] && !g.per[1] && !(g.n[0] & 1) && g.n[0] >= 4 && g.n[0] <= 256 &&
-           sh.TY <= g.n[1] && (g.n[0] / 2 + 31) / 32 * 32 <= sh.bx && (perz < 0 || perz == g.per[2]);
+           sh.TY <= g.n[1] && (g.n[0] / 2 + 31) / 32 * 32 <= sh.bx &&
+           pair_threads(g.n[0], sh.TY) <= 512 && (perz < 0 || perz == g.per[2]);
       perz = g.per[2];
     }
     if (!ok) {
