@@ -53,6 +53,25 @@ struct Ptr3d {
   double* a[3];
 };
 
+// FP32 to FP64 on the integer pipes, for passes bound by the FP64 rate: the
+// conversion instruction would take a slot of the FP64 pipe. Exact.
+__device__ __forceinline__ double wide64(float f) {
+  const unsigned b = __float_as_uint(f), e = (b >> 23) & 255u;
+  if (e - 1u >= 254u && (b << 1) != 0u) return (double)f;   // subnormal, infinity or NaN
+  const unsigned m = ((b & 0x7fffffffu) >> 3) + (896u << 20);
+  return __hiloint2double((int)((b & 0x80000000u) | ((b << 1) ? m : 0u)), (int)(b << 29));
+}
+
+// FP64 to FP32, rounded to nearest even, on the integer pipes as well.
+__device__ __forceinline__ float narrow32(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 2047u;
+  if (e - 897u >= 253u) return (float)v;   // outside FP32's normal range, its last binade, NaN
+  const unsigned long long a =
+      (b & 0x7fffffffffffffffull) + 0x0fffffffull + ((b >> 29) & 1ull);
+  return __uint_as_float((hi & 0x80000000u) | ((unsigned)(a >> 29) - (896u << 23)));
+}
+
 // The FP64 operator passes of the mixed-precision solves (op64.cu): the tile
 // of columns of a block, the planes of a chunk and their counts.
 constexpr int kOpThreads = 512;
@@ -486,7 +505,7 @@ bool tma_plan_of(int K, const Geo& g, int out[5]);
 // L.idg and L.pdg from the level's coefficients
 void launch_idg64(int D, const Geo& g, const LevelPtrs<double>& L, double inv_re, cudaStream_t s);
 void launch_coef_fine(int D, const Geo& g, double* const rho[3], double* beta[3], double* m[3],
-                      double msc, cudaStream_t s);
+                      double msc, double rho_f, cudaStream_t s);
 void launch_coef_restrict(int D, const Geo& gf, const Geo& gc, const LevelPtrs<double>& F,
                           const LevelPtrs<double>& C, double gamma, cudaStream_t s);
 void launch_adv_rhs(int D, const Geo& g, double* const uvel[3], double* const rho[3],
@@ -548,7 +567,8 @@ struct NodeSet {
   double* F;    // eta x 3
   int* tile;    // eta: tile of each node
   int* perm;    // eta: nodes sorted by tile
-  int* count;   // ntiles + 1
+  int* count;   // ntiles + 1 (the last: occupied tiles)
+  int* active;  // ntiles: the occupied tiles, in no particular order
   int* start;   // ntiles + 1
   int* cursor;  // ntiles
   int* clamped; // 1 counter

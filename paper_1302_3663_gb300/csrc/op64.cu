@@ -44,15 +44,9 @@ __device__ __forceinline__ unsigned long long op_umax(unsigned long long a, unsi
   return a > b ? a : b;
 }
 
-// FP32 to FP64 and a sign flip on the integer pipes, which are idle here: the
-// conversion instruction would take a slot of the FP64 pipe.
-__device__ __forceinline__ double op_wide(float f) {
-  const unsigned b = __float_as_uint(f), e = (b >> 23) & 255u;
-  if (e - 1u >= 254u && (b << 1) != 0u) return (double)f;   // subnormal, infinity or NaN
-  const unsigned m = ((b & 0x7fffffffu) >> 3) + (896u << 20);
-  return __hiloint2double((int)((b & 0x80000000u) | ((b << 1) ? m : 0u)), (int)(b << 29));
-}
+__device__ __forceinline__ double op_wide(float f) { return wide64(f); }
 __device__ __forceinline__ double op_wide(double f) { return f; }
+// a sign flip on the integer pipe
 __device__ __forceinline__ double op_neg_if(double v, bool neg) {
   return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000u : 0), __double2loint(v));
 }
@@ -213,7 +207,7 @@ __device__ __forceinline__ void v_op_body(const Blk& B, const Geo& g, const OpSh
           } else {
             const double r = wall ? 0.0 : qF[d] - Au;
             if (a.r32[d]) {
-              a.r32[d][F] = (float)r;
+              a.r32[d][F] = narrow32(r);
               a.e32[d][F] = 0.f;
             }
             if (a.w[d]) a.w[d][F] = r;
@@ -292,7 +286,7 @@ __device__ __forceinline__ void p_op_body(const Blk& B, const Geo& g, const OpSh
     if (q.own) {
       if (k > k0) {
         const double r = fma(-a.ih2, part + (fz - fzp), f);
-        a.r32[F] = (float)r;
+        a.r32[F] = narrow32(r);
         a.e32[F] = 0.f;
         acc = fma(r, r, acc);
         mx = op_umax(mx, (unsigned long long)__double_as_longlong(r) & 0x7fffffffffffffffull);

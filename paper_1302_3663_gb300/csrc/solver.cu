@@ -1048,7 +1048,8 @@ void inverse_diagonals(bfibm_ctx* c, int l) {
 
 void build_coefficients(bfibm_ctx* c) {
   Level& L0 = c->lev[0];
-  launch_coef_fine(c->D, L0.g, c->rho, L0.d.beta, L0.d.m, c->P.sigma / c->P.dt, c->stream);
+  launch_coef_fine(c->D, L0.g, c->rho, L0.d.beta, L0.d.m, c->P.sigma / c->P.dt, c->P.rho_f,
+                   c->stream);
   for (int l = 1; l < c->L; ++l) {
     // Eq. (ViscCoarseGrid): gamma_lh may differ per coarse grid
     const double gam = (l < 8 && c->P.gamma_levels[l] > 0.0) ? c->P.gamma_levels[l]
@@ -1284,7 +1285,7 @@ bfibm_status copy_field(bfibm_ctx* c, int which, int comp, int level, void* ext,
 void free_lag(bfibm_ctx* c, bool nodes, bool springs) {
   if (nodes) {
     for (void* q : {(void*)c->N.X, (void*)c->N.U, (void*)c->N.F, (void*)c->N.tile, (void*)c->N.perm,
-                    (void*)c->N.count, (void*)c->N.start, (void*)c->N.cursor, (void*)c->N.tw,
+                    (void*)c->N.count, (void*)c->N.active, (void*)c->N.start, (void*)c->N.cursor, (void*)c->N.tw,
                     (void*)c->N.tlo})
       if (q) cudaFree(q);
     long long keep_eta = 0;
@@ -2402,7 +2403,7 @@ bfibm_status bfibm_set_nodes(bfibm_ctx* c, int64_t eta, const double* X) {
   int nt = c->tg.ntiles;
   long long e3 = 3 * std::max<long long>(eta, 1);
   if (dmalloc(&N.X, e3) || dmalloc(&N.U, e3) || dmalloc(&N.F, e3) ||
-      dmalloc(&N.tile, eta) || dmalloc(&N.perm, eta) || dmalloc(&N.count, nt + 1) ||
+      dmalloc(&N.tile, eta) || dmalloc(&N.perm, eta) || dmalloc(&N.count, nt + 1) || dmalloc(&N.active, nt) ||
       dmalloc(&N.start, nt + 1) || dmalloc(&N.cursor, nt + 1) || dmalloc(&N.tw, 48 * (e3 / 3)) ||
       dmalloc(&N.tlo, 24 * (e3 / 3))) {
     cudaGetLastError();

@@ -782,8 +782,11 @@ struct Ptr3 {
   double* a[3];
 };
 
+// (rho_f, inv_rho: the fluid's density and its reciprocal. Most faces hold the
+// plain fluid, and three FP64 divisions per point took 213 us on the
+// 128x128x256 duct, four times the pass's memory traffic.)
 __global__ void __launch_bounds__(256) k_coef_fine(Geo g, int D, Ptr3 rho, Ptr3 beta, Ptr3 m,
-                                                   double msc) {
+                                                   double msc, double rho_f, double inv_rho) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z * blockDim.z + threadIdx.z;
@@ -791,7 +794,10 @@ __global__ void __launch_bounds__(256) k_coef_fine(Geo g, int D, Ptr3 rho, Ptr3 
   long long c = gidx(g, i, j, k);
   for (int d = 0; d < D; ++d) {
     double r = rho.a[d][c];
-    beta.a[d][c] = r != 0.0 ? 1.0 / r : 0.0;
+    const bool plain = __double_as_longlong(r) == __double_as_longlong(rho_f);
+    double b = inv_rho;
+    if (!plain) b = r != 0.0 ? 1.0 / r : 0.0;
+    beta.a[d][c] = b;
     m.a[d][c] = r * msc;
   }
 }
@@ -940,7 +946,7 @@ __device__ __forceinline__ void adv_rhs_point(const Geo& g, const Ptr3& uv, cons
 template <int D>
 __global__ void __launch_bounds__(256) k_adv_rhs(Geo g, Ptr3 uv, Ptr3 rho, Ptr3 frc,
                                                  LevelPtrs<double> L0, double c_force, int flow,
-                                                 const double* __restrict__ G_dev) {
+                                                 const double* __restrict__ G_dev, double c4) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int j = blockIdx.y * blockDim.y + threadIdx.y;
   int k = blockIdx.z * blockDim.z + threadIdx.z;
@@ -949,7 +955,6 @@ __global__ void __launch_bounds__(256) k_adv_rhs(Geo g, Ptr3 uv, Ptr3 rho, Ptr3 
   int ci[3] = {i, j, k};
   long long F = gidx(g, i, j, k);
   double G = *G_dev;
-  const double c4 = 0.25 / g.h;
   adv_rhs_point<D, 0>(g, uv, rho, frc, L0, ci, F, c_force, flow == 0 ? G : 0.0, c4);
   adv_rhs_point<D, 1>(g, uv, rho, frc, L0, ci, F, c_force, flow == 1 ? G : 0.0, c4);
   if constexpr (D == 3)
@@ -959,12 +964,21 @@ __global__ void __launch_bounds__(256) k_adv_rhs(Geo g, Ptr3 uv, Ptr3 rho, Ptr3 
 // ---------------------------------------------------------------------------
 // Divergence, projection and reductions.
 // ---------------------------------------------------------------------------
+// a / h from the correctly rounded ih = 1 / h and one correction of the quotient
+// by its exact remainder: the rounding of a division in 3 FP64 operations
+// instead of about 10 (GB300's FP64 rate bounds these passes).
+__device__ __forceinline__ double over_h(double a, double h, double ih) {
+  const double q = a * ih;
+  if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;   // infinite or NaN: as it is
+  return fma(fma(-q, h, a), ih, q);
+}
+
 template <int D>
 __device__ __forceinline__ double div_at(const Geo& g, const Ptr3& u, const int ci[3],
-                                         long long c) {
+                                         long long c, double ih) {
   double s = 0.0;
 #pragma unroll
-  for (int a = 0; a < D; ++a) s += (u.a[a][c + offp(g, a, ci[a])] - u.a[a][c]) / g.h;
+  for (int a = 0; a < D; ++a) s += over_h(u.a[a][c + offp(g, a, ci[a])] - u.a[a][c], g.h, ih);
   return s;
 }
 
@@ -974,6 +988,7 @@ __global__ void __launch_bounds__(256) k_divergence(Geo g, Ptr3 u, double* __res
                                                     const double* __restrict__ beta_open,
                                                     double pbc) {
   __shared__ double sh[32];
+  const double ih = 1.0 / g.h;
   long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
   double acc = 0.0;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ncell;
@@ -981,7 +996,7 @@ __global__ void __launch_bounds__(256) k_divergence(Geo g, Ptr3 u, double* __res
     int ci[3];
     decode(g, q, ci[0], ci[1], ci[2]);
     long long c = gidx(g, ci[0], ci[1], ci[2]);
-    double v = scale * div_at<D>(g, u, ci, c);
+    double v = scale * div_at<D>(g, u, ci, c, ih);
     // the held outflow pressure: b -= 2 beta_out p_out / h^2 (pbc = 2 p_out / h^2)
     if (last_open_cell(g, ci)) v -= beta_open[c + st_of(g, g.open)] * pbc;
     b[c] = v;
@@ -1046,8 +1061,8 @@ __global__ void __launch_bounds__(256) k_sub_scalar(Geo g, double* __restrict__ 
 // below the face along d. One function for the face a thread owns and for
 // the upper faces it recomputes, so both round alike.
 __device__ __forceinline__ double proj_face(double ut, double beta, double pF, double pM,
-                                            double coef, double h) {
-  return ut - coef * beta * ((pF - pM) / h);
+                                            double coef, double h, double ih) {
+  return ut - coef * beta * over_h(pF - pM, h, ih);
 }
 
 // Projection, Eq. (NSdis2), with the check of Eq. (NSdis4) fused in: each
@@ -1060,7 +1075,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* __restrict__ p,
                                                  Ptr3 beta, Ptr3 uv, double coef,
                                                  unsigned long long* __restrict__ divacc,
-                                                 double p_out) {
+                                                 double p_out, double ih) {
   __shared__ double sh[32];
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1078,7 +1093,7 @@ __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* _
       if (beyond) {
         long long F = gidx(g, i, j, k);
         const double pm = p[F - g.st[o]];
-        uv.a[o][F] = proj_face(ut.a[o][F], beta.a[o][F], 2.0 * p_out - pm, pm, coef, g.h);
+        uv.a[o][F] = proj_face(ut.a[o][F], beta.a[o][F], 2.0 * p_out - pm, pm, coef, g.h, ih);
       }
     }
   }
@@ -1095,18 +1110,18 @@ __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* _
         lo = ut.a[d][F];
         uv.a[d][F] = lo;
       } else {
-        lo = proj_face(ut.a[d][F], beta.a[d][F], pF, p[F + offm(g, d, ci[d])], coef, g.h);
+        lo = proj_face(ut.a[d][F], beta.a[d][F], pF, p[F + offm(g, d, ci[d])], coef, g.h, ih);
         uv.a[d][F] = lo;
       }
       double hi = 0.0;   // the upper wall face holds 0
       if (g.per[d] || ci[d] != g.n[d] - 1) {
         long long Fu = F + offp(g, d, ci[d]);
-        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], p[Fu], pF, coef, g.h);
+        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], p[Fu], pF, coef, g.h, ih);
       } else if (is_open(g, d)) {   // the outflow face: ghost 2 p_out - p
         long long Fu = F + st_of(g, d);
-        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], 2.0 * p_out - pF, pF, coef, g.h);
+        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], 2.0 * p_out - pF, pF, coef, g.h, ih);
       }
-      s += (hi - lo) / g.h;
+      s += over_h(hi - lo, g.h, ih);
     }
     mx = fabs(s);
     if (!(mx <= CUDART_INF)) mx = CUDART_INF;
@@ -1180,6 +1195,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_div_ke(Geo g, Ptr3 u, double* __restrict__ pmax,
                                                 double* __restrict__ psum) {
   __shared__ double sh[32];
+  const double ih = 1.0 / g.h;
   long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
   double mx = 0.0, acc = 0.0;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ncell;
@@ -1187,7 +1203,7 @@ __global__ void __launch_bounds__(256) k_div_ke(Geo g, Ptr3 u, double* __restric
     int ci[3];
     decode(g, q, ci[0], ci[1], ci[2]);
     long long c = gidx(g, ci[0], ci[1], ci[2]);
-    mx = fmax(mx, fabs(div_at<D>(g, u, ci, c)));
+    mx = fmax(mx, fabs(div_at<D>(g, u, ci, c, ih)));
     for (int d = 0; d < D; ++d) {
       if (d == g.open && ci[d] == g.n[d] - 1) {   // the outflow face
         double v = u.a[d][c + g.st[d]];
@@ -1710,10 +1726,10 @@ static Ptr3 ptr3(double* const a[3]) {
 }
 
 void launch_coef_fine(int D, const Geo& g, double* const rho[3], double* beta[3], double* m[3],
-                      double msc, cudaStream_t s) {
+                      double msc, double rho_f, cudaStream_t s) {
   dim3 b = blk3(D);
   dim3 gr = grd3(g.s[0], g.s[1], g.s[2], b);
-  k_coef_fine<<<gr, b, 0, s>>>(g, D, ptr3(rho), ptr3(beta), ptr3(m), msc);
+  k_coef_fine<<<gr, b, 0, s>>>(g, D, ptr3(rho), ptr3(beta), ptr3(m), msc, rho_f, 1.0 / rho_f);
 }
 
 void launch_coef_restrict(int D, const Geo& gf, const Geo& gc, const LevelPtrs<double>& F,
@@ -1738,9 +1754,11 @@ void launch_adv_rhs(int D, const Geo& g, double* const uvel[3], double* const rh
   dim3 b = blk3(D);
   dim3 gr = grd3(ext(g, 0, true), ext(g, 1, true), ext(g, 2, true), b);
   if (D == 3)
-    k_adv_rhs<3><<<gr, b, 0, s>>>(g, ptr3(uvel), ptr3(rho), ptr3(frc), L0, c_force, flow_axis, G_dev);
+    k_adv_rhs<3><<<gr, b, 0, s>>>(g, ptr3(uvel), ptr3(rho), ptr3(frc), L0, c_force, flow_axis, G_dev,
+                                 0.25 / g.h);
   else
-    k_adv_rhs<2><<<gr, b, 0, s>>>(g, ptr3(uvel), ptr3(rho), ptr3(frc), L0, c_force, flow_axis, G_dev);
+    k_adv_rhs<2><<<gr, b, 0, s>>>(g, ptr3(uvel), ptr3(rho), ptr3(frc), L0, c_force, flow_axis, G_dev,
+                                 0.25 / g.h);
 }
 
 void launch_divergence(int D, const Geo& g, double* const u[3], double* b, double scale,
@@ -1772,9 +1790,9 @@ void launch_project(int D, const Geo& g, double* const ut[3], const double* p,
   dim3 gr = grd3(ext(g, 0, true), ext(g, 1, true), ext(g, 2, true), b);
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(dc.out + dc.acc);
   if (D == 3)
-    k_project<3><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out);
+    k_project<3><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, 1.0 / g.h);
   else
-    k_project<2><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out);
+    k_project<2><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, 1.0 / g.h);
   k_div_check<<<1, 32, 0, s>>>(dc.out, dc.acc, dc.step, dc.all, dc.tol, dc.viol);
 }
 
