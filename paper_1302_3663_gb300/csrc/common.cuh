@@ -427,6 +427,9 @@ void launch_b_fcg_update(const BArgs& A, int sl_pq, int sl_pr, int grid, cudaStr
 // nx x ny x nz points, the flat conversions over n elements
 int red_grid_of(long long n);
 dim3 stencil_grid3(long long nx, long long ny, long long nz);
+dim3 v_residual_grid(const Geo& g);   // FP32, 3D
+dim3 p_residual_grid(const Geo& g);
+dim3 prolong_grid(const Geo& gf, size_t elem);     // 3D, closed
 int flat_convert_blocks(long long n);
 // smooth.cu: one ring sweep of viscous component K (0..2) or the pressure
 // (K = 3) on level A.lev of every listed member, out of place (the output

@@ -1358,7 +1358,7 @@ struct Persist {
   // per level l: the members that smooth on l (l below their coarsest level)
   PList swv[kMaxLevels], swp[kMaxLevels];   // ring-sweep blocks (viscous, pressure shape)
   PShape shv[kMaxLevels], shp[kMaxLevels];
-  PList en[kMaxLevels];   // 3D blocks over the cells of l: residuals, prolongations
+  PList pl[kMaxLevels], rv[kMaxLevels], rp[kMaxLevels];   // prolongations to l; residuals on l
   PList rs[kMaxLevels];   // over the stored faces of l + 1: face restriction
   PList rn[kMaxLevels];   // over the cells of l + 1: cell restriction
   PList fl[kMaxLevels];   // flat blocks over the elements of l: copies after odd sweep counts
@@ -1748,11 +1748,12 @@ bfibm_status persist_build(Persist& P, bool tune) {
   auto tail_of = [&](int m) { return P.ptail[m]; };
   for (int l = 0; l < P.depth; ++l) {
     auto smooths = [&](int m) { return l < std::min(tail_of(m), P.mem[m]->L - 1); };
-    ok &= make_items(nm, smooths, [&](int m) {
-      const Geo& g = lev(m, l);
-      return stencil_grid3(g.n[0], g.n[1], g.n[2]);
-    }, v);
-    PK(upload(P, v, P.en[l]));
+    ok &= make_items(nm, smooths, [&](int m) { return prolong_grid(lev(m, l), sizeof(float)); }, v);
+    PK(upload(P, v, P.pl[l]));
+    ok &= make_items(nm, smooths, [&](int m) { return v_residual_grid(lev(m, l)); }, v);
+    PK(upload(P, v, P.rv[l]));
+    ok &= make_items(nm, smooths, [&](int m) { return p_residual_grid(lev(m, l)); }, v);
+    PK(upload(P, v, P.rp[l]));
     ok &= make_items(nm, smooths, [&](int m) {
       const Geo& g = lev(m, l + 1);
       return stencil_grid3(g.s[0], g.s[1], g.s[2]);
@@ -1911,20 +1912,20 @@ void b_level(Persist& P, int l, bool V) {
   if (P.co[l].n) launch_b_coarse(bargs(P, P.co[l], l), V, P.co_smem[l][V ? 1 : 0], s);
   launch_cluster(3, false, V, P.per, P.tab, P.cco[l], P.ncco[l], P.masked ? P.act : nullptr, true, P.C,
                  P.tail_smem[l][V ? 1 : 0], s);
-  if (!P.en[l].n) return;
+  if (!P.pl[l].n) return;
   b_smooth(P, l, P.nu1, V);
   if (V) {
-    launch_b_v_residual32(bargs(P, P.en[l], l), P.en[l].grid, s);
+    launch_b_v_residual32(bargs(P, P.rv[l], l), P.rv[l].grid, s);
     launch_b_restrict_face32(bargs(P, P.rs[l], l), P.rs[l].grid, s);
   } else {
-    launch_b_p_residual32(bargs(P, P.en[l], l), P.en[l].grid, s);
+    launch_b_p_residual32(bargs(P, P.rp[l], l), P.rp[l].grid, s);
     launch_b_restrict_cell32(bargs(P, P.rn[l], l), P.rn[l].grid, s);
   }
   b_vcycle(P, l + 1, V);
   if (V)
-    launch_b_prolong_face32(bargs(P, P.en[l], l), P.en[l].grid, s);
+    launch_b_prolong_face32(bargs(P, P.pl[l], l), P.pl[l].grid, s);
   else
-    launch_b_prolong_cell32(bargs(P, P.en[l], l), P.en[l].grid, s);
+    launch_b_prolong_cell32(bargs(P, P.pl[l], l), P.pl[l].grid, s);
   b_smooth(P, l, P.nu2, V);
 }
 

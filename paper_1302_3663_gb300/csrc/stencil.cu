@@ -323,6 +323,213 @@ __device__ __forceinline__ void v_residual_body(const Blk& B, Geo g, LevelPtrs<T
   if constexpr (D == 3) v_residual_point<D, 2, T>(g, L, ci, q, ir);
 }
 
+// The FP32 residuals in 3D (closed ducts), two points along x per thread: the
+// pair's rows are read as one float2 each, plus the values left and right of
+// it where a stencil reaches there. Bound by the rows that go through L2 (27
+// arrays' worth where 16 pass through HBM, with a plane a block): the viscous
+// one marches a chunk of planes and reads 16 to 17. On 128x128x256: one point
+// per thread 74 us, pairs 71, pairs marching 59 (HBM's share 40); the pressure
+// one 32 to 23. Pairs of a plane are numbered without gaps along x of the
+// grid, chunks of planes along y (pair_grid). The expressions are those of
+// v_residual_point and p_residual_at.
+constexpr int kVResSM = 2;   // resident blocks of the viscous one
+struct PairAt {
+  int x0, j;
+  int dl, dr;        // offsets of the points left (x0 - 1) and right (x0 + 2) of the pair
+  int oj, ojm, ojp;  // row offsets: this row, the rows below and above
+  bool ok, two, wm0, wp0, wp1;   // wm0: x0 on the lower wall; wp: a point below the upper wall
+};
+__device__ __forceinline__ PairAt pair_at(const Geo& g, const Blk& B) {
+  PairAt p;
+  const int np = (g.n[0] + 1) >> 1;
+  const int q = (B.x + B.gx * B.z) * (int)blockDim.x + (int)threadIdx.x;
+  p.j = q / np;
+  p.x0 = 2 * (q - p.j * np);
+  p.ok = p.j < g.n[1];
+  const bool per = g.per[0] != 0;
+  p.dl = p.x0 > 0 ? -1 : (per ? g.n[0] - 1 : 0);
+  p.dr = per && p.x0 + 2 >= g.n[0] ? -p.x0 : (p.x0 + 2 < g.s[0] ? 2 : 1);
+  p.two = p.x0 + 1 < g.n[0];
+  p.wm0 = !per && p.x0 == 0;
+  p.wp0 = !per && p.x0 == g.n[0] - 1;
+  p.wp1 = !per && p.x0 + 1 == g.n[0] - 1;
+  const int st1 = (int)g.st[1];
+  const int jm = p.j > 0 ? p.j - 1 : (g.per[1] ? g.n[1] - 1 : 0);
+  const int jp = g.per[1] && p.j == g.n[1] - 1 ? 0 : p.j + 1;
+  p.oj = p.x0 + st1 * p.j;
+  p.ojm = p.x0 + st1 * jm;
+  p.ojp = p.x0 + st1 * jp;
+  return p;
+}
+struct PairRow {
+  float v[4];   // x0 - 1, x0, x0 + 1, x0 + 2
+};
+template <bool LEFT, bool RIGHT>
+__device__ __forceinline__ PairRow pair_row(const float* __restrict__ a, int o, const PairAt& p) {
+  PairRow r;
+  const float2 c = *reinterpret_cast<const float2*>(a + o);
+  r.v[0] = LEFT ? a[o + p.dl] : 0.f;
+  r.v[1] = c.x;
+  r.v[2] = c.y;
+  r.v[3] = RIGHT ? a[o + p.dr] : 0.f;
+  return r;
+}
+__device__ __forceinline__ void pair_store(float* __restrict__ a, int o, const PairAt& p,
+                                           const float r[2]) {
+  if (p.two) *reinterpret_cast<float2*>(a + o) = make_float2(r[0], r[1]);
+  else a[o] = r[0];
+}
+
+// Marches the chunk's planes upwards: what the stencil reads of the planes
+// below and above is kept from the plane before, or kept for the next one,
+// in registers, which halves the rows read through L2.
+__device__ __forceinline__ void v_residual_pair_body(const Blk& B, const Geo& g,
+                                                     const LevelPtrs<float>& L, float ir) {
+  const PairAt p = pair_at(g, B);
+  if (!p.ok) return;
+  const int st2 = (int)g.st[2], KC = (g.n[2] + B.gy - 1) / B.gy;
+  const int k0 = B.y * KC, k1 = k0 + KC < g.n[2] ? k0 + KC : g.n[2];
+  if (k0 >= k1) return;
+  const bool wmy = !g.per[1] && p.j == 0, wpy = !g.per[1] && p.j == g.n[1] - 1;
+  const int zb = (k0 > 0 ? k0 - 1 : (g.per[2] ? g.n[2] - 1 : 0)) * st2;
+  // the plane below: u_x, u_y (and its row above), u_z, mu_c
+  PairRow Xm = pair_row<false, true>(L.u[0], p.oj + zb, p);
+  PairRow Ym = pair_row<false, false>(L.u[1], p.oj + zb, p);
+  PairRow Yq = pair_row<false, false>(L.u[1], p.ojp + zb, p);
+  PairRow Zm = pair_row<false, false>(L.u[2], p.oj + zb, p);
+  PairRow Cm = pair_row<false, false>(L.muc, p.oj + zb, p);
+  // this plane
+  PairRow X = pair_row<true, true>(L.u[0], p.oj + k0 * st2, p);
+  PairRow Y = pair_row<true, true>(L.u[1], p.oj + k0 * st2, p);
+  PairRow Z = pair_row<true, true>(L.u[2], p.oj + k0 * st2, p);
+  PairRow Zym = pair_row<false, false>(L.u[2], p.ojm + k0 * st2, p);
+  PairRow Exz = pair_row<false, true>(L.mue[1], p.oj + k0 * st2, p);
+  PairRow Eyz = pair_row<false, false>(L.mue[2], p.oj + k0 * st2, p);
+  for (int k = k0; k < k1; ++k) {
+    const int zc = k * st2, zp = (g.per[2] && k == g.n[2] - 1 ? 0 : k + 1) * st2;
+    const bool wmz = !g.per[2] && k == 0, wpz = !g.per[2] && k == g.n[2] - 1;
+    const PairRow Xp = pair_row<true, true>(L.u[0], p.oj + zp, p);
+    const PairRow Yp = pair_row<true, true>(L.u[1], p.oj + zp, p);
+    const PairRow Zp = pair_row<true, true>(L.u[2], p.oj + zp, p);
+    const PairRow Zq = pair_row<false, false>(L.u[2], p.ojm + zp, p);
+    const PairRow Fxz = pair_row<false, true>(L.mue[1], p.oj + zp, p);
+    const PairRow Fyz = pair_row<false, false>(L.mue[2], p.oj + zp, p);
+    const PairRow Xym = pair_row<false, true>(L.u[0], p.ojm + zc, p);
+    const PairRow Yyp = pair_row<true, false>(L.u[1], p.ojp + zc, p);
+    const PairRow C = pair_row<true, false>(L.muc, p.oj + zc, p);
+    const PairRow Exy = pair_row<false, true>(L.mue[0], p.oj + zc, p);
+    float r[2];
+    {   // x
+      const PairRow Xyp = pair_row<false, false>(L.u[0], p.ojp + zc, p);
+      const PairRow Fxy = pair_row<false, false>(L.mue[0], p.ojp + zc, p);
+      const PairRow f = pair_row<false, false>(L.uf[0], p.oj + zc, p);
+      const PairRow m = pair_row<false, false>(L.m[0], p.oj + zc, p);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int i = 1 + e;
+        const float u = X.v[i];
+        float V = vr_normal(C.v[i], X.v[i + 1], u, C.v[i - 1], X.v[i - 1]);
+        V = vr_edge(V, u, Fxy.v[i], wpy ? -u : Xyp.v[i], Yyp.v[i], Yyp.v[i - 1], Exy.v[i],
+                    wmy ? -u : Xym.v[i], Y.v[i], Y.v[i - 1]);
+        V = vr_edge(V, u, Fxz.v[i], wpz ? -u : Xp.v[i], Zp.v[i], Zp.v[i - 1], Exz.v[i],
+                    wmz ? -u : Xm.v[i], Z.v[i], Z.v[i - 1]);
+        r[e] = e == 0 && p.wm0 ? 0.f : vr_final(f.v[i], m.v[i], u, ir, V);
+      }
+      pair_store(L.ur[0], p.oj + zc, p, r);
+    }
+    {   // y
+      const PairRow Yym = pair_row<false, false>(L.u[1], p.ojm + zc, p);
+      const PairRow Cym = pair_row<false, false>(L.muc, p.ojm + zc, p);
+      const PairRow f = pair_row<false, false>(L.uf[1], p.oj + zc, p);
+      const PairRow m = pair_row<false, false>(L.m[1], p.oj + zc, p);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int i = 1 + e;
+        const float u = Y.v[i];
+        const bool wp = e == 0 ? p.wp0 : p.wp1, wm = e == 0 && p.wm0;
+        float V = vr_normal(C.v[i], Yyp.v[i], u, Cym.v[i], Yym.v[i]);
+        V = vr_edge(V, u, Exy.v[i + 1], wp ? -u : Y.v[i + 1], X.v[i + 1], Xym.v[i + 1], Exy.v[i],
+                    wm ? -u : Y.v[i - 1], X.v[i], Xym.v[i]);
+        V = vr_edge(V, u, Fyz.v[i], wpz ? -u : Yp.v[i], Zp.v[i], Zq.v[i], Eyz.v[i],
+                    wmz ? -u : Ym.v[i], Z.v[i], Zym.v[i]);
+        r[e] = wmy ? 0.f : vr_final(f.v[i], m.v[i], u, ir, V);
+      }
+      pair_store(L.ur[1], p.oj + zc, p, r);
+    }
+    {   // z
+      const PairRow Zyp = pair_row<false, false>(L.u[2], p.ojp + zc, p);
+      const PairRow Gyz = pair_row<false, false>(L.mue[2], p.ojp + zc, p);
+      const PairRow f = pair_row<false, false>(L.uf[2], p.oj + zc, p);
+      const PairRow m = pair_row<false, false>(L.m[2], p.oj + zc, p);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int i = 1 + e;
+        const float u = Z.v[i];
+        const bool wp = e == 0 ? p.wp0 : p.wp1, wm = e == 0 && p.wm0;
+        float V = vr_normal(C.v[i], Zp.v[i], u, Cm.v[i], Zm.v[i]);
+        V = vr_edge(V, u, Exz.v[i + 1], wp ? -u : Z.v[i + 1], X.v[i + 1], Xm.v[i + 1], Exz.v[i],
+                    wm ? -u : Z.v[i - 1], X.v[i], Xm.v[i]);
+        V = vr_edge(V, u, Gyz.v[i], wpy ? -u : Zyp.v[i], Yyp.v[i], Yq.v[i], Eyz.v[i],
+                    wmy ? -u : Zym.v[i], Y.v[i], Ym.v[i]);
+        r[e] = wmz ? 0.f : vr_final(f.v[i], m.v[i], u, ir, V);
+      }
+      pair_store(L.ur[2], p.oj + zc, p, r);
+    }
+    Xm = X, X = Xp, Ym = Y, Y = Yp, Yq = Yyp, Zm = Z, Z = Zp, Zym = Zq, Cm = C;
+    Exz = Fxz, Eyz = Fyz;
+  }
+}
+
+__device__ __forceinline__ void p_residual_pair_body(const Blk& B, const Geo& g,
+                                                     const LevelPtrs<float>& L, float ih2) {
+  const PairAt p = pair_at(g, B);
+  if (!p.ok) return;
+  const int st2 = (int)g.st[2];
+  const bool wmy = !g.per[1] && p.j == 0, wpy = !g.per[1] && p.j == g.n[1] - 1;
+  for (int k = B.y; k < g.n[2]; k += B.gy) {
+    const int zc = k * st2;
+    const int zm = (k > 0 ? k - 1 : (g.per[2] ? g.n[2] - 1 : 0)) * st2;
+    const int zp = (g.per[2] && k == g.n[2] - 1 ? 0 : k + 1) * st2;
+    const bool wmz = !g.per[2] && k == 0, wpz = !g.per[2] && k == g.n[2] - 1;
+    const PairRow P = pair_row<true, true>(L.p, p.oj + zc, p);
+    const PairRow ym = pair_row<false, false>(L.p, p.ojm + zc, p);
+    const PairRow yp = pair_row<false, false>(L.p, p.ojp + zc, p);
+    const PairRow zmr = pair_row<false, false>(L.p, p.oj + zm, p);
+    const PairRow zpr = pair_row<false, false>(L.p, p.oj + zp, p);
+    const PairRow bx = pair_row<false, true>(L.beta[0], p.oj + zc, p);
+    const PairRow by = pair_row<false, false>(L.beta[1], p.oj + zc, p);
+    const PairRow byp = pair_row<false, false>(L.beta[1], p.ojp + zc, p);
+    const PairRow bz = pair_row<false, false>(L.beta[2], p.oj + zc, p);
+    const PairRow bzp = pair_row<false, false>(L.beta[2], p.oj + zp, p);
+    const PairRow f = pair_row<false, false>(L.pf, p.oj + zc, p);
+    float r[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int i = 1 + e;
+      float num = 0.f, dg = 0.f;
+      if (!(e == 0 && p.wm0)) px_acc(num, dg, bx.v[i], P.v[i - 1]);
+      if (!(e == 0 ? p.wp0 : p.wp1)) px_acc(num, dg, bx.v[i + 1], P.v[i + 1]);
+      if (!wmy) px_acc(num, dg, by.v[i], ym.v[i]);
+      if (!wpy) px_acc(num, dg, byp.v[i], yp.v[i]);
+      if (!wmz) px_acc(num, dg, bz.v[i], zmr.v[i]);
+      if (!wpz) px_acc(num, dg, bzp.v[i], zpr.v[i]);
+      r[e] = pr_final(f.v[i], num, dg, P.v[i], ih2);
+    }
+    pair_store(L.pr, p.oj + zc, p, r);
+  }
+}
+
+__global__ void __launch_bounds__(256, kVResSM) k_v_residual_pair(const __grid_constant__ Geo g,
+                                                         const __grid_constant__ LevelPtrs<float> L,
+                                                         float ir) {
+  v_residual_pair_body(own_blk(), g, L, ir);
+}
+__global__ void __launch_bounds__(256) k_p_residual_pair(const __grid_constant__ Geo g,
+                                                         const __grid_constant__ LevelPtrs<float> L,
+                                                         float ih2) {
+  p_residual_pair_body(own_blk(), g, L, ih2);
+}
+
 template <int D, typename T>
 __global__ void __launch_bounds__(256) k_v_residual(Geo g, LevelPtrs<T> L, T ir) {
   v_residual_body<D, T>(own_blk(), g, L, ir);
@@ -432,109 +639,117 @@ __global__ void __launch_bounds__(256) k_prolong_face(Geo gf, Geo gc, const T* _
   prolong_face_body<D, d, T>(own_blk(), gf, gc, ec, xf);
 }
 
-// the three components in one pass over the fine cells (3D, no open axis).
-// Each axis's 1D weights and indices are formed once per cell, by the cell
-// rule (a tangential axis, odd mirror at walls) and by the face rule (the
-// component's own axis), and shared by the components; the sums are those of
-// prolong_face_at, term for term.
+// The prolongations of closed 3D ducts: the three velocity components (NC = 3)
+// or the pressure (NC = 1). Two fine points along x per thread, 2I and 2I + 1,
+// which share the coarse x index I, marching a chunk of coarse planes: the
+// sums over x and y on a coarse plane are formed once and serve the four fine
+// planes that take a share of it, and the fine values are read and written as
+// one vector a pair. On 128x128x256 (FP32) 29 us against 40 with the four
+// coarse rows loaded for each pair of points (NC = 3; the bytes are worth 16),
+// 12 against 24 (NC = 1).
+// Each point's sum is prol_sum's, term for term. Blocks as prolong_grid says.
+constexpr int prol_sm(size_t elem) { return elem == 4 ? 4 : 2; }   // resident blocks
 template <typename T>
-__device__ __forceinline__ void prolong_face3_body(const Blk& B, const Geo& gf, const Geo& gc,
-                                                   const Faces3<T>& ec, const Faces3<T>& xf) {
-  const int fi[3] = {(int)(B.x * blockDim.x + threadIdx.x), (int)(B.y * blockDim.y + threadIdx.y),
-                     (int)(B.z * blockDim.z + threadIdx.z)};
-  if (fi[0] >= gf.n[0] || fi[1] >= gf.n[1] || fi[2] >= gf.n[2]) return;
-  int cidx[3][2], fidx[3][2];
-  T cw[3][2], fw[3][2];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    prol_cell_1d<T>(fi[a], gc.n[a], gc.per[a], -1, -1, cidx[a], cw[a]);
-    prol_face_1d<T>(fi[a], gc.n[a], gc.per[a], fidx[a], fw[a]);
+struct Vec2;
+template <>
+struct Vec2<float> {
+  using type = float2;
+};
+template <>
+struct Vec2<double> {
+  using type = double2;
+};
+template <int NC, typename T>
+__device__ __forceinline__ void prolong_pair_body(const Blk& B, const Geo& gf, const Geo& gc,
+                                                  const Faces3<T>& ec, const Faces3<T>& xf) {
+  const int np = gc.n[0], q = (B.x + B.gx * B.z) * (int)blockDim.x + (int)threadIdx.x;
+  const int j = q / np, I = q - j * np;
+  const int nk = gc.n[2], KC = (nk + B.gy - 1) / B.gy;
+  const int K0 = B.y * KC, K1 = K0 + KC < nk ? K0 + KC : nk;
+  if (j >= gf.n[1] || K0 >= K1) return;
+  // per axis the cell-centred and, for velocities, the face weights (x: both points)
+  constexpr int mir = NC == 3 ? -1 : +1;   // tangential velocities are odd at walls
+  int cxa[2], cxb[2], fxa[2], fxb[2], cy[2], fy[2];
+  T wcxa[2], wcxb[2], wfxa[2], wfxb[2], wcy[2], wfy[2];
+  prol_cell_1d<T>(2 * I, gc.n[0], gc.per[0], mir, mir, cxa, wcxa);
+  prol_cell_1d<T>(2 * I + 1, gc.n[0], gc.per[0], mir, mir, cxb, wcxb);
+  prol_cell_1d<T>(j, gc.n[1], gc.per[1], mir, mir, cy, wcy);
+  if constexpr (NC == 3) {
+    prol_face_1d<T>(2 * I, gc.n[0], gc.per[0], fxa, wfxa);
+    prol_face_1d<T>(2 * I + 1, gc.n[0], gc.per[0], fxb, wfxb);
+    prol_face_1d<T>(j, gc.n[1], gc.per[1], fy, wfy);
   }
-  const long long x = gidx(gf, fi[0], fi[1], fi[2]);
+  const int cst1 = (int)gc.st[1], cst2 = (int)gc.st[2];
+  struct Col {
+    T a, b;
+  };
+  auto plane = [&](int d, int K) {   // the sums over x and y of component d on coarse plane K
+    const bool fx = NC == 3 && d == 0, fyy = NC == 3 && d == 1;
+    T ra[2], rb[2];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    if (!gf.per[d] && fi[d] == 0) continue;   // the wall face
-    int idx[3][2];
-    T w[3][2];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        idx[a][t] = a == d ? fidx[a][t] : cidx[a][t];
-        w[a][t] = a == d ? fw[a][t] : cw[a][t];
-      }
-    xf.a[d][x] = padd(xf.a[d][x], prol_sum<T>(gc, ec.a[d], idx, w));
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_prolong_face3(Geo gf, Geo gc, Faces3<T> ec, Faces3<T> xf) {
-  prolong_face3_body<T>(own_blk(), gf, gc, ec, xf);
-}
-
-// The same corrections, two fine points along x per thread: cells or faces
-// 2I and 2I + 1 share the coarse x index I and every y and z index and
-// weight, so each coarse row is addressed once and its value at I loaded once
-// for both; each point's sum is prol_sum's, term for term. The fine x extent
-// is even (twice the coarse one).
-template <typename T>
-__device__ __forceinline__ void prol_pair_sum(const Geo& gc, const T* __restrict__ e, int I,
-                                              const int xa[2], const T wa[2], const int xb[2],
-                                              const T wb[2], const int iy[2], const T wy[2],
-                                              const int iz[2], const T wz[2], T& va, T& vb) {
-  T cola[2], colb[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    T rowa[2], rowb[2];
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const T* __restrict__ r = e + gidx(gc, 0, iy[b], iz[c]);
-      const T e0 = r[I];   // xa[0] == xb[0] == I
-      rowa[b] = pfma(wa[1], r[xa[1]], pmul(wa[0], e0));
-      rowb[b] = pfma(wb[1], r[xb[1]], pmul(wb[0], e0));
+    for (int t = 0; t < 2; ++t) {
+      const T* __restrict__ r = ec.a[d] + (fyy ? fy[t] : cy[t]) * cst1 + K * cst2;
+      const T e0 = r[I], eb = r[fx ? fxb[1] : cxb[1]];
+      const T ea = fx ? e0 : r[cxa[1]];   // a face 2I lies on the coarse face I
+      ra[t] = pfma(fx ? wfxa[1] : wcxa[1], ea, pmul(fx ? wfxa[0] : wcxa[0], e0));
+      rb[t] = pfma(fx ? wfxb[1] : wcxb[1], eb, pmul(fx ? wfxb[0] : wcxb[0], e0));
     }
-    cola[c] = pfma(wy[1], rowa[1], pmul(wy[0], rowa[0]));
-    colb[c] = pfma(wy[1], rowb[1], pmul(wy[0], rowb[0]));
+    const T w0 = fyy ? wfy[0] : wcy[0], w1 = fyy ? wfy[1] : wcy[1];
+    return Col{pfma(w1, ra[1], pmul(w0, ra[0])), pfma(w1, rb[1], pmul(w0, rb[0]))};
+  };
+  const bool perz = gc.per[2] != 0;
+  Col c[NC], cm[NC];
+  const int Kb = K0 > 0 ? K0 - 1 : (perz ? nk - 1 : 0);
+#pragma unroll
+  for (int d = 0; d < NC; ++d) {
+    c[d] = plane(d, K0);
+    if (!(NC == 3 && d == 2)) cm[d] = plane(d, Kb);
   }
-  va = pfma(wz[1], cola[1], pmul(wz[0], cola[0]));
-  vb = pfma(wz[1], colb[1], pmul(wz[0], colb[0]));
+  for (int K = K0; K < K1; ++K) {
+    const bool last = K + 1 == nk;
+    const int Kc = last ? (perz ? 0 : K) : K + 1, Kf = last && perz ? 0 : K + 1;
+    Col cp[NC];
+#pragma unroll
+    for (int d = 0; d < NC; ++d) cp[d] = plane(d, NC == 3 && d == 2 ? Kf : Kc);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const int k = 2 * K + o;
+      int iz[2];
+      T wc[2], wf[2];
+      prol_cell_1d<T>(k, nk, gc.per[2], mir, mir, iz, wc);
+      prol_face_1d<T>(k, nk, gc.per[2], iz, wf);
+      const int x = 2 * I + (int)gf.st[1] * j + (int)gf.st[2] * k;
+#pragma unroll
+      for (int d = 0; d < NC; ++d) {
+        const bool fz = NC == 3 && d == 2;
+        // (the wall faces of y and z stay; the one of x is put back)
+        if (NC == 3 && d == 1 && !gf.per[1] && j == 0) continue;
+        if (fz && !gf.per[2] && k == 0) continue;
+        // the second term: below an even cell, above an odd one; an even face has none
+        const Col& t = o ? cp[d] : (fz ? c[d] : cm[d]);
+        const T w0 = fz ? wf[0] : wc[0], w1 = fz ? wf[1] : wc[1];
+        using V = typename Vec2<T>::type;
+        V* at = reinterpret_cast<V*>(xf.a[d] + x);
+        V v = *at;
+        if (!(NC == 3 && d == 0) || gf.per[0] || I != 0) v.x = padd(v.x, pfma(w1, t.a, pmul(w0, c[d].a)));
+        v.y = padd(v.y, pfma(w1, t.b, pmul(w0, c[d].b)));
+        *at = v;
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < NC; ++d) {
+      cm[d] = c[d];
+      c[d] = cp[d];
+    }
+  }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_prolong_face3_pair(Geo gf, Geo gc, Faces3<T> ec,
-                                                           Faces3<T> xf) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z * blockDim.z + threadIdx.z;
-  const int i0 = 2 * I;
-  if (i0 >= gf.n[0] || j >= gf.n[1] || k >= gf.n[2]) return;
-  // per axis the cell-centred and the face weights (x: both points)
-  int cxa[2], cxb[2], fxa[2], fxb[2], cy[2], fy[2], cz[2], fz[2];
-  T wcxa[2], wcxb[2], wfxa[2], wfxb[2], wcy[2], wfy[2], wcz[2], wfz[2];
-  prol_cell_1d<T>(i0, gc.n[0], gc.per[0], -1, -1, cxa, wcxa);
-  prol_cell_1d<T>(i0 + 1, gc.n[0], gc.per[0], -1, -1, cxb, wcxb);
-  prol_face_1d<T>(i0, gc.n[0], gc.per[0], fxa, wfxa);
-  prol_face_1d<T>(i0 + 1, gc.n[0], gc.per[0], fxb, wfxb);
-  prol_cell_1d<T>(j, gc.n[1], gc.per[1], -1, -1, cy, wcy);
-  prol_face_1d<T>(j, gc.n[1], gc.per[1], fy, wfy);
-  prol_cell_1d<T>(k, gc.n[2], gc.per[2], -1, -1, cz, wcz);
-  prol_face_1d<T>(k, gc.n[2], gc.per[2], fz, wfz);
-  const long long x = gidx(gf, i0, j, k);
-  T va, vb;
-  // x-faces: the wall face 0 (the first point of the first pair) is fixed
-  prol_pair_sum<T>(gc, ec.a[0], I, fxa, wfxa, fxb, wfxb, cy, wcy, cz, wcz, va, vb);
-  if (gf.per[0] || i0 != 0) xf.a[0][x] = padd(xf.a[0][x], va);
-  xf.a[0][x + 1] = padd(xf.a[0][x + 1], vb);
-  if (gf.per[1] || j != 0) {   // y-faces
-    prol_pair_sum<T>(gc, ec.a[1], I, cxa, wcxa, cxb, wcxb, fy, wfy, cz, wcz, va, vb);
-    xf.a[1][x] = padd(xf.a[1][x], va);
-    xf.a[1][x + 1] = padd(xf.a[1][x + 1], vb);
-  }
-  if (gf.per[2] || k != 0) {   // z-faces
-    prol_pair_sum<T>(gc, ec.a[2], I, cxa, wcxa, cxb, wcxb, cy, wcy, fz, wfz, va, vb);
-    xf.a[2][x] = padd(xf.a[2][x], va);
-    xf.a[2][x + 1] = padd(xf.a[2][x + 1], vb);
-  }
+template <int NC, typename T>
+__global__ void __launch_bounds__(256, prol_sm(sizeof(T))) k_prolong_pair(const __grid_constant__ Geo gf,
+                                                               const __grid_constant__ Geo gc,
+                                                               const Faces3<T> ec,
+                                                               const Faces3<T> xf) {
+  prolong_pair_body<NC, T>(own_blk(), gf, gc, ec, xf);
 }
 
 // ---------------------------------------------------------------------------
@@ -1333,15 +1548,19 @@ __global__ void k_fill(double* a, long long n, double v) {
 // copies a member's geometry and pointers out of the table before the body
 // runs, so the body's stores cannot alias them.
 // ===========================================================================
-__global__ void __launch_bounds__(256) kb_v_residual32(BArgs A) {
+__global__ void __launch_bounds__(256, kVResSM) kb_v_residual32(BArgs A) {
   for_items(A, [&](const BMember& M, const Blk& B) {
-    v_residual_body<3, float>(B, M.g[A.lev], cur_ptrs(M.f[A.lev], A.cur), (float)M.ir[A.lev]);
+    const Geo g = M.g[A.lev];
+    const LevelPtrs<float> L = cur_ptrs(M.f[A.lev], A.cur);
+    v_residual_pair_body(B, g, L, (float)M.ir[A.lev]);
   });
 }
 
 __global__ void __launch_bounds__(256) kb_p_residual32(BArgs A) {
   for_items(A, [&](const BMember& M, const Blk& B) {
-    p_residual_body<3, float>(B, M.g[A.lev], cur_ptrs(M.f[A.lev], A.cur), (float)M.ih2[A.lev]);
+    const Geo g = M.g[A.lev];
+    const LevelPtrs<float> L = cur_ptrs(M.f[A.lev], A.cur);
+    p_residual_pair_body(B, g, L, (float)M.ih2[A.lev]);
   });
 }
 
@@ -1365,7 +1584,7 @@ __global__ void __launch_bounds__(256) kb_restrict_cell32(BArgs A) {
   });
 }
 
-__global__ void __launch_bounds__(256) kb_prolong_face32(BArgs A) {
+__global__ void __launch_bounds__(256, prol_sm(4)) kb_prolong_face32(BArgs A) {
   for_items(A, [&](const BMember& M, const Blk& B) {
     const int l = A.lev;
     Faces3<float> ec, xf;
@@ -1373,14 +1592,17 @@ __global__ void __launch_bounds__(256) kb_prolong_face32(BArgs A) {
       ec.a[d] = M.f[l + 1].u[d];
       xf.a[d] = M.f[l].u[d];
     }
-    prolong_face3_body<float>(B, M.g[l], M.g[l + 1], ec, xf);
+    prolong_pair_body<3, float>(B, M.g[l], M.g[l + 1], ec, xf);
   });
 }
 
-__global__ void __launch_bounds__(256) kb_prolong_cell32(BArgs A) {
+__global__ void __launch_bounds__(256, prol_sm(4)) kb_prolong_cell32(BArgs A) {
   for_items(A, [&](const BMember& M, const Blk& B) {
     const int l = A.lev;
-    prolong_cell_body<3, float>(B, M.g[l], M.g[l + 1], M.f[l + 1].p, M.f[l].p);
+    Faces3<float> ec, xf;
+    ec.a[0] = M.f[l + 1].p;
+    xf.a[0] = M.f[l].p;
+    prolong_pair_body<1, float>(B, M.g[l], M.g[l + 1], ec, xf);
   });
 }
 
@@ -1533,13 +1755,40 @@ void launch_p_rbgs(int D, const Geo& g, const LevelPtrs<T>& L, int colour, cudaS
   else L.pdg ? run(k_p_rbgs<2, T, true>) : run(k_p_rbgs<2, T, false>);
 }
 
+// Blocks of a pair kernel: a plane's pairs along x (and z, where x would pass
+// the 16 bits of a work item), chunks of planes along y: as many planes a
+// chunk as take the least time with per_sm blocks resident on an SM, a chunk
+// costing about one plane more than it holds (per_sm 0: a plane a block).
+dim3 pair_grid(const Geo& g, int planes, int per_sm) {
+  const long long nb = ((long long)((g.n[0] + 1) / 2) * g.n[1] + 255) / 256;
+  const long long x = nb < 32768 ? nb : 32768, z = (nb + x - 1) / x;
+  int KC = (planes + 32767) / 32768;
+  if (per_sm > 0) {
+    const long long slots = 152LL * per_sm;
+    double best = 1e300;
+    for (int q = KC; q <= planes && q <= KC + 63; ++q) {
+      const long long blocks = x * z * ((planes + q - 1) / q);
+      const double t = (double)((blocks + slots - 1) / slots) * (q + 1.0);
+      if (t < best) {
+        best = t;
+        KC = q;
+      }
+    }
+  }
+  return dim3((unsigned)x, (unsigned)((planes + KC - 1) / KC), (unsigned)z);
+}
+dim3 v_residual_grid(const Geo& g) { return pair_grid(g, g.n[2], kVResSM); }
+dim3 p_residual_grid(const Geo& g) { return pair_grid(g, g.n[2], 0); }
+dim3 prolong_grid(const Geo& gf, size_t elem) { return pair_grid(gf, gf.n[2] / 2, prol_sm(elem)); }
+
 template <typename T>
 void launch_p_residual(int D, const Geo& g, const LevelPtrs<T>& L, cudaStream_t s) {
   dim3 b = blk3(D);
   dim3 gr = grd3(g.n[0], g.n[1], g.n[2], b);
   const T ih2 = (T)(1.0 / (g.h * g.h));
-  if (D == 3) k_p_residual<3, T><<<gr, b, 0, s>>>(g, L, ih2);
-  else k_p_residual<2, T><<<gr, b, 0, s>>>(g, L, ih2);
+  if (D == 2) k_p_residual<2, T><<<gr, b, 0, s>>>(g, L, ih2);
+  else if constexpr (sizeof(T) == 4) k_p_residual_pair<<<p_residual_grid(g), 256, 0, s>>>(g, L, ih2);
+  else k_p_residual<3, T><<<gr, b, 0, s>>>(g, L, ih2);
 }
 
 template <typename T>
@@ -1564,8 +1813,9 @@ void launch_v_residual(int D, const Geo& g, const LevelPtrs<T>& L, double inv_re
   dim3 b = blk3(D);
   dim3 gr = grd3(ext(g, 0, true), ext(g, 1, true), ext(g, 2, true), b);
   T ir = (T)(inv_re / (g.h * g.h));
-  if (D == 3) k_v_residual<3, T><<<gr, b, 0, s>>>(g, L, ir);
-  else k_v_residual<2, T><<<gr, b, 0, s>>>(g, L, ir);
+  if (D == 2) k_v_residual<2, T><<<gr, b, 0, s>>>(g, L, ir);
+  else if constexpr (sizeof(T) == 4) k_v_residual_pair<<<v_residual_grid(g), 256, 0, s>>>(g, L, ir);
+  else k_v_residual<3, T><<<gr, b, 0, s>>>(g, L, ir);
 }
 
 template <typename T>
@@ -1596,8 +1846,16 @@ template <typename T>
 void launch_prolong_cell(int D, const Geo& gf, const Geo& gc, const T* ec, T* xf, cudaStream_t s) {
   dim3 b = blk3(D);
   dim3 gr = grd3(gf.n[0], gf.n[1], gf.n[2], b);
-  if (D == 3) k_prolong_cell<3, T><<<gr, b, 0, s>>>(gf, gc, ec, xf);
-  else k_prolong_cell<2, T><<<gr, b, 0, s>>>(gf, gc, ec, xf);
+  if (D == 2) {
+    k_prolong_cell<2, T><<<gr, b, 0, s>>>(gf, gc, ec, xf);
+  } else if (gf.open < 0) {
+    Faces3<T> e, x;
+    e.a[0] = const_cast<T*>(ec);
+    x.a[0] = xf;
+    k_prolong_pair<1, T><<<prolong_grid(gf, sizeof(T)), 256, 0, s>>>(gf, gc, e, x);
+  } else if constexpr (sizeof(T) == 8) {   // open ducts run in FP64
+    k_prolong_cell<3, T><<<gr, b, 0, s>>>(gf, gc, ec, xf);
+  }
 }
 
 template <typename T>
@@ -1636,11 +1894,7 @@ void launch_prolong_face3(const Geo& gf, const Geo& gc, T* const ec[3], T* const
     e.a[d] = ec[d];
     x.a[d] = xf[d];
   }
-  dim3 b = blk3(3);
-  if (gf.n[0] % 2 == 0)
-    k_prolong_face3_pair<T><<<grd3(gf.n[0] / 2, gf.n[1], gf.n[2], b), b, 0, s>>>(gf, gc, e, x);
-  else
-    k_prolong_face3<T><<<grd3(gf.n[0], gf.n[1], gf.n[2], b), b, 0, s>>>(gf, gc, e, x);
+  k_prolong_pair<3, T><<<prolong_grid(gf, sizeof(T)), 256, 0, s>>>(gf, gc, e, x);
 }
 template void launch_restrict_face3<float>(const Geo&, const Geo&, float* const[3],
                                            float* const[3], float* const[3], cudaStream_t);
@@ -1874,10 +2128,10 @@ dim3 stencil_grid3(long long nx, long long ny, long long nz) { return grd3(nx, n
 
 // ------------------------------------------------------------------ batched
 void launch_b_v_residual32(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_v_residual32<<<grid, blk3(3), 0, s>>>(A);
+  if (A.n > 0) kb_v_residual32<<<grid, 256, 0, s>>>(A);
 }
 void launch_b_p_residual32(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_p_residual32<<<grid, blk3(3), 0, s>>>(A);
+  if (A.n > 0) kb_p_residual32<<<grid, 256, 0, s>>>(A);
 }
 void launch_b_restrict_face32(const BArgs& A, int grid, cudaStream_t s) {
   if (A.n > 0) kb_restrict_face32<<<grid, blk3(3), 0, s>>>(A);
@@ -1886,10 +2140,10 @@ void launch_b_restrict_cell32(const BArgs& A, int grid, cudaStream_t s) {
   if (A.n > 0) kb_restrict_cell32<<<grid, blk3(3), 0, s>>>(A);
 }
 void launch_b_prolong_face32(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_prolong_face32<<<grid, blk3(3), 0, s>>>(A);
+  if (A.n > 0) kb_prolong_face32<<<grid, 256, 0, s>>>(A);
 }
 void launch_b_prolong_cell32(const BArgs& A, int grid, cudaStream_t s) {
-  if (A.n > 0) kb_prolong_cell32<<<grid, blk3(3), 0, s>>>(A);
+  if (A.n > 0) kb_prolong_cell32<<<grid, 256, 0, s>>>(A);
 }
 size_t b_coarse_smem(const Geo& g, bool viscous) {
   const size_t b = coarse_bytes(3, g, (int)sizeof(double), viscous);

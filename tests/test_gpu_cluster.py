@@ -38,6 +38,16 @@ def test_mixed_precision_bits(n, per):
         assert np.array_equal(a, b), np.abs(a - b).max()
 
 
+# the launches' FP32 residuals take two points along x: every pair beside a wall,
+# planes of one and of several blocks, more cells than a cluster's slabs hold on the finest level
+@pytest.mark.parametrize("n,per", [((4, 8, 8), (0, 0, 1)), ((12, 4, 12), (0, 1, 0)),
+                                   ((4, 12, 8), (1, 0, 0)), ((68, 36, 20), (0, 0, 1)),
+                                   ((44, 24, 72), (1, 1, 0))])
+def test_residual_pairs_bits(n, per):
+    for a, b in zip(solve(n, per, 1 << 15, 1), solve(n, per, 0, 1)):
+        assert np.array_equal(a, b), np.abs(a - b).max()
+
+
 @pytest.mark.parametrize("n,per", GRIDS)
 def test_fp64_to_rounding(n, per):
     for a, b in zip(solve(n, per, 1 << 20, 0), solve(n, per, 0, 0)):
