@@ -1494,6 +1494,29 @@ cudaError_t sweep_list(Persist& P, int l, int K, PShape& sh, PList& L) {
   return cudaSuccess;
 }
 
+// Chunk planes of an untuned batched pair sweep: the least time of 304 blocks
+// resident on 152 SMs, a chunk costing about one plane more than it holds.
+// (16 planes whatever the size left the second level of twelve 48x48x96
+// members with 108 blocks: 53.8 ms a step, 52.6 with this rule.)
+int pair_chunk(const Persist& P, int l, int TY) {
+  int best = 16;
+  double bc = 1e300;
+  for (int KC : {2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32}) {
+    long long items = 0;
+    for (size_t m = 0; m < P.mem.size(); ++m)
+      if (p_smooths(P, (int)m, l)) {
+        const Geo& g = P.mem[m]->lev[l].g;
+        items += (long long)((g.n[1] + TY - 1) / TY) * ((g.n[2] + KC - 1) / KC);
+      }
+    const double c = (double)((items + 303) / 304) * (KC + 1.0);
+    if (c < bc) {
+      bc = c;
+      best = KC;
+    }
+  }
+  return best;
+}
+
 // The built-in sweep shape of level l: one thread per point pair of the
 // widest member's rows (at most 128), 4 rows, chunks giving about three
 // blocks per SM.
@@ -1518,8 +1541,8 @@ PShape default_shape(const Persist& P, int l) {
   sh.KC = (int)std::max(4LL, std::min(16LL, KC));
   // the pair sweep where every member smoothing here can take it and the
   // level holds at least 2^19 cells in all: as many tile rows as the block
-  // holds of the widest member's rows (at most 14), 16-plane chunks, one block
-  // per item
+  // holds of the widest member's rows (at most 14), chunks that fill the chip, one
+  // block per item
   int bxu = 0, wid = 2, perz = -1;
   long long cells = 0;
   bool pair_ok = true;
@@ -1539,7 +1562,7 @@ PShape default_shape(const Persist& P, int l) {
     sh.kern = 1;
     sh.perz = perz;
     sh.TY = pTY;
-    sh.KC = 16;
+    sh.KC = pair_chunk(P, l, pTY);
     sh.NP = 1;
     sh.bx = bxu;
     sh.all = 1;
