@@ -10,10 +10,14 @@
 // (three edge stresses, three normal stresses; three fluxes), hands those its
 // neighbours need on through shared memory and carries those of the plane
 // below in registers. About 42 FP64 operations per cell for the viscous
-// operator instead of about 80, 14 instead of about 30 for the pressure, and
+// operator instead of about 80, 13 instead of about 30 for the pressure, and
 // one reduction per chunk instead of one per 256 points. w = A z on the
 // 128x128x256 duct: 506 us with the FP64 pipe 74 % busy, against 665 us (86 %)
 // face by face plus 34 us for an FP64 copy of z, which this form reads in FP32.
+// The pressure's planes are short, so each is loaded while the one before is
+// worked on: 147 us there and 269 us on 160x160x320 against 183 and 371 with
+// the loads in front of their use. (The viscous planes hold four times the
+// work; prefetching them towards L2 left 507 us at 507.)
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -256,45 +260,53 @@ __device__ __forceinline__ void p_op_body(const Blk& B, const Geo& g, const OpSh
     const int kw = k < 0 ? k + g.n[2] : (k >= g.n[2] ? k - g.n[2] : k);
     return st2 * (g.per[2] ? kw : min(max(k, 0), g.n[2] - 1));
   };
-  double pp = 0.0, fzp = 0.0, part = 0.0, acc = 0.0;
+  struct Raw {
+    double p, bx, by, bz, f;
+  };
+  auto load = [&](int k) {   // what the column needs of plane k (f: of the plane below)
+    Raw r{0.0, 0.0, 0.0, 0.0, 0.0};
+    if (q.in && k <= k1) {
+      const int pk = plane(k);
+      r.p = a.p[q.o + pk];
+      if (k < k1 && mid) {
+        if (!wx) r.bx = a.beta[0][q.om + pk];
+        if (!wy) r.by = a.beta[1][q.om + pk];
+      }
+      if (q.own && (g.per[2] || (k > 0 && k < g.n[2]))) r.bz = a.beta[2][q.o + pk];
+      if (q.own && k > k0) r.f = a.f[q.o + st2 * (k - 1)];
+    }
+    return r;
+  };
+  double pp = 0.0, part = 0.0, acc = 0.0;
   unsigned long long mx = 0ull;
   if (q.own) pp = a.p[q.o + plane(k0 - 1)];
+  Raw v = load(k0);
   for (int k = k0; k <= k1; ++k) {
-    double p = 0.0, bx = 0.0, by = 0.0, bz = 0.0, f = 0.0;
-    const int F = q.o + st2 * (k - 1);
-    if (q.in) {
-      const int pk = plane(k);
-      p = a.p[q.o + pk];
-      if (k < k1 && mid) {
-        if (!wx) bx = a.beta[0][q.om + pk];
-        if (!wy) by = a.beta[1][q.om + pk];
-      }
-      if (q.own && (g.per[2] || (k > 0 && k < g.n[2]))) bz = a.beta[2][q.o + pk];
-      if (q.own && k > k0) f = a.f[F];
-      A[t] = p;
-    }
+    A[t] = v.p;
     __syncthreads();
-    double fx = 0.0, fy = 0.0, fz = 0.0;
+    const Raw nx = load(k + 1);   // in flight over this plane's work
+    double fx = 0.0, fy = 0.0;
     if (mid && k < k1) {
-      fx = bx * (p - A[t - 1]);
-      fy = by * (p - A[t - w]);
+      fx = v.bx * (v.p - A[t - 1]);
+      fy = v.by * (v.p - A[t - w]);
       E[0][t] = fx;
       E[1][t] = fy;
     }
-    if (q.own) fz = bz * (p - pp);
     __syncthreads();
     if (q.own) {
+      const double dz = v.p - pp;
       if (k > k0) {
-        const double r = fma(-a.ih2, part + (fz - fzp), f);
+        const int F = q.o + st2 * (k - 1);
+        const double r = fma(-a.ih2, fma(v.bz, dz, part), v.f);
         a.r32[F] = narrow32(r);
         a.e32[F] = 0.f;
         acc = fma(r, r, acc);
         mx = op_umax(mx, (unsigned long long)__double_as_longlong(r) & 0x7fffffffffffffffull);
       }
-      if (k < k1) part = (E[0][t + 1] - fx) + (E[1][t + w] - fy);
+      if (k < k1) part = fma(-v.bz, dz, (E[0][t + 1] - fx) + (E[1][t + w] - fy));
     }
-    fzp = fz;
-    pp = p;
+    pp = v.p;
+    v = nx;
   }
   if (a.partial) {
     acc = op_block_sum(acc, sh);

@@ -1496,8 +1496,8 @@ cudaError_t sweep_list(Persist& P, int l, int K, PShape& sh, PList& L) {
 
 // Chunk planes of an untuned batched pair sweep: the least time of 304 blocks
 // resident on 152 SMs, a chunk costing about one plane more than it holds.
-// (16 planes whatever the size left the second level of twelve 48x48x96
-// members with 108 blocks: 53.8 ms a step, 52.6 with this rule.)
+// (16 planes whatever the size left the second level of twelve
+// members, edges 32 to 96, with 108 blocks: 53.8 ms a step, 52.6 with this rule.)
 int pair_chunk(const Persist& P, int l, int TY) {
   int best = 16;
   double bc = 1e300;

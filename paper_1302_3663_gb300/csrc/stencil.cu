@@ -329,7 +329,7 @@ __device__ __forceinline__ void v_residual_body(const Blk& B, Geo g, LevelPtrs<T
 // arrays' worth where 16 pass through HBM, with a plane a block): the viscous
 // one marches a chunk of planes and reads 16 to 17. On 128x128x256: one point
 // per thread 74 us, pairs 71, pairs marching 59 (HBM's share 40); the pressure
-// one 32 to 23. Pairs of a plane are numbered without gaps along x of the
+// one takes 23 with a plane a block (HBM 15). Pairs of a plane are numbered without gaps along x of the
 // grid, chunks of planes along y (pair_grid). The expressions are those of
 // v_residual_point and p_residual_at.
 constexpr int kVResSM = 2;   // resident blocks of the viscous one
