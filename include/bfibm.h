@@ -332,7 +332,8 @@ bfibm_status bfibm_sweep_shape(bfibm_ctx* c, int level, int kind, int32_t out[5]
    chunk (0: built-in), planes per phase (1 or 2), threads per row (0 or a
    multiple of 32 up to 128), kernel (0 ring sweep; 1 pair sweep, which takes
    tile rows >= 1, planes per chunk >= 1, planes per phase 1, threads per row
-   0 and a level with walls in x and y and an even row of at most 256 points)} for the shape of one level and kind, process-wide, in
+   0, at most 1024 threads (half a row's points for each tile row and two more) and a level
+   with walls in x and y and an even row of at most 256 points)} for the shape of one level and kind, process-wide, in
    place of the autotuner's choice (the TMA sweep is no longer used there);
    the next step captures a new step graph. 3D mixed-precision contexts only;
    BFIBM_EINVAL otherwise or for a shape outside those ranges. Same results to

@@ -1,6 +1,6 @@
 """Build libbfibm.so in-tree for sm_103a (GB300) with nvcc.
 
-The three translation units compile in parallel; the shared library lands in
+The translation units compile in parallel; the shared library lands in
 ``paper_1302_3663_gb300/_build/libbfibm.so``. Rebuilds only when a source or
 header is newer than the library.
 """

@@ -436,6 +436,14 @@ __device__ __forceinline__ float psolve(const PSet& c, float ir, float up_d, flo
 // points and room for 3 to 6 rows where 5 to 18 fit (finest viscous sweep of a
 // component, best of the tuner's shapes: 96x96x192 25.7 -> 22.1 us, 144x144x288
 // 98.9 (ring sweep) -> 60.3, 160x160x320 129.6 -> 87, 128x128x256 44.2 -> 43.6).
+// A block may hold 1024 threads (64 registers a thread either way): a long
+// row's tile then has 10 or more rows beside its two ring rows where 512
+// threads hold 4 or 5. Best shapes, 512 against 1024 threads allowed, viscous
+// and pressure: 144x144x288 60.3 -> 58.5 and 53.4 -> 49.3 us, 160x160x320 87.0
+// -> 78.7 and 78.0 -> 66.0; up to 128 points a row the tuner keeps two
+// smaller blocks an SM, which overlap at each other's barriers. The batched
+// forms stay at 512: their blocks pass several members' rows.
+constexpr int kPairThreads = 1024;
 struct PairLane {
   int r, x0;
   bool ok;
@@ -735,10 +743,9 @@ __device__ __forceinline__ void v_rb_pair_body(const Blk& B, const Geo& g, const
 }
 
 template <int d, bool PERZ>
-__global__ void __launch_bounds__(512, 2) k_v_rb_pair(const __grid_constant__ Geo g,
-                                                   const __grid_constant__ LevelPtrs<float> L,
-                                                   float* __restrict__ out, int TY, int KC,
-                                                   float ir) {
+__global__ void __launch_bounds__(kPairThreads, 1)
+    k_v_rb_pair(const __grid_constant__ Geo g, const __grid_constant__ LevelPtrs<float> L,
+                float* __restrict__ out, int TY, int KC, float ir) {
   v_rb_pair_body<d, PERZ>(own_blk(), g, L, out, TY, KC, ir);
 }
 
@@ -971,7 +978,7 @@ __device__ __forceinline__ void p_rb_pair_body(const Blk& B, Geo g, LevelPtrs<fl
 }
 
 template <bool PERZ>
-__global__ void __launch_bounds__(512, 2) k_p_rb_pair(Geo g, LevelPtrs<float> L,
+__global__ void __launch_bounds__(kPairThreads, 1) k_p_rb_pair(Geo g, LevelPtrs<float> L,
                                                    float* __restrict__ out, int TY, int KC,
                                                    float h2) {
   p_rb_pair_body<PERZ>(own_blk(), g, L, out, TY, KC, h2);
@@ -1078,11 +1085,11 @@ int pair_threads(int n0, int TY) {
   return (ne * np + 31) / 32 * 32 + ((nr - ne) * np + 31) / 32 * 32;
 }
 
-// Pair sweep: blocks of at most 512 threads over (row tiles, plane chunks); 3D,
+// Pair sweep: blocks of at most kPairThreads threads over (row tiles, plane chunks); 3D,
 // walls in x and y, an even row of at most 256 points.
 bool pair_eligible(int D, const Geo& g, int TY) {
   if (D != 3 || g.per[0] || g.per[1] || (g.n[0] & 1) || g.n[0] < 4 || g.n[0] > 256) return false;
-  return TY >= 1 && TY <= g.n[1] && pair_threads(g.n[0], TY) <= 512;
+  return TY >= 1 && TY <= g.n[1] && pair_threads(g.n[0], TY) <= kPairThreads;
 }
 
 const void* pair_kernel(int d, bool perz) {

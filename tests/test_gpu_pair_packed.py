@@ -14,6 +14,10 @@ SHAPES = [((48, 40, 20), (18, 5)), ((48, 21, 12), (17, 4)), ((144, 12, 10), (5, 
           ((72, 20, 18), (12, 3)), ((96, 17, 10), (8, 3)), ((160, 9, 8), (4, 3)),
           ((250, 6, 6), (2, 2)), ((4, 20, 8), (18, 3)), ((10, 30, 6), (14, 6))]
 
+# blocks of 960 to 1024 threads, ragged last tiles
+SHAPES += [((144, 30, 10), (12, 4)), ((160, 21, 8), (10, 3)), ((128, 28, 10), (14, 5)),
+           ((250, 13, 6), (6, 3)), ((102, 40, 8), (18, 4))]
+
 
 @pytest.mark.parametrize("n,pair", SHAPES)
 def test_packed_rows_bit_identical_to_ring_sweep(n, pair):
