@@ -332,7 +332,9 @@ __device__ __forceinline__ void v_residual_body(const Blk& B, Geo g, LevelPtrs<T
 // one takes 23 with a plane a block (HBM 15). Pairs of a plane are numbered without gaps along x of the
 // grid, chunks of planes along y (pair_grid). The expressions are those of
 // v_residual_point and p_residual_at.
-constexpr int kVResSM = 2;   // resident blocks of the viscous one
+// Resident blocks of the viscous one: at three (80 registers) fewer of a plane's
+// loads are in flight at once, 85 us instead of 59.
+constexpr int kVResSM = 2;
 struct PairAt {
   int x0, j;
   int dl, dr;        // offsets of the points left (x0 - 1) and right (x0 + 2) of the pair
@@ -669,8 +671,8 @@ __device__ __forceinline__ void prolong_pair_body(const Blk& B, const Geo& gf, c
   if (j >= gf.n[1] || K0 >= K1) return;
   // per axis the cell-centred and, for velocities, the face weights (x: both points)
   constexpr int mir = NC == 3 ? -1 : +1;   // tangential velocities are odd at walls
-  int cxa[2], cxb[2], fxa[2], fxb[2], cy[2], fy[2];
-  T wcxa[2], wcxb[2], wfxa[2], wfxb[2], wcy[2], wfy[2];
+  int cxa[2], cxb[2], fxa[2] = {}, fxb[2] = {}, cy[2], fy[2] = {};
+  T wcxa[2], wcxb[2], wfxa[2] = {}, wfxb[2] = {}, wcy[2], wfy[2] = {};
   prol_cell_1d<T>(2 * I, gc.n[0], gc.per[0], mir, mir, cxa, wcxa);
   prol_cell_1d<T>(2 * I + 1, gc.n[0], gc.per[0], mir, mir, cxb, wcxb);
   prol_cell_1d<T>(j, gc.n[1], gc.per[1], mir, mir, cy, wcy);
