@@ -106,6 +106,7 @@ __host__ __device__ inline int cl_layout(int D, bool V, bool inv, const Geo& g, 
       o += (v.pc + (a == S ? 1 : 0)) * v.PS;
     }
   }
+  for (int d = 0; d < 3; ++d) v.f[d] = v.g[d] = -1;   // not in shared memory
   if (fs)
     for (int d = 0; d < nc; ++d) {
       v.f[d] = o - v.PS;
@@ -130,11 +131,12 @@ __host__ __device__ inline void cl_rank(ClLv& v, int rank) {
 
 // Lays out levels from .. L - 1; returns their bytes (0: they do not fit). The
 // first level keeps its right-hand sides in shared memory where all fits with
-// them (the deeper ones always do, and the FP64 coarsest level of a mixed cycle,
-// which converts its right-hand side into the slab). nd > 0: the coarsest solve
-// is a matrix of nd rows and holds only its right-hand side, from element u[0].
+// them. The deeper ones always do, and so does the coarsest where it is the
+// first and its right-hand side is rewritten in the slab: converted in a mixed
+// cycle, without its mean for the pressure. nd > 0: the coarsest solve is a
+// matrix of nd rows and holds only its right-hand side, from element u[0].
 size_t cl_total(int D, bool fp64, bool V, const Geo* g, int L, int from, int C, int nd, ClLv* lv) {
-  for (int f = 1; f >= (!fp64 && from == L - 1 ? 1 : 0); --f) {
+  for (int f = 1; f >= (from == L - 1 && (!fp64 || !V) ? 1 : 0); --f) {
     size_t b = 0;
     for (int l = from; l < L; ++l) {
       const int el = fp64 || l == L - 1 ? 8 : 4;
