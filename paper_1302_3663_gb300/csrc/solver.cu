@@ -94,8 +94,10 @@ bool has_idg64(const bfibm_params& P, int l, int L) { return P.precision == 0 ||
 // Rows of the coarsest solve's matrix (0: none). Solves to a tolerance run tens
 // of V-cycles on one set of coefficients. A fixed count of at least two gains
 // while the columns run side by side in one wave (their build then takes as long
-// as one solve by sweeps).
-int matrix_rows(const bfibm_params& P, bool V, const Geo& g) {
+// as one solve by sweeps). The matrix is the sweeps from zero: an FP64 context
+// of one level, whose coarsest solve continues from the solution so far, has none.
+int matrix_rows(const bfibm_params& P, bool V, const Geo& g, int L) {
+  if (P.precision == 0 && L == 1) return 0;
   const int n = cl_matrix_rows(P.dim, V, g), vc = V ? P.vc_visc : P.vc_p;
   return vc <= 0 || (vc >= 2 && n <= 384) ? n : 0;
 }
@@ -112,8 +114,10 @@ size_t grid_pool_bytes(const bfibm_params& P, int* nlev = nullptr) {
              (l == 0 && P.precision == 1 ? 2 * P.dim : 0) +
              (has_idg64(P, l, L) ? P.dim + 1 : 0);
     if (l == L - 1)
-      for (int V = 0; V < 2; ++V)
-        bytes += (size_t)round_up(8LL * matrix_rows(P, V, g[l]) * matrix_rows(P, V, g[l]), 256);
+      for (int V = 0; V < 2; ++V) {
+        const long long n = matrix_rows(P, V, g[l], L);
+        bytes += (size_t)round_up(8 * n * n, 256);
+      }
     bytes += arr * na;
     if (P.precision == 1)   // the level's arrays and the inverse viscous diagonals
       bytes += (size_t)round_up(level_elems(g[l]) * 4, 256) * (arrays_per_level(P.dim) + P.dim);
@@ -522,10 +526,14 @@ cudaError_t upload_self(bfibm_ctx* c) {
   const Geos q = geos_of(c);
   const bool fp64 = c->P.precision == 0;
   const int C = cl_max_ctas();
-  c->tail_lev = cl_first_level(c->D, fp64, q.g, c->L, c->tail_cells, C, c->ncm);
+  // The one level of an FP64 context without coarse grids is the problem itself:
+  // its solve takes the mean off the right-hand side that the residual then
+  // reads, so it runs on the global arrays, in one block.
+  const bool none = c->P.open_flow || (fp64 && c->L == 1);
+  c->tail_lev = none ? c->L : cl_first_level(c->D, fp64, q.g, c->L, c->tail_cells, C, c->ncm);
   for (int V = 0; V < 2; ++V) {
     c->cl_smem[0][V] = c->tail_lev < c->L ? cl_bytes(c->D, fp64, V, q.g, c->L, c->tail_lev, C, c->ncm[V]) : 0;
-    c->cl_smem[1][V] = c->P.open_flow ? 0 : cl_bytes(c->D, fp64, V, q.g, c->L, c->L - 1, C, c->ncm[V]);
+    c->cl_smem[1][V] = none ? 0 : cl_bytes(c->D, fp64, V, q.g, c->L, c->L - 1, C, c->ncm[V]);
   }
   if (!c->self_tab) return cudaSuccess;
   BMember B;
@@ -2218,7 +2226,7 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
     }
     if (l == c->L - 1)
       for (int V = 0; V < 2; ++V) {
-        const long long n = c->ncm[V] = matrix_rows(*p, V, Lv.g);
+        const long long n = c->ncm[V] = matrix_rows(*p, V, Lv.g, c->L);
         c->cmat[V] = n ? (double*)cur : nullptr;
         cur += round_up(8 * n * n, 256);
       }

@@ -1,6 +1,7 @@
 """The coarsest level of FP64 contexts against the oracle: levels that only
 just fit the cluster kernel's shared memory (csrc/cluster.cu), which
-test_cluster_layout.py looks at on the CPU."""
+test_cluster_layout.py looks at on the CPU, and contexts whose coarsest level is
+their only one, where each solve continues from the one before."""
 import numpy as np
 import pytest
 
@@ -50,4 +51,31 @@ def solve_and_compare(g, o, cycles):
 def test_coarsest_levels_at_the_edge_of_shared_memory(n, per):
     g, o = contexts(n, per, 21)
     solve_and_compare(g, o, 2)
+    g.close()
+
+
+# grids that cannot be halved (an odd half of a periodic axis), and one kept at one level; up to
+# 800 unknowns a solve (a matrix's rows in deeper contexts) and more
+ONE_LEVEL = [((22, 16), (1, 0), 6), ((14, 12), (1, 0), 6), ((6, 6, 6), (0, 0, 1), 6),
+             ((7, 10, 4), (0, 0, 1), 6), ((8, 8, 16), (0, 0, 1), 1), ((32, 24), (1, 0), 1)]
+
+
+@pytest.mark.parametrize("cycles", [3, 30])
+@pytest.mark.parametrize("n,per,levels", ONE_LEVEL)
+def test_one_level_continues_from_its_iterate(n, per, levels, cycles):
+    g, o = contexts(n, per, 22, mg_levels_max=levels)
+    assert g.levels == 1
+    solve_and_compare(g, o, cycles)
+    # the mean is taken off the right-hand side itself, which the residual reads
+    assert_close(g.get_field("prhs"), o.get("prhs"), TOL, "prhs")
+    g.close()
+
+
+@pytest.mark.parametrize("n,per,levels", ONE_LEVEL)
+def test_one_level_reaches_a_tolerance(n, per, levels):
+    g, _ = contexts(n, per, 23, mg_levels_max=levels, vc_visc=0, vc_p=0, rtol=1e-6,
+                    max_cycles=1000)
+    for solve, which in ((g.solve_viscous, "res_visc"), (g.solve_pressure, "res_p")):
+        assert 0 < solve(0) < 1000
+        assert g.get_stats()[which] <= 1e-6
     g.close()
