@@ -57,8 +57,8 @@ __device__ __forceinline__ int cl_div(int q, unsigned m, int d) {
   return d == 1 ? q : (int)__umulhi((unsigned)q, m);
 }
 
-// Lays a level out from element `base`; returns the end. INV: inverse
-// diagonals are kept for the pressure too (FP64).
+// Lays a level out from element `base`; returns the end. inv: inverse
+// diagonals are kept for the pressure too, and in two parts (FP64).
 __host__ __device__ inline int cl_layout(int D, bool V, bool inv, const Geo& g, int C, int fs,
                                          int base, ClLv& v) {
   const int S = D - 1;
@@ -106,13 +106,17 @@ __host__ __device__ inline int cl_layout(int D, bool V, bool inv, const Geo& g, 
       o += (v.pc + (a == S ? 1 : 0)) * v.PS;
     }
   }
-  for (int d = 0; d < 3; ++d) v.f[d] = v.g[d] = -1;   // not in shared memory
+  for (int d = 0; d < 3; ++d) v.f[d] = v.g[d] = v.gl[d] = -1;   // not in shared memory
   if (fs)
     for (int d = 0; d < nc; ++d) {
       v.f[d] = o - v.PS;
       o += v.pc * v.PS;
       if (V || inv) {
         v.g[d] = o - v.PS;
+        o += v.pc * v.PS;
+      }
+      if (inv) {
+        v.gl[d] = o - v.PS;
         o += v.pc * v.PS;
       }
     }
@@ -254,7 +258,8 @@ __device__ __forceinline__ void cl_colour(const ClLv& v, int colour, F&& f) {
 // v_red and p_red (point.cuh) on the slab: u_d at its new value
 template <int D, int d, typename T>
 __device__ __forceinline__ T cl_v_update(const ClLv& v, const T* __restrict__ sm,
-                                         const ClPt<D>& q, int own, int opp, T f, T idg, T ir) {
+                                         const ClPt<D>& q, int own, int opp, T f, T idg, T idl,
+                                         T ir) {
   const int dmd = q.dm[d];
   const T* ud = sm + v.u[d];
   const T mcp = sm[v.c + own], mcm = sm[v.c + opp + dmd];
@@ -281,7 +286,8 @@ __device__ __forceinline__ T cl_v_update(const ClLv& v, const T* __restrict__ sm
     if (!q.wm[e]) off = pfma(cem[n], ud[opp + q.dm[e]], off);
     ++n;
   }
-  return pmul(pfma(ir, off, f), idg);
+  if constexpr (sizeof(T) == 4) return pmul(pfma(ir, off, f), idg);
+  else return pt_quot(pfma(ir, off, f), idg, idl);
 }
 
 template <int D, typename T>
@@ -309,7 +315,8 @@ __device__ __forceinline__ void cl_p_terms(const ClLv& v, const T* __restrict__ 
 // one colour of component d, or of the pressure; coef: ir or h^2
 template <int D, int d, typename T, bool PER>
 __device__ __forceinline__ void cl_v_phase(const ClLv& v, const T* __restrict__ f,
-                                           const T* __restrict__ g, int colour, T ir) {
+                                           const T* __restrict__ g, const T* __restrict__ gl,
+                                           int colour, T ir) {
   T* sm = cl_sm<T>();
   cl_colour(v, colour, [&](int h, int par, int r, int lp) {
     ClPt<D> q;
@@ -318,14 +325,17 @@ __device__ __forceinline__ void cl_v_phase(const ClLv& v, const T* __restrict__ 
     const int own = q.b + (colour ? v.CP : 0), opp = q.b + (colour ? 0 : v.CP);
     const T fv = v.fs ? sm[v.f[d] + own] : __ldg(f + cl_F(v, q));
     const T gv = v.fs ? sm[v.g[d] + own] : __ldg(g + cl_F(v, q));
-    cl_put(v, sm, v.u[d] + own, lp, cl_v_update<D, d, T>(v, sm, q, own, opp, fv, gv, ir));
+    T lv = T(0);
+    if constexpr (sizeof(T) == 8) lv = v.fs ? sm[v.gl[d] + own] : __ldg(gl + cl_F(v, q));
+    cl_put(v, sm, v.u[d] + own, lp, cl_v_update<D, d, T>(v, sm, q, own, opp, fv, gv, lv, ir));
   });
   cl_phase_sync(v);
 }
 
 template <int D, typename T, bool PER>
 __device__ __forceinline__ void cl_p_phase(const ClLv& v, const T* __restrict__ f,
-                                           const T* __restrict__ g, int colour, T h2) {
+                                           const T* __restrict__ g, const T* __restrict__ gl,
+                                           int colour, T h2) {
   T* sm = cl_sm<T>();
   cl_colour(v, colour, [&](int h, int par, int r, int lp) {
     ClPt<D> q;
@@ -336,7 +346,8 @@ __device__ __forceinline__ void cl_p_phase(const ClLv& v, const T* __restrict__ 
     cl_p_terms<D, T>(v, sm, q, own, opp, num, dg);
     T pv;
     if constexpr (sizeof(T) == 4) pv = px_final(num, dg, h2, fv);
-    else pv = pmul(pfma(-h2, fv, num), v.fs ? sm[v.g[0] + own] : __ldg(g + cl_F(v, q)));
+    else pv = pt_quot(pfma(-h2, fv, num), v.fs ? sm[v.g[0] + own] : __ldg(g + cl_F(v, q)),
+                      v.fs ? sm[v.gl[0] + own] : __ldg(gl + cl_F(v, q)));
     cl_put(v, sm, v.u[0] + own, lp, pv);
   });
   cl_phase_sync(v);
@@ -347,12 +358,15 @@ __device__ __forceinline__ void cl_smooth(const ClLv& v, const LevelPtrs<T>& L, 
   if (v.C == 1 && v.npl == 0) return;   // the first CTA's level
   for (int it = 0; it < n; ++it) {
     if constexpr (V) {
-      for (int c = 0; c < 2; ++c) cl_v_phase<D, 0, T, PER>(v, L.uf[0], L.idg[0], c, coef);
-      for (int c = 0; c < 2; ++c) cl_v_phase<D, 1, T, PER>(v, L.uf[1], L.idg[1], c, coef);
+      for (int c = 0; c < 2; ++c)
+        cl_v_phase<D, 0, T, PER>(v, L.uf[0], L.idg[0], L.idl[0], c, coef);
+      for (int c = 0; c < 2; ++c)
+        cl_v_phase<D, 1, T, PER>(v, L.uf[1], L.idg[1], L.idl[1], c, coef);
       if constexpr (D == 3)
-        for (int c = 0; c < 2; ++c) cl_v_phase<D, 2, T, PER>(v, L.uf[2], L.idg[2], c, coef);
+        for (int c = 0; c < 2; ++c)
+          cl_v_phase<D, 2, T, PER>(v, L.uf[2], L.idg[2], L.idl[2], c, coef);
     } else {
-      for (int c = 0; c < 2; ++c) cl_p_phase<D, T, PER>(v, L.pf, L.pdg, c, coef);
+      for (int c = 0; c < 2; ++c) cl_p_phase<D, T, PER>(v, L.pf, L.pdg, L.pdl, c, coef);
     }
   }
 }
@@ -496,7 +510,7 @@ __device__ __forceinline__ void cl_load(const ClLv& v, const Geo& g, const Level
   if (v.npl == 0) return;
   const int np = (v.npl + 2) * v.sR * v.s0;
   for (int q0 = threadIdx.x; q0 < np; q0 += UN * blockDim.x) {
-    TC u[UN][nc], c[UN], e[UN][ne], f[UN][nc], gi[UN][nc];
+    TC u[UN][nc], c[UN], e[UN][ne], f[UN][nc], gi[UN][nc], gl[UN][nc];
     int idx[UN], lpn[UN];
 #pragma unroll
     for (int n = 0; n < UN; ++n) {
@@ -521,6 +535,7 @@ __device__ __forceinline__ void cl_load(const ClLv& v, const Geo& g, const Level
         f[n][d] = own && first ? (TC)(V ? F.uf[d] : F.pf)[o] : TC(0);
         if constexpr (V) gi[n][d] = own ? __ldg(L.idg[d] + o) : TC(0);
         else if constexpr (sizeof(TC) == 8) gi[n][d] = own ? __ldg(L.pdg + o) : TC(0);
+        if constexpr (sizeof(TC) == 8) gl[n][d] = own ? __ldg((V ? L.idl[d] : L.pdl) + o) : TC(0);
       }
     }
 #pragma unroll
@@ -541,6 +556,7 @@ __device__ __forceinline__ void cl_load(const ClLv& v, const Geo& g, const Level
         for (int d = 0; d < nc; ++d) {
           if (first) sm[v.f[d] + x] = f[n][d];
           if constexpr (V || sizeof(TC) == 8) sm[v.g[d] + x] = gi[n][d];
+          if constexpr (sizeof(TC) == 8) sm[v.gl[d] + x] = gl[n][d];
         }
       }
     }

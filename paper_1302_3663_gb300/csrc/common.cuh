@@ -47,6 +47,8 @@ struct LevelPtrs {
   T* u2[3];      // second buffers of u
   T* idg[3];     // 1 / diagonal of the viscous operator of component d
   T* pdg;        // FP64: 1 / (sum of beta) of the pressure operator
+  T* idl[3];     // FP64: what the rounding of idg and pdg left out (pt_quot)
+  T* pdl;
 };
 
 struct Ptr3d {
@@ -162,6 +164,7 @@ struct ClLv {
   int st1, st2;              // strides of the global arrays: row, plane
   int fs;                    // right-hand sides and inverse diagonals are in shared memory
   int u[3], f[3], g[3], c, e[3];
+  int gl[3];                 // FP64: the low parts of the inverse diagonals
 };
 
 // ------------------------------------------------------- batched launches
@@ -505,7 +508,7 @@ bool tma_chosen(int K, const Geo& g);
 bool tma_plan_of(int K, const Geo& g, int out[5]);
 
 // FP64-only grid stages.
-// L.idg and L.pdg from the level's coefficients
+// L.idg, L.pdg and their low parts from the level's coefficients
 void launch_idg64(int D, const Geo& g, const LevelPtrs<double>& L, double inv_re, cudaStream_t s);
 void launch_coef_fine(int D, const Geo& g, double* const rho[3], double* beta[3], double* m[3],
                       double msc, double rho_f, cudaStream_t s);

@@ -112,7 +112,7 @@ size_t grid_pool_bytes(const bfibm_params& P, int* nlev = nullptr) {
     // flexible-CG vectors p and q
     int na = arrays_per_level(P.dim) + (l == 0 ? 3 * P.dim : 0) +
              (l == 0 && P.precision == 1 ? 2 * P.dim : 0) +
-             (has_idg64(P, l, L) ? P.dim + 1 : 0);
+             (has_idg64(P, l, L) ? 2 * (P.dim + 1) : 0);
     if (l == L - 1)
       for (int V = 0; V < 2; ++V) {
         const long long n = matrix_rows(P, V, g[l], L);
@@ -2221,8 +2221,12 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
     d.muc = take(Lv.g);
     for (int e = 0; e < E; ++e) d.mue[e] = take(Lv.g);
     if (has_idg64(*p, l, c->L)) {
-      for (int a = 0; a < D; ++a) d.idg[a] = take(Lv.g);
+      for (int a = 0; a < D; ++a) {
+        d.idg[a] = take(Lv.g);
+        d.idl[a] = take(Lv.g);
+      }
       d.pdg = take(Lv.g);
+      d.pdl = take(Lv.g);
     }
     if (l == c->L - 1)
       for (int V = 0; V < 2; ++V) {

@@ -149,10 +149,11 @@ __device__ __forceinline__ void p_terms(const Geo& g, const LevelPtrs<T>& L, con
 // numbered without gaps along blockIdx.x (an FP64 instruction costs the same
 // for one lane as for 32, and a row seldom fills whole warps), planes along
 // blockIdx.y. nh: points per row, mnh = ceil(2^32 / nh).
-// INV: multiply by the inverse diagonal (L.idg, L.pdg) instead of forming the
-// diagonal and dividing. The sweeps are bound by the FP64 rate: about 20
-// operations per viscous point instead of 40, 8 instead of 26 for the pressure.
-// Three sweeps of both systems on a 101x75x130 grid: 1165 -> 669 us.
+// INV: multiply by the inverse diagonal in two parts (L.idg, L.idl; L.pdg,
+// L.pdl) instead of forming the diagonal and dividing. The sweeps are bound by the
+// FP64 rate: about 21 operations per viscous point instead of 40, 9 instead of 26
+// for the pressure. Three sweeps of both systems on a 101x75x130 grid:
+// 1165 -> 706 us (661 with the rounded inverse alone).
 // f(i, j, k) for the thread's points of e0 x e1 x e2 of one colour
 template <class F>
 __device__ __forceinline__ void colour_points(int nh, unsigned mnh, int e0, int e1, int e2,
@@ -177,7 +178,7 @@ __global__ void __launch_bounds__(256) k_p_rbgs(Geo g, LevelPtrs<T> L, int colou
     const long long c = gidx(g, i, j, k);
     T num, dg;
     p_terms<D, T>(g, L, ci, c, num, dg);
-    if constexpr (INV) L.p[c] = pmul(pfma(-h2, L.pf[c], num), L.pdg[c]);
+    if constexpr (INV) L.p[c] = pt_quot(pfma(-h2, L.pf[c], num), L.pdg[c], L.pdl[c]);
     else L.p[c] = (num - h2 * L.pf[c]) / dg;
   });
 }
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(256) k_v_rbgs(Geo g, LevelPtrs<T> L, int colou
     const long long F = gidx(g, i, j, k);
     T off, dgV;
     v_terms<D, d, T>(g, L, ci, F, off, dgV);
-    if constexpr (INV) L.u[d][F] = pmul(pfma(ir, off, L.uf[d][F]), L.idg[d][F]);
+    if constexpr (INV) L.u[d][F] = pt_quot(pfma(ir, off, L.uf[d][F]), L.idg[d][F], L.idl[d][F]);
     else L.u[d][F] = (L.uf[d][F] + ir * off) / (L.m[d][F] + ir * dgV);
   });
 }
@@ -956,19 +957,21 @@ __global__ void __launch_bounds__(1024) k_coarse_v(Geo g, LevelPtrs<T> Lg, int s
 }
 
 // 1 / diagonal of both FP64 operators on every unknown of a level (0 on the
-// fixed wall faces), formed once when the coefficients change: an FP64
-// division and the diagonal's sums cost as much as the rest of an update.
+// fixed wall faces), in two parts, formed once when the coefficients change: an
+// FP64 division and the diagonal's sums cost as much as the rest of an update.
 template <int D, int d>
 __device__ __forceinline__ void idg64_point(const Geo& g, const LevelPtrs<double>& L,
                                             const int ci[3], long long F, double ir) {
   if (beyond_outflow<d>(g, ci)) return;
-  double v = 0.0;
+  double v = 0.0, dg = 0.0;
   if (g.per[d] || ci[d] != 0) {
     double off, dgV;
     v_terms<D, d, double>(g, L, ci, F, off, dgV);
-    v = 1.0 / (L.m[d][F] + ir * dgV);
+    dg = L.m[d][F] + ir * dgV;
+    v = 1.0 / dg;
   }
   L.idg[d][F] = v;
+  L.idl[d][F] = pt_low(dg, v);
 }
 template <int D>
 __global__ void __launch_bounds__(256) k_idg64(Geo g, LevelPtrs<double> L, double ir) {
@@ -985,7 +988,9 @@ __global__ void __launch_bounds__(256) k_idg64(Geo g, LevelPtrs<double> L, doubl
   if (i < g.n[0] && j < g.n[1] && k < g.n[2]) {
     double num, dg;
     p_terms<D, double>(g, L, ci, F, num, dg);
-    L.pdg[F] = 1.0 / dg;
+    const double v = 1.0 / dg;
+    L.pdg[F] = v;
+    L.pdl[F] = pt_low(dg, v);
   }
 }
 

@@ -26,7 +26,8 @@ class ClLv(ctypes.Structure):
                 [(f, ctypes.c_uint) for f in "mnh mR ms0 msR".split()] +
                 [(f, ctypes.c_int) for f in "C pc na last k0 npl lo hi nlo per0 perR perS "
                  "st1 st2 fs".split()] +
-                [("u", I3), ("f", I3), ("g", I3), ("c", ctypes.c_int), ("e", I3)])
+                [("u", I3), ("f", I3), ("g", I3), ("c", ctypes.c_int), ("e", I3),
+                 ("gl", I3)])
 
 
 def cl_bytes():
@@ -103,8 +104,10 @@ def check(lv, D, fp64, V, L, start, total):
                 add(v.f[d], 1, v.pc)
                 if V or el == 8:
                     add(v.g[d], 1, v.pc)
+                if el == 8:
+                    add(v.gl[d], 1, v.pc)
         else:
-            assert l == start and set(v.f) | set(v.g) == {-1}
+            assert l == start and set(v.f) | set(v.g) | set(v.gl) == {-1}
         # the kernel writes these right-hand sides: the restricted one below the first level,
         # the converted one of a mixed cycle, the pressure's without its mean
         if l > start or (l == L - 1 and (not V or not fp64)):
