@@ -157,11 +157,9 @@ __global__ void __launch_bounds__(256) k_v_idg32(Geo g, LevelPtrs<double> L, F32
       if (d == 0) dg = v_diag64<D, 0>(g, L, ci, F, ir);
       else if (d == 1) dg = v_diag64<D, 1>(g, L, ci, F, ir);
       else dg = v_diag64<D, (D == 3 ? 2 : 1)>(g, L, ci, F, ir);
-      // 1 / dg to about 46 bits, more than the rounding to FP32 keeps: an FP32
-      // reciprocal and one FP64 Newton step instead of an FP64 division
-      const float r0 = 1.0f / (float)dg;
-      const double r = (double)r0;
-      v = (float)fma(r, fma(-dg, r, 1.0), r);
+      // (divided in FP64: an FP32 reciprocal and one Newton step have about 46
+      // bits, too few beside a tie of the rounding to FP32, and no range beyond it)
+      v = (float)(1.0 / dg);
     }
     idg.a[d][F] = v;
   }
