@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <cmath>
+
 #include "common.cuh"
 #include "point.cuh"
 #include "transfer.cuh"
@@ -1186,21 +1188,36 @@ __global__ void __launch_bounds__(256) k_adv_rhs(Geo g, Ptr3 uv, Ptr3 rho, Ptr3 
 // ---------------------------------------------------------------------------
 // Divergence, projection and reductions.
 // ---------------------------------------------------------------------------
-// a / h from the correctly rounded ih = 1 / h and one correction of the quotient
-// by its exact remainder: the rounding of a division in 3 FP64 operations
-// instead of about 10 (GB300's FP64 rate bounds these passes).
-__device__ __forceinline__ double over_h(double a, double h, double ih) {
-  const double q = a * ih;
-  if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;   // infinite or NaN: as it is
-  return fma(fma(-q, h, a), ih, q);
+// a / h by 1 / h in two parts (pt_quot): the rounding of a division in 2 FP64
+// operations instead of about 10 (GB300's FP64 rate bounds these passes). hi is
+// NaN where h or its inverse leaves the range in which the low part is exact.
+struct Rcp {
+  double h, hi, lo;
+};
+Rcp rcp_of(double h) {
+  Rcp r;
+  r.h = h;
+  r.hi = h > 1e-250 && h < 1e250 ? 1.0 / h : std::nan("");
+  r.lo = std::fma(-h, r.hi, 1.0) * r.hi;
+  return r;
+}
+__device__ __noinline__ double over_h_div(double a, double h) { return a / h; }
+__device__ __forceinline__ double over_h(double a, const Rcp& r) {
+  const double q = pt_quot(a, r.hi, r.lo);
+  // quotients below 2^-900, where a * lo underflows, infinities and NaN are
+  // divided; a zero is its own quotient (zeros are common: fluid at rest)
+  const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 2047u;
+  if (e - 123u < 1920u) return q;
+  if (a == 0.0) return a;
+  return over_h_div(a, r.h);
 }
 
 template <int D>
 __device__ __forceinline__ double div_at(const Geo& g, const Ptr3& u, const int ci[3],
-                                         long long c, double ih) {
+                                         long long c, const Rcp& ih) {
   double s = 0.0;
 #pragma unroll
-  for (int a = 0; a < D; ++a) s += over_h(u.a[a][c + offp(g, a, ci[a])] - u.a[a][c], g.h, ih);
+  for (int a = 0; a < D; ++a) s += over_h(u.a[a][c + offp(g, a, ci[a])] - u.a[a][c], ih);
   return s;
 }
 
@@ -1208,9 +1225,8 @@ template <int D>
 __global__ void __launch_bounds__(256) k_divergence(Geo g, Ptr3 u, double* __restrict__ b,
                                                     double scale, double* __restrict__ partial,
                                                     const double* __restrict__ beta_open,
-                                                    double pbc) {
+                                                    double pbc, const __grid_constant__ Rcp ih) {
   __shared__ double sh[32];
-  const double ih = 1.0 / g.h;
   long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
   double acc = 0.0;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ncell;
@@ -1283,8 +1299,8 @@ __global__ void __launch_bounds__(256) k_sub_scalar(Geo g, double* __restrict__ 
 // below the face along d. One function for the face a thread owns and for
 // the upper faces it recomputes, so both round alike.
 __device__ __forceinline__ double proj_face(double ut, double beta, double pF, double pM,
-                                            double coef, double h, double ih) {
-  return ut - coef * beta * over_h(pF - pM, h, ih);
+                                            double coef, const Rcp& ih) {
+  return ut - coef * beta * over_h(pF - pM, ih);
 }
 
 // Projection, Eq. (NSdis2), with the check of Eq. (NSdis4) fused in: each
@@ -1297,7 +1313,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* __restrict__ p,
                                                  Ptr3 beta, Ptr3 uv, double coef,
                                                  unsigned long long* __restrict__ divacc,
-                                                 double p_out, double ih) {
+                                                 double p_out, const __grid_constant__ Rcp ih) {
   __shared__ double sh[32];
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1315,7 +1331,7 @@ __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* _
       if (beyond) {
         long long F = gidx(g, i, j, k);
         const double pm = p[F - g.st[o]];
-        uv.a[o][F] = proj_face(ut.a[o][F], beta.a[o][F], 2.0 * p_out - pm, pm, coef, g.h, ih);
+        uv.a[o][F] = proj_face(ut.a[o][F], beta.a[o][F], 2.0 * p_out - pm, pm, coef, ih);
       }
     }
   }
@@ -1332,18 +1348,18 @@ __global__ void __launch_bounds__(256) k_project(Geo g, Ptr3 ut, const double* _
         lo = ut.a[d][F];
         uv.a[d][F] = lo;
       } else {
-        lo = proj_face(ut.a[d][F], beta.a[d][F], pF, p[F + offm(g, d, ci[d])], coef, g.h, ih);
+        lo = proj_face(ut.a[d][F], beta.a[d][F], pF, p[F + offm(g, d, ci[d])], coef, ih);
         uv.a[d][F] = lo;
       }
       double hi = 0.0;   // the upper wall face holds 0
       if (g.per[d] || ci[d] != g.n[d] - 1) {
         long long Fu = F + offp(g, d, ci[d]);
-        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], p[Fu], pF, coef, g.h, ih);
+        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], p[Fu], pF, coef, ih);
       } else if (is_open(g, d)) {   // the outflow face: ghost 2 p_out - p
         long long Fu = F + st_of(g, d);
-        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], 2.0 * p_out - pF, pF, coef, g.h, ih);
+        hi = proj_face(ut.a[d][Fu], beta.a[d][Fu], 2.0 * p_out - pF, pF, coef, ih);
       }
-      s += over_h(hi - lo, g.h, ih);
+      s += over_h(hi - lo, ih);
     }
     mx = fabs(s);
     if (!(mx <= CUDART_INF)) mx = CUDART_INF;
@@ -1415,9 +1431,9 @@ __global__ void __launch_bounds__(256) k_norm2(Geo g, Ptr3 a, int ncomp,
 
 template <int D>
 __global__ void __launch_bounds__(256) k_div_ke(Geo g, Ptr3 u, double* __restrict__ pmax,
-                                                double* __restrict__ psum) {
+                                                double* __restrict__ psum,
+                                                const __grid_constant__ Rcp ih) {
   __shared__ double sh[32];
-  const double ih = 1.0 / g.h;
   long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
   double mx = 0.0, acc = 0.0;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ncell;
@@ -2027,8 +2043,9 @@ void launch_divergence(int D, const Geo& g, double* const u[3], double* b, doubl
   long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
   int nb = red_grid(ncell);
   const double pbc = 2.0 * p_out / (g.h * g.h);
-  if (D == 3) k_divergence<3><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), b, scale, sc.partial, beta_open, pbc);
-  else k_divergence<2><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), b, scale, sc.partial, beta_open, pbc);
+  const Rcp ih = rcp_of(g.h);
+  if (D == 3) k_divergence<3><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), b, scale, sc.partial, beta_open, pbc, ih);
+  else k_divergence<2><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), b, scale, sc.partial, beta_open, pbc, ih);
   if (g.open >= 0) return;   // a regular problem: the mean stays
   k_finalize<<<1, 1024, 0, s>>>(sc.partial, nb, sc.out, 0, 1.0 / (double)ncell, 0);
   dim3 bb = blk3(D);
@@ -2050,10 +2067,11 @@ void launch_project(int D, const Geo& g, double* const ut[3], const double* p,
   dim3 b = blk3(D);
   dim3 gr = grd3(ext(g, 0, true), ext(g, 1, true), ext(g, 2, true), b);
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(dc.out + dc.acc);
+  const Rcp ih = rcp_of(g.h);
   if (D == 3)
-    k_project<3><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, 1.0 / g.h);
+    k_project<3><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, ih);
   else
-    k_project<2><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, 1.0 / g.h);
+    k_project<2><<<gr, b, 0, s>>>(g, ptr3(ut), p, ptr3(beta), ptr3(uvel), coef, acc, dc.p_out, ih);
   k_div_check<<<1, 32, 0, s>>>(dc.out, dc.acc, dc.step, dc.all, dc.tol, dc.viol);
 }
 
@@ -2071,8 +2089,9 @@ void launch_div_ke(int D, const Geo& g, double* const u[3], Scalars sc, int slot
   int nb = red_grid(ncell);
   double* pmax = sc.partial;
   double* psum = sc.partial + kRedBlocks;
-  if (D == 3) k_div_ke<3><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), pmax, psum);
-  else k_div_ke<2><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), pmax, psum);
+  const Rcp ih = rcp_of(g.h);
+  if (D == 3) k_div_ke<3><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), pmax, psum, ih);
+  else k_div_ke<2><<<nb, kBlock1D, 0, s>>>(g, ptr3(u), pmax, psum, ih);
   double hD = D == 3 ? g.h * g.h * g.h : g.h * g.h;
   k_finalize<<<1, 1024, 0, s>>>(pmax, nb, sc.out, slot, 1.0, 1);
   k_finalize<<<1, 1024, 0, s>>>(psum, nb, sc.out, slot + 1, hD, 0);
