@@ -236,6 +236,8 @@ struct bfibm_ctx {
                                  // the tuner timed them faster, 2 wherever a level allows
   bool collect_stats = true;
   bool dirty = true;
+  bool stale[kMaxLevels] = {};    // the level's inverse diagonals (and matrices) are older than
+                                  // its coefficients: formed again before the next use
   int poisoned = 0;
   long long step_host = 0;
   int inner = 1;                 // FP32 V-cycles per FP64 defect-correction iteration
@@ -1054,6 +1056,15 @@ void inverse_diagonals(bfibm_ctx* c, int l) {
                              c->ncm[V], c->stream);
 }
 
+// Before a sweep or a cycle: what coefficients set by hand made stale. (Formed
+// in each set, one field of 97x97x96 points took 107 us instead of 21 and one of a
+// coarsest level with matrices 399 instead of 12, up to ten times over.)
+void refresh_inverses(bfibm_ctx* c) {
+  for (int l = 0; l < c->L; ++l)
+    if (c->stale[l]) inverse_diagonals(c, l);
+  std::memset(c->stale, 0, sizeof(c->stale));
+}
+
 void build_coefficients(bfibm_ctx* c) {
   Level& L0 = c->lev[0];
   launch_coef_fine(c->D, L0.g, c->rho, L0.d.beta, L0.d.m, c->P.sigma / c->P.dt, c->P.rho_f,
@@ -1129,8 +1140,10 @@ bfibm_status ensure_ready(bfibm_ctx* c) {
   if (c->dirty) {
     refresh(c);
     c->dirty = false;
-    CK(cudaGetLastError());
+    std::memset(c->stale, 0, sizeof(c->stale));   // (not in refresh: a step graph's capture runs it)
   }
+  refresh_inverses(c);
+  CK(cudaGetLastError());
   return BFIBM_OK;
 }
 
@@ -1280,12 +1293,9 @@ bfibm_status copy_field(bfibm_ctx* c, int which, int comp, int level, void* ext,
     CK(cudaMemcpy2DAsync(ext, row, p, pitch, row, rows, kind, c->stream));
   else
     CK(cudaMemcpy2DAsync(p, pitch, ext, row, row, rows, kind, c->stream));
-  // the inverse diagonals follow their coefficients
   if (!to_ext &&
-      (which == BFIBM_F_BETA || which == BFIBM_F_M || which == BFIBM_F_MUC || which == BFIBM_F_MUE)) {
-    inverse_diagonals(c, level);
-    CK(cudaGetLastError());
-  }
+      (which == BFIBM_F_BETA || which == BFIBM_F_M || which == BFIBM_F_MUC || which == BFIBM_F_MUE))
+    c->stale[level] = true;
   CK(cudaStreamSynchronize(c->stream));
   return BFIBM_OK;
 }
@@ -2656,6 +2666,7 @@ bfibm_status bfibm_refresh(bfibm_ctx* c) {
   READY(c);
   refresh(c);
   c->dirty = false;
+  std::memset(c->stale, 0, sizeof(c->stale));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->stream));
   return BFIBM_OK;
@@ -2664,6 +2675,7 @@ bfibm_status bfibm_refresh(bfibm_ctx* c) {
 bfibm_status bfibm_build_coefficients(bfibm_ctx* c) {
   READY(c);
   build_coefficients(c);
+  std::memset(c->stale, 0, sizeof(c->stale));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->stream));
   return BFIBM_OK;
@@ -2686,6 +2698,7 @@ bfibm_status bfibm_stage(bfibm_ctx* c, int stage) {
 
 bfibm_status bfibm_solve_pressure(bfibm_ctx* c, int ncycles, int32_t* cycles) {
   READY(c);
+  refresh_inverses(c);
   int used = 0;
   bfibm_status st = c->P.precision == 1 ? solve_p_mixed(c, ncycles, &used)
                                         : solve_p(c, ncycles, &used);
@@ -2707,6 +2720,7 @@ bfibm_status bfibm_set_gamma(bfibm_ctx* c, const double gamma_levels[8]) {
   drop_graph(c);
   for (int l = 0; l < 8; ++l) c->P.gamma_levels[l] = gamma_levels[l];
   build_coefficients(c);
+  std::memset(c->stale, 0, sizeof(c->stale));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->stream));
   return BFIBM_OK;
@@ -2714,6 +2728,7 @@ bfibm_status bfibm_set_gamma(bfibm_ctx* c, const double gamma_levels[8]) {
 
 bfibm_status bfibm_solve_viscous(bfibm_ctx* c, int ncycles, int32_t* cycles) {
   READY(c);
+  refresh_inverses(c);
   int used = 0;
   bfibm_status st = c->P.precision == 1 ? (c->krylov ? solve_v_fcg(c, ncycles, &used)
                                                      : solve_v_mixed(c, ncycles, &used))
@@ -2729,6 +2744,7 @@ bfibm_status bfibm_solve_viscous(bfibm_ctx* c, int ncycles, int32_t* cycles) {
 bfibm_status bfibm_smooth_pressure(bfibm_ctx* c, int level, int nsweeps) {
   READY(c);
   if (level < 0 || level >= c->L || nsweeps < 0) return set_err(c, BFIBM_EINVAL, "bad level");
+  refresh_inverses(c);
   smooth_p(c, level, nsweeps);
   CK(cudaGetLastError());
   return BFIBM_OK;
@@ -2737,6 +2753,7 @@ bfibm_status bfibm_smooth_pressure(bfibm_ctx* c, int level, int nsweeps) {
 bfibm_status bfibm_smooth_viscous(bfibm_ctx* c, int level, int nsweeps) {
   READY(c);
   if (level < 0 || level >= c->L || nsweeps < 0) return set_err(c, BFIBM_EINVAL, "bad level");
+  refresh_inverses(c);
   smooth_v(c, level, nsweeps);
   CK(cudaGetLastError());
   return BFIBM_OK;
