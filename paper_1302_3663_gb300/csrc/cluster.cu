@@ -809,8 +809,6 @@ void launch_coarse_matrix(int D, bool viscous, const Geo& g, const LevelPtrs<dou
 }
 
 int cl_max_ctas() {
-  static int c = 0;
-  if (c) return c;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(16);
   cfg.blockDim = dim3(kClThreads);
@@ -824,7 +822,7 @@ int cl_max_ctas() {
   int n = 0;
   const bool ok = cudaOccupancyMaxActiveClusters(&n, cl_kernel(3, false, true, true), &cfg) == cudaSuccess;
   if (!ok) cudaGetLastError();
-  return c = ok && n >= 1 ? 16 : 8;
+  return ok && n >= 1 ? 16 : 8;
 }
 
 cudaError_t cl_setup() {

@@ -478,7 +478,7 @@ int cl_first_level(int D, bool fp64, const Geo* g, int L, long long cells, int C
 int cl_matrix_rows(int D, bool viscous, const Geo& g);
 void launch_coarse_matrix(int D, bool viscous, const Geo& g, const LevelPtrs<double>& L, int sweeps,
                           double inv_re, double* B, int n, cudaStream_t s);
-int cl_max_ctas();   // the largest cluster this device schedules: 16 or 8
+int cl_max_ctas();   // the largest cluster the current device schedules: 16 or 8 (after cl_setup)
 cudaError_t cl_setup();
 
 // ---------------------------------------------------------------- smooth_tma.cu

@@ -251,6 +251,7 @@ struct bfibm_ctx {
   long long tail_cells = kTailCells32;   // BFIBM_OPT_TAIL: V-cycle levels of at most this many
                                   // cells run in the cluster V-cycle (0: none)
   int tail_lev = kMaxLevels;      // the first of them (L: none)
+  int cl_ctas = 8;                // CTAs of its cluster: as many as the device schedules
   size_t cl_smem[2][2] = {};      // its shared memory: [from the tail, the coarsest level alone]
                                   // [pressure, viscous] (0: it does not fit)
   double* cmat[2] = {nullptr, nullptr};   // the coarsest solve as a matrix: pressure, viscous
@@ -381,7 +382,7 @@ bool cluster_per(const bfibm_ctx* c) {
 bool cluster_cycle(bfibm_ctx* c, int l, bool V) {
   if (l != c->tail_lev) return false;
   launch_cluster(c->D, c->P.precision == 0, V, cluster_per(c), c->self_tab, c->self_list, 1, nullptr,
-                 false, cl_max_ctas(), c->cl_smem[0][V], c->stream);
+                 false, c->cl_ctas, c->cl_smem[0][V], c->stream);
   return true;
 }
 
@@ -391,7 +392,7 @@ void coarse_solve(bfibm_ctx* c, bool V) {
   Level& Lv = c->lev[c->L - 1];
   if (c->cl_smem[1][V])
     launch_cluster(c->D, true, V, cluster_per(c), c->self_tab, c->self_list, 1, nullptr, true,
-                   cl_max_ctas(), c->cl_smem[1][V], c->stream);
+                   c->cl_ctas, c->cl_smem[1][V], c->stream);
   else if (V)
     launch_coarse_v<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->P.inv_re, c->stream);
   else
@@ -527,7 +528,7 @@ void fill_member(const bfibm_ctx* c, BMember& B, int tail, int C) {
 cudaError_t upload_self(bfibm_ctx* c) {
   const Geos q = geos_of(c);
   const bool fp64 = c->P.precision == 0;
-  const int C = cl_max_ctas();
+  const int C = c->cl_ctas;
   // The one level of an FP64 context without coarse grids is the problem itself:
   // its solve takes the mean off the right-hand side that the residual then
   // reads, so it runs on the global arrays, in one block.
@@ -1753,13 +1754,15 @@ bfibm_status persist_build(Persist& P, bool tune) {
   // the batch's own threshold, and clusters small enough that the members' run
   // side by side in one wave; at least as large as every coarsest level that
   // runs there needs (a member's results do not depend on the cluster's size)
+  int most = 16;
+  for (const bfibm_ctx* c : P.mem) most = std::min(most, c->cl_ctas);
   P.C = 1;
-  while (2 * P.C * nm <= device_sms() && 2 * P.C <= cl_max_ctas()) P.C *= 2;
+  while (2 * P.C * nm <= device_sms() && 2 * P.C <= most) P.C *= 2;
   for (int m = 0; m < nm; ++m) {
     const bfibm_ctx* c = P.mem[m];
     const Geos q = geos_of(c);
     for (int V = 0; V < 2; ++V)
-      while (c->cl_smem[1][V] && P.C < cl_max_ctas() &&
+      while (c->cl_smem[1][V] && P.C < most &&
              !cl_bytes(3, false, V, q.g, c->L, c->L - 1, P.C, c->ncm[V]))
         P.C *= 2;
   }
@@ -2341,6 +2344,7 @@ bfibm_status bfibm_create(const bfibm_params* p, void* stream, bfibm_ctx** out) 
     bfibm_destroy(c);
     return BFIBM_ECUDA;
   }
+  c->cl_ctas = cl_max_ctas();
   if (!p->open_flow) {
     static const int zero = 0;
     if (cudaMalloc((void**)&c->self_tab, sizeof(BMember)) != cudaSuccess ||
