@@ -323,6 +323,7 @@ int pair_fill_kc(const Geo& g, int d, int TY, int waves);
 // Mixed precision (mixed.cu).
 OpShape op_shape(const Geo& g);
 int op_blocks(const OpShape& S);
+dim3 op_grid3(const OpShape& S);   // the same blocks as a batch's items name them
 int op_blocks(int D, const Geo& g, const OpShape& S);
 void launch_v_op(bool fcg, const Geo& g, const OpShape& S, const VOpArgs& a, cudaStream_t s);
 void launch_p_op(const Geo& g, const OpShape& S, const POpArgs& a, cudaStream_t s);
@@ -397,7 +398,7 @@ void launch_b_norm2(const BArgs& A, bool viscous, int grid, cudaStream_t s);
 // level 0: the two passes of the pressure's mean removal around a finalize
 void launch_b_partial_sum_p(const BArgs& A, int grid, cudaStream_t s);
 void launch_b_sub_scalar_p(const BArgs& A, int grid, cudaStream_t s);
-// one item per member with gx = nb, the partials its producer wrote:
+// one item per member with nb, the partials its producer wrote, in x and y:
 // out[slot] = scale * (sum or max of partial[off nb .. off nb + nb)), scale
 // 1, or 1 / cells with `mean`
 void launch_b_finalize(const BArgs& A, int off, int slot, bool is_max, bool mean,

@@ -339,7 +339,12 @@ __global__ void __launch_bounds__(kOpThreads, 2)
 }
 
 // The batched forms stage the member's geometry and pointers in shared
-// memory: read there at each use, they cost no registers.
+// memory: read there at each use, they cost no registers. Their items name a
+// block by (tile along x, tile along y, chunk), each within 16 bits (op_grid3):
+// the single launch's (tile, chunk), in the same order.
+__device__ __forceinline__ Blk op_blk(const Blk& B) {
+  return Blk{B.x + B.gx * B.y, B.z, 0, B.gx * B.gy, B.gz, 1};
+}
 template <bool FCG>
 __global__ void __launch_bounds__(kOpThreads, 2) kb_v_op(BArgs A, int with_partial, int with_r64) {
   __shared__ Geo g;
@@ -364,7 +369,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) kb_v_op(BArgs A, int with_parti
       }
     }
     __syncthreads();
-    v_op_body<FCG>(B, g, S, a);
+    v_op_body<FCG>(op_blk(B), g, S, a);
   });
 }
 
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(kOpThreads, 2) kb_p_op(BArgs A, int with_parti
       a.partial = with_partial ? M.sc.partial : nullptr;
     }
     __syncthreads();
-    p_op_body(B, g, S, a);
+    p_op_body(op_blk(B), g, S, a);
   });
 }
 
@@ -428,6 +433,7 @@ OpShape op_shape(const Geo& g) {
 }
 
 int op_blocks(const OpShape& S) { return S.nx * S.ny * S.nc; }
+dim3 op_grid3(const OpShape& S) { return dim3(S.nx, S.ny, S.nc); }
 
 void launch_v_op(bool fcg, const Geo& g, const OpShape& S, const VOpArgs& a, cudaStream_t s) {
   const dim3 grid(S.nx * S.ny, S.nc);

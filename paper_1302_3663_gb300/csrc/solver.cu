@@ -1396,7 +1396,7 @@ struct Persist {
   cudaEvent_t tfork[kMaxLevels] = {}, tjoin[kMaxLevels] = {};
   // level 0, every member
   PList a3, aop, ared, aflat;        // 3D, FP64 operator passes, cell reductions, flat CG passes
-  PList finop, finred, finflat;       // one item per member, gx = its producer's blocks
+  PList finop, finred, finflat;      // one item per member with its producer's block count
   bool masked = false;               // queuing the body of a device loop
   cudaStream_t stream = nullptr, aux = nullptr;
   cudaEvent_t fork = nullptr, done = nullptr;
@@ -1863,16 +1863,15 @@ bfibm_status persist_build(Persist& P, bool tune) {
   PK(upload(P, v, P.ared));
   ok &= make_items(nm, all, [&](int m) { return dim3(fcg_flat_blocks(lev(m, 0)), 1, 1); }, v);
   PK(upload(P, v, P.aflat));
-  ok &= make_items(nm, all, [&](int m) {
-    const OpShape& S = P.mem[m]->op;
-    return dim3(S.nx * S.ny, S.nc, 1);
-  }, v);
+  ok &= make_items(nm, all, [&](int m) { return op_grid3(P.mem[m]->op); }, v);
   PK(upload(P, v, P.aop));
   P.aop.grid = std::min(P.aop.n, 2 * device_sms());   // two blocks resident per SM
   auto one_per = [&](auto nb_of) {
     v.clear();
-    for (int m = 0; m < nm; ++m)
-      v.push_back(BItem{m, 0, 0, 0, (unsigned short)nb_of(m), 1, 1});
+    for (int m = 0; m < nm; ++m) {   // the count in the halves of x and y
+      const int nb = nb_of(m);
+      v.push_back(BItem{m, (unsigned short)(nb & 65535), (unsigned short)(nb >> 16), 0, 1, 1, 1});
+    }
   };
   one_per([&](int m) { return op_blocks(P.mem[m]->op); });
   PK(upload(P, v, P.finop));

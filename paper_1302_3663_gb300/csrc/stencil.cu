@@ -1692,7 +1692,7 @@ __global__ void __launch_bounds__(256) kb_sub_scalar_p(BArgs A) {
 __global__ void __launch_bounds__(1024) kb_finalize(BArgs A, int off, int slot, int is_max,
                                                     int mean) {
   for_items(A, [&](const BMember& M, const Blk& B) {
-    const int nb = B.gx;
+    const int nb = B.x + 65536 * B.y;   // the member's blocks of the pass before
     const Geo& g = M.g[0];
     const double scale = mean ? 1.0 / (double)((long long)g.n[0] * g.n[1] * g.n[2]) : 1.0;
     finalize_body(B, M.sc.partial + (long long)off * nb, nb, M.sc.out, slot, scale, is_max);
