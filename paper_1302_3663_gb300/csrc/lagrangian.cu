@@ -755,7 +755,8 @@ __global__ void __launch_bounds__(1024) k_spread_scale(NodeSet N, int D, double 
     for (int k = 0; k < 2; ++k) {
       int e = 0;
       frexp(bound[k], &e);   // bound < 2^e
-      scale[k] = (bound[k] > 0.0 && isfinite(bound[k])) ? ldexp(1.0, 61 - e) : 1.0;
+      // (at most 2^1022: the reciprocal of a larger one is no normal number)
+      scale[k] = (bound[k] > 0.0 && isfinite(bound[k])) ? ldexp(1.0, min(61 - e, 1022)) : 1.0;
     }
   }
 }
@@ -768,7 +769,7 @@ __global__ void __launch_bounds__(kBlock) k_spread_finish(int D, Geo g, Ptr3d fr
   int k = blockIdx.z * blockDim.z + threadIdx.z;
   if (i >= g.s[0] || j >= g.s[1] || k >= g.s[2]) return;
   long long c = gidx(g, i, j, k);
-  // the scales are powers of two: their reciprocals by the exponents alone (an
+  // the scales are powers of two from 2^-963 to 2^1022: their reciprocals by the exponents alone (an
   // FP64 division per point costs more than the pass's memory traffic)
   auto inv = [](double s) {
     return __longlong_as_double((2046ll << 52) - __double_as_longlong(s));
