@@ -420,13 +420,14 @@ __device__ __forceinline__ void cl_residual(const ClLv& v, const LevelPtrs<T>& L
 }
 
 // ---------------------------------------------------------------- transfers
-// the coarse level's right-hand side from the fine residual (global): into
-// its slab (slab), into the global array too (out: the coarsest level's, which
-// the pressure's mean and the matrix solve read whole)
+// the coarse level's right-hand side from the fine residual (global): into its
+// slab (slab) and the global array, which holds every level's after a cycle as the
+// launches leave it (the coarsest one's is read whole there by the pressure's mean
+// and the matrix solve)
 template <int D, typename T, typename TC, bool V>
 __device__ __forceinline__ void cl_restrict(const ClLv& v, const Geo& gf, const Geo& gc,
                                             const LevelPtrs<T>& F, const LevelPtrs<T>& Lc,
-                                            bool slab, bool out) {
+                                            bool slab) {
   TC* sm = cl_sm<TC>();
   for (int colour = 0; colour < 2; ++colour)
     cl_colour(v, colour, [&](int h, int par, int r, int lp) {
@@ -441,12 +442,12 @@ __device__ __forceinline__ void cl_restrict(const ClLv& v, const Geo& gf, const 
 #pragma unroll
         for (int d = 0; d < D; ++d) {
           if (slab) sm[v.f[d] + own] = (TC)w[d];
-          if (out) Lc.uf[d][cl_F(v, q)] = w[d];
+          Lc.uf[d][cl_F(v, q)] = w[d];
         }
       } else {
         const T w = restrict_cell_val<D, T, true>(gf, F.pr, q.ci[0], q.ci[1], q.ci[2]);
         if (slab) sm[v.f[0] + own] = (TC)w;
-        if (out) Lc.pf[cl_F(v, q)] = w;
+        Lc.pf[cl_F(v, q)] = w;
       }
     });
 }
@@ -681,10 +682,9 @@ __global__ void __launch_bounds__(kClThreads, 1)
     else __syncthreads();
     const LevelPtrs<T>& Lc = cl_ptrs<D, T>(M, l + 1);
     if (mixed && last)
-      cl_restrict<D, T, double, V>(lvs[l + 1], M.g[l], M.g[l + 1], L, Lc, !dense, !V || dense);
+      cl_restrict<D, T, double, V>(lvs[l + 1], M.g[l], M.g[l + 1], L, Lc, !dense);
     else
-      cl_restrict<D, T, T, V>(lvs[l + 1], M.g[l], M.g[l + 1], L, Lc, !(dense && last),
-                              last && (!V || dense));
+      cl_restrict<D, T, T, V>(lvs[l + 1], M.g[l], M.g[l + 1], L, Lc, !(dense && last));
     if (last && (!V || dense)) cl_sync();   // every CTA's part is read
     else __syncthreads();
   }
