@@ -399,6 +399,20 @@ void coarse_solve(bfibm_ctx* c, bool V) {
     launch_coarse_p<double>(c->D, Lv.g, Lv.d, c->P.coarse_sweeps, c->stream);
 }
 
+// The FP64 solve of a mixed cycle's only level on its FP32 arrays, converted in
+// shared memory: on this level the FP64 arrays hold the problem itself.
+void only_level_solve(bfibm_ctx* c, bool V) {
+  launch_cluster(c->D, false, V, cluster_per(c), c->self_tab, c->self_list, 1, nullptr, true,
+                 c->cl_ctas, c->cl_smem[1][V], c->stream);
+}
+
+// Whether a solve runs FP64 cycles: in FP64 contexts, and in mixed ones of a
+// single level that the cluster kernel cannot hold (an FP32 cycle would be the
+// coarsest FP64 solve alone, with no arrays to run it in).
+bool fp64_cycles(const bfibm_ctx* c, bool V) {
+  return c->P.precision == 0 || (c->L == 1 && !c->cl_smem[1][V]);
+}
+
 void vcycle_p(bfibm_ctx* c, int l) {
   Level& Lv = c->lev[l];
   cudaStream_t s = c->stream;
@@ -769,6 +783,7 @@ void vcycle_p32(bfibm_ctx* c, int l) {
   cudaStream_t s = c->stream;
   if (cluster_cycle(c, l, false)) return;
   if (l == c->L - 1) {
+    if (l == 0) return only_level_solve(c, false);
     long long n = level_elems(Lv.g);
     launch_f32_to_f64(Lv.f.pf, Lv.d.pf, n, s);
     cudaMemsetAsync(Lv.d.p, 0, n * sizeof(double), s);
@@ -790,6 +805,7 @@ void vcycle_v32(bfibm_ctx* c, int l) {
   cudaStream_t s = c->stream;
   if (cluster_cycle(c, l, true)) return;
   if (l == c->L - 1) {
+    if (l == 0) return only_level_solve(c, true);
     long long n = level_elems(Lv.g);
     for (int d = 0; d < c->D; ++d) {
       launch_f32_to_f64(Lv.f.uf[d], Lv.d.uf[d], n, s);
@@ -1118,17 +1134,21 @@ void refresh(bfibm_ctx* c) {
   build_coefficients(c);
 }
 
+bfibm_status solve_v_any(bfibm_ctx* c, int ncycles, int* used) {
+  if (fp64_cycles(c, true)) return solve_v(c, ncycles, used);
+  return c->krylov ? solve_v_fcg(c, ncycles, used) : solve_v_mixed(c, ncycles, used);
+}
+bfibm_status solve_p_any(bfibm_ctx* c, int ncycles, int* used) {
+  return fp64_cycles(c, false) ? solve_p(c, ncycles, used) : solve_p_mixed(c, ncycles, used);
+}
+
 // One time step (Sec. 3.4 order).
 bfibm_status queue_step(bfibm_ctx* c) {
   stage_rhs(c);
-  bool mixed = c->P.precision == 1;
-  bfibm_status st = mixed ? (c->krylov ? solve_v_fcg(c, c->P.vc_visc, &c->cycles_visc)
-                                        : solve_v_mixed(c, c->P.vc_visc, &c->cycles_visc))
-                          : solve_v(c, c->P.vc_visc, &c->cycles_visc);
+  bfibm_status st = solve_v_any(c, c->P.vc_visc, &c->cycles_visc);
   if (st != BFIBM_OK && st != BFIBM_ENOCONV) return st;
   stage_divergence(c);
-  bfibm_status st2 = mixed ? solve_p_mixed(c, c->P.vc_p, &c->cycles_p)
-                           : solve_p(c, c->P.vc_p, &c->cycles_p);
+  bfibm_status st2 = solve_p_any(c, c->P.vc_p, &c->cycles_p);
   if (st2 != BFIBM_OK && st2 != BFIBM_ENOCONV) return st2;
   stage_project(c);
   stage_interp_advance(c);
@@ -1708,6 +1728,7 @@ bool persist_compatible(const bfibm_ctx* a, const bfibm_ctx* c, std::string& why
   if (c->D != 3 || c->P.precision != 1) why = "every member must be a 3D mixed-precision context";
   else if (c->P.open_flow) why = "the open duct is not batched";
   else if (c->P.vc_visc > 0 || c->P.vc_p > 0) why = "members must solve to a tolerance (vc_visc = vc_p = 0)";
+  else if (fp64_cycles(c, true) || fp64_cycles(c, false)) why = "a member has one level, too large for the coarse-level kernel";
   else if ((uintptr_t)c->stream <= 2) why = "members need a stream of their own";
   else if (a && (a->P.nu1 != c->P.nu1 || a->P.nu2 != c->P.nu2 || a->inner != c->inner ||
                  a->krylov != c->krylov))
@@ -2703,8 +2724,7 @@ bfibm_status bfibm_solve_pressure(bfibm_ctx* c, int ncycles, int32_t* cycles) {
   READY(c);
   refresh_inverses(c);
   int used = 0;
-  bfibm_status st = c->P.precision == 1 ? solve_p_mixed(c, ncycles, &used)
-                                        : solve_p(c, ncycles, &used);
+  bfibm_status st = solve_p_any(c, ncycles, &used);
   if (st != BFIBM_OK && st != BFIBM_ENOCONV) return st;
   c->cycles_p = used;
   if (cycles) *cycles = used;
@@ -2733,9 +2753,7 @@ bfibm_status bfibm_solve_viscous(bfibm_ctx* c, int ncycles, int32_t* cycles) {
   READY(c);
   refresh_inverses(c);
   int used = 0;
-  bfibm_status st = c->P.precision == 1 ? (c->krylov ? solve_v_fcg(c, ncycles, &used)
-                                                     : solve_v_mixed(c, ncycles, &used))
-                                        : solve_v(c, ncycles, &used);
+  bfibm_status st = solve_v_any(c, ncycles, &used);
   if (st != BFIBM_OK && st != BFIBM_ENOCONV) return st;
   c->cycles_visc = used;
   if (cycles) *cycles = used;
