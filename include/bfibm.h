@@ -282,7 +282,9 @@ bfibm_status bfibm_body_force(bfibm_ctx* c, double* G);
    memory of a cluster of 16 thread blocks, with a cluster barrier between
    phases and in-place red-black sweeps; default 32768 in mixed precision, 8192
    in FP64; 0 keeps one launch per sweep, residual and transfer; the same
-   results either way, to the bit in mixed precision, to rounding in FP64). */
+   results either way, to the bit in mixed precision, to rounding in FP64. A
+   coarsest level that fits is solved in that kernel with 0 as well; the only
+   level of an FP64 context never is). */
 enum {
   BFIBM_OPT_STATS = 0,
   BFIBM_OPT_GRAPH = 1,
@@ -411,7 +413,8 @@ void bfibm_batch_destroy(bfibm_batch* b);
    while any member still iterates, and a member whose tolerance test is met
    drops out of the mask every launch of the loop reads. The stages around the
    solves run per member on forked branches of the graph. Every member must be
-   3D, mixed precision (precision 1), closed (no open duct), solve to a
+   3D, mixed precision (precision 1), closed (no open duct), of more than one
+   level or a level that the cluster kernel holds, solve to a
    tolerance (vc_visc = vc_p = 0), have a stream of its own, and share nu1,
    nu2, BFIBM_OPT_INNER and BFIBM_OPT_KRYLOV with the others; each member then
    gets the same bits as stepped alone. bfibm_batch_step must then give every
@@ -420,8 +423,8 @@ void bfibm_batch_destroy(bfibm_batch* b);
    BFIBM_BATCH_TUNE (default 1): time the batched sweeps' kernel (ring or pair),
    tile rows, chunk planes, planes per phase and grid on every level of at
    least 2^19 cells in all when a plan is built (0: such levels take the pair
-   sweep with up to 6 tile rows and 16-plane chunks where every member can, the
-   ring sweep otherwise; smaller levels always keep a built-in ring shape).
+   sweep where every member can, with up to 14 tile rows and chunks that fill the
+   chip, the ring sweep otherwise; smaller levels always keep a built-in ring shape).
    BFIBM_BATCH_UNROLL (default 0): k > 0 queues each solve loop as k
    iterations one after another instead of a device-side loop; the masks
    still stop every member where its tolerance is met, so results are the

@@ -24,8 +24,9 @@
 // 1.46 -> 0.74 ms.
 //
 // The point updates, residuals and transfers are those of the per-level
-// launches, rounding for rounding, so a level gives the same bits either way,
-// and with any cluster size.
+// launches, rounding for rounding, so an FP32 level gives the same bits either
+// way; FP64 residuals have the flux form here, and agree to rounding. The cluster's
+// size changes no bit.
 #include <cuda_runtime.h>
 
 #include <algorithm>
