@@ -1076,10 +1076,15 @@ void inverse_diagonals(bfibm_ctx* c, int l) {
 // Before a sweep or a cycle: what coefficients set by hand made stale. (Formed
 // in each set, one field of 97x97x96 points took 107 us instead of 21 and one of a
 // coarsest level with matrices 399 instead of 12, up to ten times over.)
-void refresh_inverses(bfibm_ctx* c) {
+bool refresh_inverses(bfibm_ctx* c) {
+  bool any = false;
   for (int l = 0; l < c->L; ++l)
-    if (c->stale[l]) inverse_diagonals(c, l);
+    if (c->stale[l]) {
+      inverse_diagonals(c, l);
+      any = true;
+    }
   std::memset(c->stale, 0, sizeof(c->stale));
+  return any;   // whether anything was queued
 }
 
 void build_coefficients(bfibm_ctx* c) {
@@ -1162,9 +1167,10 @@ bfibm_status ensure_ready(bfibm_ctx* c) {
     refresh(c);
     c->dirty = false;
     std::memset(c->stale, 0, sizeof(c->stale));   // (not in refresh: a step graph's capture runs it)
+    CK(cudaGetLastError());
+  } else if (refresh_inverses(c)) {
+    CK(cudaGetLastError());
   }
-  refresh_inverses(c);
-  CK(cudaGetLastError());
   return BFIBM_OK;
 }
 
